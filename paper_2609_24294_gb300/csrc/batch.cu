@@ -116,47 +116,52 @@ __device__ __forceinline__ void fill_plane4(const BatchGeom &bg, Tab &tab)
 // its home group -- the SMs are split between groups in proportion to their
 // work, so an SM mostly runs one kind's code and keeps it in its instruction
 // cache -- and then helps the other groups until every queue is empty.
+// fn has one call site for both cases: the kernels inline the codec of every
+// kind into it, and a second copy of that code costs instruction-cache misses.
 template <class Fn>
 __device__ __forceinline__ void for_each_unit(const BatchGeom &bg, int lane, Fn &&fn)
 {
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    if (bg.nunits <= nwarps) {                                   // a small batch: one unit per warp, no claims
+    const bool single = bg.nunits <= nwarps;                     // a small batch: one unit per warp, no claims
+    const uint32_t C = (uint32_t)bg.upc;
+    int gi = 0, tried = 1;                                       // the group in work, groups seen so far
+    uint32_t u = 0;                                              // the unit inside it
+    auto claim = [&]() {
+        uint32_t v = 0;
+        if (lane == 0) v = atomicAdd(bg.ctr + gi, C);
+        return v;
+    };
+    if (single) {
         const int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-        if (c < bg.nunits) {
-            int gi = 0;
-            while (gi + 1 < bg.ngroups && c >= bg.groups[gi + 1].u0) gi++;
-            fn(bg.groups[gi], c, item_of_unit(bg.items, bg.nitems, c));
-        }
-        return;
+        if (c >= bg.nunits) return;
+        while (gi + 1 < bg.ngroups && c >= bg.groups[gi + 1].u0) gi++;
+        u = (uint32_t)(c - bg.groups[gi].u0);
+    } else {
+        uint32_t smid, nsmid;
+        asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+        asm volatile("mov.u32 %0, %%nsmid;" : "=r"(nsmid));
+        const float x = ((float)smid + 0.5f) / (float)nsmid;
+        while (gi + 1 < bg.ngroups && x >= bg.groups[gi].cum1) gi++;
+        u = __shfl_sync(0xffffffffu, claim(), 0);
     }
-    uint32_t smid, nsmid;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-    asm volatile("mov.u32 %0, %%nsmid;" : "=r"(nsmid));
-    const float x = ((float)smid + 0.5f) / (float)nsmid;
-    int home = 0;
-    while (home + 1 < bg.ngroups && x >= bg.groups[home].cum1) home++;
-    for (int t = 0; t < bg.ngroups; t++) {
-        const int gi = (home + t) % bg.ngroups;
-        const GroupDev G = bg.groups[gi];
-        uint32_t *ctr = bg.ctr + gi;
-        const uint32_t C = (uint32_t)bg.upc;
-        uint32_t u = 0;
-        if (lane == 0) u = atomicAdd(ctr, C);
-        u = __shfl_sync(0xffffffffu, u, 0);
-        while ((int64_t)u < G.n) {
-            uint32_t next = 0;                                   // claimed ahead: its latency hides behind fn
-            if (lane == 0) next = atomicAdd(ctr, C);
-            next = __shfl_sync(0xffffffffu, next, 0);
-            // the claim's units in order; a unit's item is the last one starting at or before it
-            const uint32_t ue = (uint32_t)min((int64_t)u + C, G.n);
-            int ii = item_of_unit(bg.items, bg.nitems, G.u0 + u);
-            for (uint32_t v = u; v < ue; v++) {
-                const int64_t c = G.u0 + v;
-                while (ii + 1 < bg.nitems && __ldg(&bg.items[ii + 1].unit0) <= c) ii++;
-                fn(G, c, ii);
-            }
-            u = next;
+    for (;;) {
+        while (!single && (int64_t)u >= bg.groups[gi].n) {       // this queue is empty: the next group's
+            if (tried++ == bg.ngroups) return;
+            gi = gi + 1 == bg.ngroups ? 0 : gi + 1;
+            u = __shfl_sync(0xffffffffu, claim(), 0);
         }
+        const GroupDev G = bg.groups[gi];
+        const uint32_t next = single ? 0u : claim();             // claimed ahead: its latency hides behind fn
+        // the claim's units in order; a unit's item is the last one starting at or before it
+        const uint32_t ue = single ? u + 1 : (uint32_t)min((int64_t)u + C, G.n);
+        int ii = item_of_unit(bg.items, bg.nitems, G.u0 + u);
+        for (; u < ue; u++) {
+            const int64_t c = G.u0 + u;
+            while (ii + 1 < bg.nitems && __ldg(&bg.items[ii + 1].unit0) <= c) ii++;
+            fn(G, c, ii);
+        }
+        if (single) return;
+        u = __shfl_sync(0xffffffffu, next, 0);
     }
 }
 
@@ -311,11 +316,14 @@ batch_encode_kernel(BatchGeom bg, uint8_t *__restrict__ out)
 {
     __shared__ enc3::Shared<16> sh[WARPS];             // rate-16 sized, shared by both rates
     __shared__ Plane4Enc tab;
-    fill_plane4(bg, tab);
+    __shared__ enc3::Expand expand;
+    enc3::load_expand(expand);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const enc3::View v = sh[wid].view();
+    const enc3::View v = sh[wid].view(expand);
     enc3::clear(v, lane, enc3::kWords<16>);
-    __syncwarp();
+    fill_plane4(bg, tab);
+    enc3::wait_expand();
+    __syncthreads();
     for_each_unit(bg, lane, [&](const GroupDev &G, int64_t c, int ii) {
         const ItemDevB it = bg.items[ii];
         const FieldDevB f = bg.fields[it.field];

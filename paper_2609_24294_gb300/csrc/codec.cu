@@ -36,15 +36,18 @@ using namespace blk;
 constexpr int kWarps = 4;
 constexpr int kThreads = 32 * kWarps;
 // Launch shapes of the 3-D kernels, chosen by measurement on GB300: encoder
-// CTAs of 2 warps (rate 8) and 3 warps (rate 16), whose shared memory packs
-// the SMs best; decoder CTAs of 4 warps, except the rate-16 decoder, whose
-// 3-warp CTAs fit six to an SM (two zero rows after its stream tile make the
-// shared memory fit); the rate-8 decoder is compiled for five resident CTAs,
-// which its shared memory allows and capping its registers to match pays for.
+// CTAs of 2 warps, nine to an SM at rate 8 and eight at rate 16, what the
+// shared memory allows (where rows don't start on 16 bytes eight at both, which
+// leaves the four scalar loads per row their registers: 194 us against 209 for
+// a 1000 x 501 x 91 field on 3 x 3 ranks); decoder CTAs of 4 warps, except the
+// rate-16 decoder, whose 3-warp CTAs fit six to an SM (two zero rows after its
+// stream tile make the shared memory fit); the rate-8 decoder is compiled for
+// five resident CTAs, which its shared memory allows and capping its registers
+// to match pays for.
 template <int RATE>
-constexpr int kEnc3Warps = RATE == 16 ? 3 : 2;
-template <int RATE>
-constexpr int kEnc3MinBlocks = RATE == 16 ? 5 : 8;     // what the shared memory allows
+constexpr int kEnc3Warps = 2;
+template <int RATE, bool VEC>
+constexpr int kEnc3MinBlocks = RATE == 8 && VEC ? 9 : 8;
 template <int RATE>
 constexpr int kDec3Warps = RATE == 16 ? 3 : 4;
 template <int RATE>
@@ -101,18 +104,20 @@ struct UnitRange {
 // instantiation reads and writes the rows of x-complete blocks as four scalar
 // accesses each, unrolled, keeping the vector kernel's code as it is.
 template <int RATE, bool VEC>
-__global__ void __launch_bounds__(32 * kEnc3Warps<RATE>, kEnc3MinBlocks<RATE>)
+__global__ void __launch_bounds__(32 * kEnc3Warps<RATE>, kEnc3MinBlocks<RATE, VEC>)
 encode3_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchGeom g, int layout)
 {
     __shared__ enc3::Shared<RATE> sh[kEnc3Warps<RATE>];
+    __shared__ enc3::Expand expand;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const enc3::View v = sh[wid].view();
+    const enc3::View v = sh[wid].view(expand);
+    enc3::load_expand(expand);
     const UnitRange ur(g, kEnc3Warps<RATE>, wid);
-    if (ur.c >= ur.c1) return;
     enc3::clear(v, lane, enc3::kWords<RATE>);
-    __syncwarp();
     MsgWalk walk;
-    walk.start(g.msgs, g.nmsg, ur.c);
+    if (ur.c < ur.c1) walk.start(g.msgs, g.nmsg, ur.c);
+    enc3::wait_expand();
+    __syncthreads();
     for (int64_t c = ur.c; c < ur.c1; c++) {
         walk.advance(c);
         const MsgDev &m = g.msgs[walk.mi];
@@ -133,16 +138,18 @@ encode3_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchG
             if (VEC && x0 + 4 <= nx) {
                 // the common case: sixteen 16-byte row loads (rows past the
                 // end of the box repeat its last row)
+                const float *p = base + (int64_t)z0 * g.ss[2] + (int64_t)y0 * g.ss[1] + x0;
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
-                    const int64_t zo = (int64_t)min(z0 + k, nz - 1) * g.ss[2];
+                    const float *row = p;
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
-                        const float4 f = __ldg(reinterpret_cast<const float4 *>(
-                            base + zo + (int64_t)min(y0 + j, ny - 1) * g.ss[1] + x0));
+                        const float4 f = __ldg(reinterpret_cast<const float4 *>(row));
                         x[16 * k + 4 * j] = f.x; x[16 * k + 4 * j + 1] = f.y;
                         x[16 * k + 4 * j + 2] = f.z; x[16 * k + 4 * j + 3] = f.w;
+                        if (y0 + j + 1 < ny) row += g.ss[1];
                     }
+                    if (z0 + k + 1 < nz) p += g.ss[2];
                 }
             } else if (!VEC && x0 + 4 <= nx) {
                 // rows not on 16 bytes: four scalar loads per row

@@ -11,11 +11,9 @@
 //          the lane's stream (2 RATE words, then four slack words that catch
 //          the bits of a plane running past the budget).  Zero on entry;
 //          store_stream() copies the stream out and zeroes the tile again.
-//   planes [32][32] 64-bit: bit plane k of lane l at k * 32 + l; pass 1
-//          reuses the slots of planes already read for its list of planes
-//          with newly significant coefficients (entry f at slot 31 - f).
-//   spos   [32][32] uint16: for list entry f, the stream position of the
-//          plane's first group bit plus one.
+//   planes [32][32] 64-bit: bit plane k of lane l at k * 32 + l; phase A
+//          reuses the slots of planes already read for its list of unfinished
+//          group-tested parts (entry f at slot 31 - f).
 //
 // The stream of a block is its header (a 1 bit and e_max + 127 in 8 bits),
 // then the bit planes from the top.  Plane k, with n coefficients already
@@ -27,14 +25,31 @@
 // without new ones and n + 1 + (h - n + 1) + c bits with them (two fewer when
 // h = 63); the stream is cut at exactly 64 RATE bits.
 //
-// Phase A walks the planes while n < 64: it writes the verbatim bits and the
-// first group bit, leaves the group-tested part as zeros and lists the plane
-// if it has new ones.  Phase B: once n = 64 every later plane is its 64 bits
-// verbatim, so the rest of the stream is the remaining planes back to back,
-// one funnel shift per 32-bit word.  Pass 2 walks the list one new
-// coefficient per step: the t-th one of a listed plane, at coefficient p,
-// has its value bit at (listed position) + p + t, its group bit right after;
-// positions only grow, so the first one past the budget ends a lane's pass.
+// Phase A walks the planes while n < 64: it writes the verbatim bits and, for
+// a plane with new ones, the group bit and the code of the first eight
+// coefficients from n on, which a table gives as up to 16 bits (Expand).  Half
+// the group-tested parts end there; the others wait in the list, the lane's
+// remaining coefficients and their position in one 64-bit word.  Phase B: once
+// n = 64 every later plane is its 64 bits verbatim, so the rest of the stream
+// is the remaining planes back to back, one funnel shift per 32-bit word.  The
+// list is walked last, eight coefficients per step: each lane steps through its
+// own entries, so the warp takes the most steps of one lane (about 6) where
+// finishing each plane on the spot would take the sum over the planes of the
+// most steps of any lane (about 22).
+//
+// What bounds it: instruction issue, half of it on the ALU pipe (ncu: issue
+// slots 58 % busy, ALU pipe 60 %, 16 to 18 warps per SM), and the latency of
+// the gather.  Per 32 blocks at rate 8 about 3500 warp instructions: gather and
+// store 270, block maximum and quantisation 210, lifting 610, planes 440, the
+// coder the rest.  With one new coefficient per step instead of eight
+// through the table, each plane's part finished in a second pass, and the block
+// maximum by integer compares it was 4200; compressing a 1280 x 640 x 137
+// field over 8 x 8 ranks took 336 us at rate 8 and 420 us at rate 16 then, 286
+// and 357 us now.
+//
+// How the lanes are kept together: phase A is one straight run of instructions
+// per plane (a lane without new ones codes zeros), each lane leaving it when
+// its own planes are done; the list is walked while any lane has entries.
 #pragma once
 #include <cstdint>
 
@@ -49,12 +64,53 @@ using namespace blk;
 template <int RATE>
 constexpr int kWords = 2 * RATE + 4;
 
+// The group-tested code of eight coefficients (bit i: coefficient i is newly
+// significant), LSB first: a value bit each, a group bit 1 after each one.
+// Entries 256 + c: the last one's group bit 0 (the plane's part ends there);
+// 512 + c: the last one is coefficient 63, whose value and group bit are not
+// sent.  A CTA keeps a copy in shared memory.
+struct __align__(16) Expand {
+    uint16_t e[3 * 256];
+};
+constexpr Expand make_expand()
+{
+    Expand t{};
+    for (int c = 0; c < 256; c++) {
+        uint32_t out = 0, top = 0;
+        int len = 0;
+        for (int i = 0; i < 8; i++) {
+            if ((c >> i) & 1) {
+                top = 1u << len;
+                out |= 3u << len;
+                len++;
+            }
+            len++;
+        }
+        t.e[c] = (uint16_t)out;
+        t.e[256 + c] = (uint16_t)(out & ~(2u * top));
+        t.e[512 + c] = (uint16_t)(out & ~(3u * top));
+    }
+    return t;
+}
+static __device__ const Expand g_expand = make_expand();
+
+// Copies the table asynchronously (every thread of the CTA takes part); ready
+// after wait_expand() by every thread and a __syncthreads().
+__device__ __forceinline__ void load_expand(Expand &tab)
+{
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(tab.e);
+    for (int i = threadIdx.x; i < (int)sizeof(Expand) / 16; i += blockDim.x)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d + 16u * (uint32_t)i), "l"(g_expand.e + 8 * i)
+                     : "memory");
+}
+__device__ __forceinline__ void wait_expand() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // One warp's shared memory: tile (kWords<RATE> * 32 words, or more), planes
 // (32 * 32), spos (32 * 32).
 struct View {
     uint32_t *tile;
     uint64_t *planes;
-    uint16_t *spos;
+    const uint16_t *expand;
 };
 
 // Storage of one warp at `rate`.
@@ -62,8 +118,7 @@ template <int RATE>
 struct Shared {
     uint32_t tile[kWords<RATE> * 32];
     uint64_t planes[32 * 32];
-    uint16_t spos[32 * 32];
-    __device__ __forceinline__ View view() { return View{tile, planes, spos}; }
+    __device__ __forceinline__ View view(const Expand &tab) { return View{tile, planes, tab.e}; }
 };
 
 __device__ __forceinline__ uint32_t shl(uint32_t a, uint32_t s)
@@ -80,37 +135,76 @@ __device__ __forceinline__ uint32_t shr(uint32_t a, uint32_t s)
 }
 // high word of (hi:lo) << s, 0 <= s < 32
 __device__ __forceinline__ uint32_t funnel(uint32_t lo, uint32_t hi, uint32_t s) { return __funnelshift_l(lo, hi, s); }
-__device__ __forceinline__ void red_or(uint32_t *p, uint32_t v) { atomicOr(p, v); }
+// max(|a|, |b|, |c|), NaN if one of them is
+__device__ __forceinline__ float max3_abs(float a, float b, float c)
+{
+    float r;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ uint32_t smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// ORs v into the shared word at address a + OFF (32-bit shared addresses: no
+// 64-bit pointer arithmetic in the coder's loops)
+template <int OFF>
+__device__ __forceinline__ void red_or(uint32_t a, uint32_t v)
+{
+    asm volatile("red.shared.or.b32 [%0+%2], %1;" ::"r"(a), "r"(v), "n"(OFF) : "memory");
+}
+
+// One step of a group-tested part: the code of the next eight coefficients
+// (the low bits of zh:zl, shifted out) ORed into the lane's stream after bit A,
+// with e0 at bit A itself (the plane's group bit ahead of its first eight);
+// A moves on by the code's length.  `last`: table offset in bytes for the
+// eight that end the part.
+__device__ __forceinline__ void chunk(uint32_t &zl, uint32_t &zh, int &A, uint32_t e0, uint32_t tb, uint32_t xb,
+                                      uint32_t last)
+{
+    const uint32_t c = zl & 255u;
+    zl = __funnelshift_r(zl, zh, 8);
+    zh >>= 8;
+    uint16_t code;
+    asm("ld.shared.u16 %0, [%1];" : "=h"(code) : "r"(xb + ((zl | zh) ? 0u : last) + 2u * c));
+    const uint32_t e = 2u * code + e0, s = (uint32_t)A & 31u, w = tb + 4u * (uint32_t)(A & ~31);
+    red_or<0>(w, e << s);
+    red_or<128>(w, shr(e, 32u - s));
+    A += 8 + popc32(c);
+}
 
 template <int RATE>
 __device__ __forceinline__ void encode(const float (&x)[64], bool valid, const View &sh, int lane)
 {
     constexpr int kSeq[64] = ZFPX_SEQ3;
     constexpr int END = 64 * RATE;
-    constexpr unsigned FULL = 0xffffffffu;
     uint32_t *tile = sh.tile + lane;                   // word w at tile[32 w]
     uint64_t *planes = sh.planes + lane;               // plane k at planes[32 k]
-    uint16_t *spos = sh.spos + lane;
-    uint32_t amax = 0;
+    // largest magnitude: the bits of max |x|, NaN where a NaN takes part
+    // (max.NaN propagates it), so its exponent field is 255 as for infinities
+    float am = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 64; i++) {
-        const uint32_t a = f2u(x[i]) & 0x7fffffffu;
-        amax = a > amax ? a : amax;
-    }
+    for (int i = 0; i < 64; i += 2) am = max3_abs(am, x[i], x[i + 1]);
+    const uint32_t amax = f2u(am) & 0x7fffffffu;
     // E = e_max + 126; a block whose maximum is zero, below 2^-127 or not
     // finite is a single 0 bit (the tile is already zero)
     const int E = (int)(amax >> 23);
-    bool act = valid && amax >= 0x00400000u && E != 255;
+    const bool act = valid && amax >= 0x00400000u && E != 255;
     const QuantScale qs(act ? E : 127);
     int32_t q[64];
+    if (act && E < 29) {                               // tiny blocks (rare): the scale in two factors
 #pragma unroll
-    for (int i = 0; i < 64; i++) q[i] = qs(x[i]);
+        for (int i = 0; i < 64; i++) q[i] = qs(x[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 64; i++) q[i] = f2i_rz(x[i] * qs.s2);
+    }
     xform3_fwd(q);
+    // negabinary is (q + M) ^ M with M = 0xAA..A: the add here, the xor as the
+    // complement of the odd planes once they are transposed (it folds into the
+    // last stage's logic operations)
     uint32_t lo[32], hi[32];
 #pragma unroll
     for (int t = 0; t < 32; t++) {
-        lo[t] = to_negabinary(q[kSeq[t]]);
-        hi[t] = to_negabinary(q[kSeq[32 + t]]);
+        lo[t] = (uint32_t)q[kSeq[t]] + 0xAAAAAAAAu;
+        hi[t] = (uint32_t)q[kSeq[32 + t]] + 0xAAAAAAAAu;
     }
     // planes kLow .. 31 finished now, 0 .. kLow - 1 half-transposed until a
     // lane needs them (the budget rarely reaches below plane 16 at rate 8,
@@ -125,7 +219,7 @@ __device__ __forceinline__ void encode(const float (&x)[64], bool valid, const V
         }
         transpose32_part1<kLow>(lo);
 #pragma unroll
-        for (int k = 0; k < 32; k++) p32[64 * k + half] = lo[k];
+        for (int k = 0; k < 32; k++) p32[64 * k + half] = k >= kLow && (k & 1) ? ~lo[k] : lo[k];
     }
     bool low_done = false;
     auto finish_low = [&]() {
@@ -138,109 +232,94 @@ __device__ __forceinline__ void encode(const float (&x)[64], bool valid, const V
         transpose32_part2<kLow>(a);
         transpose32_part2<kLow>(b);
 #pragma unroll
-        for (int i = 0; i < kLow; i++) planes[32 * i] = ((uint64_t)b[i] << 32) | a[i];
+        for (int i = 0; i < kLow; i++) {
+            const uint32_t c = i & 1 ? 0xffffffffu : 0u;
+            planes[32 * i] = ((uint64_t)(b[i] ^ c) << 32) | (a[i] ^ c);
+        }
         low_done = true;
     };
-    tile[0] = act ? 1u | ((uint32_t)(E + 1) << 1) : 0u;
+    if (act) tile[0] = 1u | ((uint32_t)(E + 1) << 1);
 
     // ---- phase A: planes while n < 64
-    int n = 0, pos = 9, nf = 0, kB = -1;
-    uint32_t lml = 0, lmh = 0;                         // low n bits
-    uint32_t gml = 1, gmh = 0;                         // bit n
-    bool pa = act;                                      // in phase A
+    int n1 = 1, pos = 9, kB = -1;                      // n + 1
+    uint64_t lm = 0;                                   // low n bits
+    const uint32_t tb = smem(tile), xb = smem(sh.expand), list0 = smem(planes + 31 * 32);
+    uint32_t list = list0;                             // where the next entry goes
 #pragma unroll 1
-    for (int k = 31; k >= 0; k--) {
-        if (!__any_sync(FULL, pa)) break;
+    for (int k = act ? 31 : -1; k >= 0; k--) {
         if (k == kLow - 1) finish_low();
         const uint64_t X = planes[32 * k];
-        const uint32_t xl = (uint32_t)X, xh = (uint32_t)(X >> 32);
-        const uint32_t yl = xl & ~lml, yh = xh & ~lmh;
-        const bool has = pa && (yl | yh) != 0;
-        const uint32_t hm = has ? 0xffffffffu : 0u, am = pa ? 0xffffffffu : 0u;
-        const uint32_t vl = ((xl & lml) | (gml & hm)) & am, vh = ((xh & lmh) | (gmh & hm)) & am;
-        const uint32_t w = (uint32_t)(pa ? pos : 0) >> 5, s = (uint32_t)pos & 31u;
-        red_or(tile + 32 * w, vl << s);
-        red_or(tile + 32 * (w + 1), funnel(vl, vh, s));
-        red_or(tile + 32 * (w + 2), funnel(vh, 0u, s));
-        const int h = yh ? 32 + highest_set32(yh) : highest_set32(yl | 1u);
-        const int c = popc32(yl) + popc32(yh);
-        if (has) {
-            planes[32 * (31 - nf)] = ((uint64_t)yh << 32) | yl;
-            spos[32 * nf] = (uint16_t)(pos + 1);
-            nf++;
-            // n = h + 1: low mask (2 << h) - 1 and bit n, as 32-bit halves
-            lml = shl(2u, (uint32_t)h) - 1u;                             // all ones from h = 31
-            lmh = h >= 32 ? shl(2u, (uint32_t)(h - 32)) - 1u : 0u;
-            gml = h < 31 ? 2u << h : 0u;
-            gmh = h >= 31 && h < 63 ? 1u << (h - 31) : 0u;
-            n = h + 1;
+        const uint64_t Y = X & ~lm, V = X & lm;
+        const uint32_t vl = (uint32_t)V, vh = (uint32_t)(V >> 32), s = (uint32_t)pos & 31u;
+        const uint32_t w = tb + 4u * (uint32_t)(pos & ~31);
+        red_or<0>(w, vl << s);
+        red_or<128>(w, funnel(vl, vh, s));
+        red_or<256>(w, funnel(vh, 0u, s));
+        // the group bit and the first eight coefficients of the group-tested
+        // part now (the next eight too where more than 53 remain), the rest
+        // listed; without new ones all of it is zeros
+        const bool any = Y != 0;
+        const uint64_t Z = Y >> (n1 - 1);
+        uint32_t zl = (uint32_t)Z, zh = (uint32_t)(Z >> 32);
+        int A = pos + n1 - 1;                          // the group bit
+        if (any) {
+            const int lead = 63 - highest_set64(Y);
+            lm = ~0ull >> lead;
+            n1 = 65 - lead;
         }
-        pos += pa ? (has ? h + c + (h < 63 ? 2 : 0) : n + 1) : 0;
-        const bool full = pa && n == 64 && pos < END;
-        kB = full ? k - 1 : kB;
-        pa = pa && n < 64 && pos < END;
+        pos += popc64(Y) + n1;
+        const uint32_t last = n1 == 65 ? 1024u : 512u;
+        chunk(zl, zh, A, any ? 1u : 0u, tb, xb, last);
+        if (zh >> 21) chunk(zl, zh, A, 0u, tb, xb, last);
+        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(list), "r"(zl),
+                     "r"(zh | (n1 == 65 ? 1u << 21 : 0u) | ((uint32_t)A << 22)) : "memory");
+        if ((zl | zh) && A < END) list -= 256;
+        kB = k - 1;
+        if (n1 == 65 || pos >= END) break;
     }
+    __syncwarp();                                      // the lanes go on together
+    if (n1 == 65) pos -= 2;                            // coefficient 63's one is implied: no value or group bit
 
-    // ---- phase B: planes kB, kB - 1, ... verbatim from bit pB = pos
-    bool pb = act && n == 64 && pos < END;
-    {
+    // ---- phase B
+    if (n1 == 65 && pos < END) {
         const uint32_t s = (uint32_t)pos & 31u;
         const int w0 = pos >> 5;
-        // the lowest plane a lane reads here: planes kB - m for the m with
-        // w0 + 2 m < 2 RATE
-        const int need = kB - ((2 * RATE - w0 + 1) / 2 - 1);
-        if (!low_done && __any_sync(FULL, pb && need < kLow)) finish_low();
+        if (!low_done && kB - ((2 * RATE - w0 + 1) / 2 - 1) < kLow) finish_low();
         uint32_t prev = 0;
 #pragma unroll 1
-        for (int m = 0;; m++) {
-            const int wa = w0 + 2 * m;                 // words wa (from the previous plane's high half) and wa + 1
-            const bool live = pb && wa < 2 * RATE;
-            if (!__any_sync(FULL, live)) break;
-            const int kp = kB - m;
-            const uint64_t X = live && kp >= 0 ? planes[32 * kp] : 0ull;
+        for (int wa = w0; wa < 2 * RATE; wa += 2) {
+            const uint64_t X = kB >= 0 ? planes[32 * kB] : 0ull;
             const uint32_t xl = (uint32_t)X, xh = (uint32_t)(X >> 32);
-            if (live) {
-                if (m == 0) red_or(tile + 32 * wa, xl << s);
-                else tile[32 * wa] = funnel(prev, xl, s);
-                tile[32 * (wa + 1)] = funnel(xl, xh, s);
-            }
+            if (wa == w0) red_or<0>(tb + 128u * wa, xl << s);
+            else tile[32 * wa] = funnel(prev, xl, s);
+            tile[32 * (wa + 1)] = funnel(xl, xh, s);
             prev = xh;
+            kB--;
         }
     }
+    __syncwarp();
 
-    // ---- pass 2: the listed planes' new coefficients
-    int f = 0, ap = 0, t = 0;
-    uint32_t rl = 0, rh = 0;
+    // ---- the list: eight coefficients per step, each lane through its own
+    // entries; a lane without any ORs zeros
+    {
+        uint32_t next = list0, zl = 0, zh = 0, last = 512u;
+        int A = 0;
 #pragma unroll 1
-    for (;;) {
-        const bool need = (rl | rh) == 0 && f < nf;
-        if (!__any_sync(FULL, need || (rl | rh) != 0)) break;
-        if (need) {
-            const uint64_t Y = planes[32 * (31 - f)];
-            rl = (uint32_t)Y;
-            rh = (uint32_t)(Y >> 32);
-            ap = spos[32 * f];
-            t = 0;
-            f++;
+        while (__any_sync(0xffffffffu, (zl | zh) != 0 || next != list)) {
+            if ((zl | zh) == 0 && next != list) {
+                asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(zl), "=r"(zh) : "r"(next));
+                next -= 256;
+                A = (int)(zh >> 22);
+                last = zh & (1u << 21) ? 1024u : 512u;
+                zh &= (1u << 21) - 1u;
+            }
+            if (A >= END) {                            // positions only grow: nothing later is sent
+                zl = zh = 0;
+                next = list;
+                A = 0;
+            }
+            chunk(zl, zh, A, 0u, tb, xb, last);
         }
-        const bool live = (rl | rh) != 0;
-        const bool inlo = rl != 0;
-        const int p = inlo ? lowest_set32(rl) : 32 + lowest_set32(rh | 0x80000000u);
-        if (inlo) rl &= rl - 1u;
-        else rh &= rh - 1u;
-        const int A = ap + p + t;
-        t++;
-        const bool ok = live && A < END;
-        if (live && A >= END) {                        // this one and every later one past the budget
-            rl = rh = 0;
-            f = nf;
-        }
-        // value bit (coefficient 63's is implied) and the group bit after it,
-        // which may land in the next word or a slack word
-        const uint32_t b = ok ? (uint32_t)(p != 63) | ((rl | rh) != 0 ? 2u : 0u) : 0u;
-        const uint32_t w = (uint32_t)(ok ? A : 0) >> 5, s = (uint32_t)A & 31u;
-        red_or(tile + 32 * w, b << s);
-        red_or(tile + 32 * (w + 1), shr(b, 32u - s));
     }
 }
 
