@@ -268,7 +268,19 @@ decode3_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchG
 
 // ================================================================= 1-D kernels
 // Blocks of 4 values along x; a block is 4r bits (32 or 64), kept in one
-// register and moved with one coalesced 4- or 8-byte access per lane.
+// register and moved with one coalesced 4- or 8-byte access per lane.  A lane
+// takes a block of each of kUnits1 consecutive units of its warp's range at a
+// time, all loads ahead of the coding.
+constexpr int kUnits1 = 2;
+
+// x origin and row offset (elements, view strides s) of block b of message m
+__device__ __forceinline__ int64_t block1_row(const MsgDev &m, const int64_t *s, uint32_t b, int &x0)
+{
+    const uint32_t t = divu(b, m.bxm, m.bxl), z = divu(t, m.bym, m.byl);
+    x0 = 4 * (int)(b - t * (uint32_t)m.bx);
+    return (int64_t)z * s[2] + (int64_t)(t - z * (uint32_t)m.by) * s[1];
+}
+
 template <int RATE>
 __global__ void __launch_bounds__(kThreads)
 encode1_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchGeom g, int layout, int vec)
@@ -284,30 +296,39 @@ encode1_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchG
     if (c >= c1) return;
     MsgWalk walk;
     walk.start(g.msgs, g.nmsg, c);
-    for (; c < c1; c++) {
+    while (c < c1) {
         walk.advance(c);
         const MsgDev &m = g.msgs[walk.mi];
-        const int64_t b0 = (c - m.unit0) * 32;
-        const int nact = (int)min((int64_t)32, m.nblocks - b0);
-        if (lane >= nact) continue;
-        const int nx = m.nx, bxn = m.bx, byn = m.by;
-        const int64_t boff = layout ? m.off[1] : m.off[0];
-        const int b = (int)b0 + lane;
-        const int t = (int)divu((uint32_t)b, m.bxm, m.bxl), bxi = b - t * bxn;
-        const int z = (int)divu((uint32_t)t, m.bym, m.byl), y = t - z * byn;
-        const int x0 = 4 * bxi;
-        const float *row = src + m.src_off + (int64_t)z * g.ss[2] + (int64_t)y * g.ss[1];
-        float r[4];
-        if (vec && x0 + 4 <= nx) {
-            const float4 f = __ldg(reinterpret_cast<const float4 *>(row + x0));
-            r[0] = f.x; r[1] = f.y; r[2] = f.z; r[3] = f.w;
-        } else {
+        const int take = (int)min((int64_t)kUnits1, min(c1, walk.next0) - c);
+        const uint32_t b0 = (uint32_t)(c - m.unit0) * 32u + lane;
+        const uint32_t end = (uint32_t)min(m.nblocks, (c - m.unit0 + take) * 32);
+        const int nx = m.nx;
+        const float *base = src + m.src_off;
+        float r[kUnits1][4];
 #pragma unroll
-            for (int i = 0; i < 4; i++) r[i] = __ldg(row + (int64_t)min(x0 + i, nx - 1) * g.ss[0]);
+        for (int k = 0; k < kUnits1; k++) {
+            const uint32_t b = b0 + 32u * k;
+            int x0;
+            const float *row = base + block1_row(m, g.ss, b < end ? b : 0u, x0);   // past the end: some block's values
+            if (vec && x0 + 4 <= nx) {
+                const float4 f = __ldg(reinterpret_cast<const float4 *>(row + x0));
+                r[k][0] = f.x; r[k][1] = f.y; r[k][2] = f.z; r[k][3] = f.w;
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; i++) r[k][i] = __ldg(row + (int64_t)min(x0 + i, nx - 1) * g.ss[0]);
+            }
         }
-        const uint64_t w = encode_block1<RATE>(r, tab);
-        if (RATE == 16) reinterpret_cast<uint64_t *>(out + boff)[b] = w;
-        else reinterpret_cast<uint32_t *>(out + boff)[b] = (uint32_t)w;
+        uint64_t w[kUnits1];
+        encode_blocks1<RATE, kUnits1>(r, tab, w);
+        uint8_t *dst = out + (layout ? m.off[1] : m.off[0]);
+#pragma unroll
+        for (int k = 0; k < kUnits1; k++) {
+            const uint32_t b = b0 + 32u * k;
+            if (b >= end) continue;
+            if (RATE == 16) reinterpret_cast<uint64_t *>(dst)[b] = w[k];
+            else reinterpret_cast<uint32_t *>(dst)[b] = (uint32_t)w[k];
+        }
+        c += take;
     }
 }
 
@@ -326,31 +347,41 @@ decode1_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchG
     if (c >= c1) return;
     MsgWalk walk;
     walk.start(g.msgs, g.nmsg, c);
-    for (; c < c1; c++) {
+    while (c < c1) {
         walk.advance(c);
         const MsgDev &m = g.msgs[walk.mi];
-        const int64_t b0 = (c - m.unit0) * 32;
-        const int nact = (int)min((int64_t)32, m.nblocks - b0);
-        if (lane >= nact) continue;
-        const int nx = m.nx, bxn = m.bx, byn = m.by;
-        const int64_t boff = layout ? m.off[1] : m.off[0];
-        const int b = (int)b0 + lane;
-        uint64_t w;
-        if (RATE == 16) w = __ldg(reinterpret_cast<const uint64_t *>(in + boff) + b);
-        else w = __ldg(reinterpret_cast<const uint32_t *>(in + boff) + b);
-        float v[4];
-        decode_block1<RATE>(w, v, tab);
-        const int t = (int)divu((uint32_t)b, m.bxm, m.bxl), bxi = b - t * bxn;
-        const int z = (int)divu((uint32_t)t, m.bym, m.byl), y = t - z * byn;
-        const int x0 = 4 * bxi;
-        float *row = dstf + m.dst_off + (int64_t)z * g.ds[2] + (int64_t)y * g.ds[1];
-        if (vec && x0 + 4 <= nx) {
-            *reinterpret_cast<float4 *>(row + x0) = make_float4(v[0], v[1], v[2], v[3]);
-        } else {
+        const int take = (int)min((int64_t)kUnits1, min(c1, walk.next0) - c);
+        const uint32_t b0 = (uint32_t)(c - m.unit0) * 32u + lane;
+        const uint32_t end = (uint32_t)min(m.nblocks, (c - m.unit0 + take) * 32);
+        const int nx = m.nx;
+        const uint8_t *src = in + (layout ? m.off[1] : m.off[0]);
+        float *base = dstf + m.dst_off;
+        uint64_t w[kUnits1];
 #pragma unroll
-            for (int i = 0; i < 4; i++)
-                if (x0 + i < nx) row[(int64_t)(x0 + i) * g.ds[0]] = v[i];
+        for (int k = 0; k < kUnits1; k++) {
+            const uint32_t b = b0 + 32u * k;
+            w[k] = 0;
+            if (b >= end) continue;
+            if (RATE == 16) w[k] = __ldg(reinterpret_cast<const uint64_t *>(src) + b);
+            else w[k] = __ldg(reinterpret_cast<const uint32_t *>(src) + b);
         }
+        float v[kUnits1][4];
+        decode_blocks1<RATE, kUnits1>(w, tab, v);
+#pragma unroll
+        for (int k = 0; k < kUnits1; k++) {
+            const uint32_t b = b0 + 32u * k;
+            if (b >= end) continue;
+            int x0;
+            float *row = base + block1_row(m, g.ds, b, x0);
+            if (vec && x0 + 4 <= nx) {
+                *reinterpret_cast<float4 *>(row + x0) = make_float4(v[k][0], v[k][1], v[k][2], v[k][3]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; i++)
+                    if (x0 + i < nx) row[(int64_t)(x0 + i) * g.ds[0]] = v[k][i];
+            }
+        }
+        c += take;
     }
 }
 

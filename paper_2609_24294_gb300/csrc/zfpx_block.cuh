@@ -1008,20 +1008,27 @@ struct WordReader {
     ZFPX_HD void skip(int k) { off += k; }
 };
 
-// With four coefficients a plane's code depends only on n (significant
-// coefficients, 0..4) and its four bits X (encoding) or the next seven stream
-// bits (decoding; no plane of four takes more).  The coders look planes up in
-// a table built from code_plane / decode_plane at launch: encoder entry
-// (n, X) = code bits 0..6, length bits 7..9, new n bits 10..12; decoder entry
-// (n, w7) = X bits 0..3, length bits 4..6, new n bits 7..9.
-// The encoder's output is the first 4 RATE bits of the unbounded code
-// (code_plane only ever cuts a plane short), so its loop just stops at the
-// budget.  For a plane the budget cuts after r bits the decoder looks up the
-// window with the bits from r on cleared: zeros past the budget add no one
-// except, when n < 4, the implied one of coefficient 3, which needs the whole
-// plane and so is dropped; what is left is what reading stops at the budget
-// gives.  Both run K blocks of a lane in lockstep so that their table
-// lookups, which each plane's successor waits for, overlap.
+// With four coefficients the code has little structure left, and both coders
+// take it by runs instead of plane by plane.  While n coefficients are
+// significant and no new one appears, a plane is n verbatim bits and a 0, so a
+// run of such planes is a bit interleave: of nothing (n = 0), of one
+// coefficient with zeros (n = 1) or of two with zeros (n = 2).  From n = 3 on a
+// plane is just its four bits: with n = 3 the group bit says whether
+// coefficient 3, whose one is then implied, is new.  So a block is at most
+// three runs, each ended by one plane with new ones, and a tail of 4-bit
+// planes; the length of a run is a count of leading zeros.  A plane with new
+// ones is coded from a table built from code_plane / decode_plane: encoder
+// entry (n, X) = code bits 0..6, length bits 7..9, new n bits 10..12; decoder
+// entry (n, the next seven bits) = X bits 0..3, length bits 4..6, new n bits
+// 7..9.
+// The encoder's output is the first 4 RATE bits of the unbounded code, which
+// is the width of the word it builds: what runs past the budget shifts out.
+// The decoder reads zeros past the budget, which add no one except, in a plane
+// with new ones that the budget cuts, the implied one of coefficient 3, which
+// needs the whole plane and so is dropped.
+// The planes are taken bit-reversed (plane 31 in bit 0), in stream order.
+// This bounds the 1-D kernels by instruction issue still, at about half the
+// instructions of one table lookup per plane.
 struct Plane4Enc {
     uint16_t e[5 * 16];
 };
@@ -1056,13 +1063,170 @@ ZFPX_HD void plane4_fill(Plane4Dec &tab, int t, int nthreads)
     for (int i = t; i < 5 * 128; i += nthreads) tab.d[i] = plane4_dec_entry(i >> 7, (uint32_t)i & 127u);
 }
 
+ZFPX_HD uint32_t reverse32(uint32_t x)
+{
+#ifdef __CUDA_ARCH__
+    return __brev(x);
+#else
+    x = (x >> 16) | (x << 16);
+    x = ((x >> 8) & 0x00ff00ffu) | ((x & 0x00ff00ffu) << 8);
+    x = ((x >> 4) & 0x0f0f0f0fu) | ((x & 0x0f0f0f0fu) << 4);
+    x = ((x >> 2) & 0x33333333u) | ((x & 0x33333333u) << 2);
+    return ((x >> 1) & 0x55555555u) | ((x & 0x55555555u) << 1);
+#endif
+}
+ZFPX_HD int leading_zeros32(uint32_t x)                          // 32 for 0
+{
+#ifdef __CUDA_ARCH__
+    return __clz((int)x);
+#else
+    return x ? __builtin_clz(x) : 32;
+#endif
+}
+// Shifts by any s >= 0, giving 0 from the width on.
+ZFPX_HD uint32_t shl_any(uint32_t x, int s)
+{
+#ifdef __CUDA_ARCH__
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(s));
+    return r;
+#else
+    return s < 32 ? x << s : 0u;
+#endif
+}
+ZFPX_HD uint32_t shr_any(uint32_t x, int s)
+{
+#ifdef __CUDA_ARCH__
+    uint32_t r;
+    asm("shr.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(s));
+    return r;
+#else
+    return s < 32 ? x >> s : 0u;
+#endif
+}
+ZFPX_HD uint64_t shl_any(uint64_t x, int s)
+{
+#ifdef __CUDA_ARCH__
+    uint64_t r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(s));
+    return r;
+#else
+    return s < 64 ? x << s : 0ull;
+#endif
+}
+ZFPX_HD uint64_t shr_any(uint64_t x, int s)
+{
+#ifdef __CUDA_ARCH__
+    uint64_t r;
+    asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(s));
+    return r;
+#else
+    return s < 64 ? x >> s : 0ull;
+#endif
+}
+
+// Bit i of x to bit 2 i, 3 i or 4 i (16, 10 and 8 bits fit a 32-bit word), and
+// back from the bits there.
+ZFPX_HD uint32_t spread2(uint32_t x)
+{
+    x &= 0xffffu;
+    x = (x | (x << 8)) & 0x00ff00ffu;
+    x = (x | (x << 4)) & 0x0f0f0f0fu;
+    x = (x | (x << 2)) & 0x33333333u;
+    return (x | (x << 1)) & 0x55555555u;
+}
+ZFPX_HD uint32_t spread3(uint32_t x)
+{
+    x &= 0x3ffu;
+    x = (x | (x << 16)) & 0x030000ffu;
+    x = (x | (x << 8)) & 0x0300f00fu;
+    x = (x | (x << 4)) & 0x030c30c3u;
+    return (x | (x << 2)) & 0x09249249u;
+}
+ZFPX_HD uint32_t spread4(uint32_t x)
+{
+    x &= 0xffu;
+    x = (x | (x << 12)) & 0x000f000fu;
+    x = (x | (x << 6)) & 0x03030303u;
+    return (x | (x << 3)) & 0x11111111u;
+}
+ZFPX_HD uint32_t gather2(uint32_t x)
+{
+    x &= 0x55555555u;
+    x = (x | (x >> 1)) & 0x33333333u;
+    x = (x | (x >> 2)) & 0x0f0f0f0fu;
+    x = (x | (x >> 4)) & 0x00ff00ffu;
+    return (x | (x >> 8)) & 0xffffu;
+}
+ZFPX_HD uint32_t gather3(uint32_t x)
+{
+    x &= 0x09249249u;
+    x = (x | (x >> 2)) & 0x030c30c3u;
+    x = (x | (x >> 4)) & 0x0300f00fu;
+    x = (x | (x >> 8)) & 0x030000ffu;
+    return (x | (x >> 16)) & 0x3ffu;
+}
+ZFPX_HD uint32_t gather4(uint32_t x)
+{
+    x &= 0x11111111u;
+    x = (x | (x >> 3)) & 0x03030303u;
+    x = (x | (x >> 6)) & 0x000f000fu;
+    return (x | (x >> 12)) & 0xffu;
+}
+
+// The word a 1-D block's 4 RATE bits fill, and the interleaves in it: as many
+// planes as can matter from bit 9 on.
+template <int RATE>
+struct Word1 {
+    typedef uint64_t T;
+    ZFPX_HD static T runs1(uint32_t a) { return ((T)spread2(a >> 16) << 32) | spread2(a); }
+    ZFPX_HD static T runs2(uint32_t a, uint32_t b)
+    {
+        return ((T)(spread3(a >> 10) | (spread3(b >> 10) << 1)) << 30) | spread3(a) | (spread3(b) << 1);
+    }
+    ZFPX_HD static T tail(const uint32_t (&v)[4], int p)
+    {
+        T r = 0;
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const uint32_t a = shr_any(v[i], p);
+            r |= (((T)spread4(a >> 8) << 32) | spread4(a)) << i;
+        }
+        return r;
+    }
+    ZFPX_HD static uint32_t of_runs1(T w) { return gather2((uint32_t)w) | (gather2((uint32_t)(w >> 32)) << 16); }
+    ZFPX_HD static uint32_t of_runs2(T w) { return gather3((uint32_t)w) | (gather3((uint32_t)(w >> 30)) << 10); }
+    ZFPX_HD static uint32_t of_tail(T w, int i)
+    {
+        return gather4((uint32_t)(w >> i)) | (gather4((uint32_t)(w >> 32) >> i) << 8);
+    }
+    static constexpr T kGroup1 = 0xaaaaaaaaaaaaaaaaull, kGroup2 = 0x4924924924924924ull;
+    ZFPX_HD static int low(T w) { return lowest_set(w); }
+};
+template <>
+struct Word1<8> {
+    typedef uint32_t T;
+    ZFPX_HD static T runs1(uint32_t a) { return spread2(a); }
+    ZFPX_HD static T runs2(uint32_t a, uint32_t b) { return spread3(a) | (spread3(b) << 1); }
+    ZFPX_HD static T tail(const uint32_t (&v)[4], int p)
+    {
+        T r = 0;
+#pragma unroll
+        for (int i = 0; i < 4; i++) r |= spread4(shr_any(v[i], p)) << i;
+        return r;
+    }
+    ZFPX_HD static uint32_t of_runs1(T w) { return gather2(w); }
+    ZFPX_HD static uint32_t of_runs2(T w) { return gather3(w); }
+    ZFPX_HD static uint32_t of_tail(T w, int i) { return gather4(w >> i); }
+    static constexpr T kGroup1 = 0xaaaaaaaau, kGroup2 = 0x24924924u;
+    ZFPX_HD static int low(T w) { return lowest_set32(w); }
+};
+
 // Encodes K blocks x[b][0..3]; w[b] = the block's 4 RATE bits.
 template <int RATE, int K>
 ZFPX_HD void encode_blocks1(const float (&x)[K][4], const Plane4Enc &tab, uint64_t (&w)[K])
 {
-    constexpr int END = 4 * RATE;
-    uint32_t u[K][4];
-    int pos[K], n[K];
+    typedef typename Word1<RATE>::T T;
 #pragma unroll
     for (int b = 0; b < K; b++) {
         uint32_t amax = 0;
@@ -1076,83 +1240,104 @@ ZFPX_HD void encode_blocks1(const float (&x)[K][4], const Plane4Enc &tab, uint64
         const QuantScale qs(zero ? 127 : E);
         int32_t q0 = qs(x[b][0]), q1 = qs(x[b][1]), q2 = qs(x[b][2]), q3 = qs(x[b][3]);
         lift_fwd(q0, q1, q2, q3);
-        u[b][0] = to_negabinary(q0); u[b][1] = to_negabinary(q1);
-        u[b][2] = to_negabinary(q2); u[b][3] = to_negabinary(q3);
-        w[b] = zero ? 0ull : 1ull | ((uint64_t)(E + 1) << 1);      // header, 9 bits
-        pos[b] = zero ? END : 9;
-        n[b] = 0;
-    }
-#pragma unroll 1
-    for (int k = 31; k >= 0; k--) {
-        bool more = false;
-#pragma unroll
-        for (int b = 0; b < K; b++) {
-            if (pos[b] >= END) continue;
-            const uint32_t X = ((u[b][0] >> k) & 1u) | (((u[b][1] >> k) & 1u) << 1) | (((u[b][2] >> k) & 1u) << 2) |
-                               (((u[b][3] >> k) & 1u) << 3);
-            const uint32_t e = tab.e[n[b] * 16 + (int)X];
-            w[b] |= (uint64_t)(e & 127u) << pos[b];                // pos < END <= 64
-            pos[b] += (int)((e >> 7) & 7u);
-            n[b] = (int)(e >> 10);
-            more |= pos[b] < END;
+        const uint32_t u[4] = {to_negabinary(q0), to_negabinary(q1), to_negabinary(q2), to_negabinary(q3)};
+        const uint32_t v[4] = {reverse32(u[0]), reverse32(u[1]), reverse32(u[2]), reverse32(u[3])};
+        const uint32_t o2 = u[2] | u[3], o1 = u[1] | o2, o0 = u[0] | o1;
+        T r = (T)(1u | ((uint32_t)(E + 1) << 1));                  // header, 9 bits
+        int n = 0, pos = 9, p = 0;                                 // p: the next plane (31 - p)
+        // a plane with new ones: its table entry, for plane 31 - e
+        auto event = [&](int e) {
+            const uint32_t X = (shr_any(v[0], e) & 1u) | ((shr_any(v[1], e) & 1u) << 1) |
+                               ((shr_any(v[2], e) & 1u) << 2) | ((shr_any(v[3], e) & 1u) << 3);
+            const uint32_t c = tab.e[n * 16 + (int)X];
+            r |= shl_any((T)(c & 127u), pos);
+            pos += (int)((c >> 7) & 7u);
+            n = (int)(c >> 10);
+            p = e + 1;
+        };
+        const int e0 = leading_zeros32(o0);                        // zeros up to the first one
+        pos += e0;
+        if (e0 < 32) event(e0);
+        if (n == 1) {
+            const int e1 = leading_zeros32(o1), run = e1 - p;
+            r |= shl_any(Word1<RATE>::runs1(shr_any(v[0], p) & (shl_any(1u, run) - 1u)), pos);
+            pos += 2 * run;
+            if (e1 < 32) event(e1);
         }
-        if (!more) break;
+        if (n == 2) {
+            const int e2 = leading_zeros32(o2), run = e2 - p;
+            const uint32_t m = shl_any(1u, run) - 1u;
+            r |= shl_any(Word1<RATE>::runs2(shr_any(v[0], p) & m, shr_any(v[1], p) & m), pos);
+            pos += 3 * run;
+            if (e2 < 32) event(e2);
+        }
+        if (n >= 3) r |= shl_any(Word1<RATE>::tail(v, p), pos);
+        w[b] = zero ? 0ull : (uint64_t)r;
     }
-#pragma unroll
-    for (int b = 0; b < K; b++) w[b] &= low_mask(END);
 }
 
 // Decodes K blocks from their 4 RATE-bit words.
 template <int RATE, int K>
 ZFPX_HD void decode_blocks1(const uint64_t (&win)[K], const Plane4Dec &tab, float (&x)[K][4])
 {
+    typedef typename Word1<RATE>::T T;
     constexpr int END = 4 * RATE;
-    uint64_t w[K];
-    uint32_t u[K][4];
-    int pos[K], n[K];
 #pragma unroll
     for (int b = 0; b < K; b++) {
-        w[b] = win[b] & low_mask(END);
-        pos[b] = (w[b] & 1ull) ? 9 : END;
-        n[b] = 0;
-        u[b][0] = u[b][1] = u[b][2] = u[b][3] = 0u;
-    }
-#pragma unroll 1
-    for (int k = 31; k >= 0; k--) {
-        bool more = false;
-#pragma unroll
-        for (int b = 0; b < K; b++) {
-            if (pos[b] >= END) continue;
-            const int r = END - pos[b];
-            uint32_t w7 = (uint32_t)(w[b] >> pos[b]) & 127u;       // pos < END <= 64
-            if (r < 7) w7 &= (1u << r) - 1u;
-            const uint32_t d = tab.d[n[b] * 128 + (int)w7];
-            uint32_t X = d & 15u;
+        T w = (T)win[b] >> 9;
+        uint32_t v[4] = {0u, 0u, 0u, 0u};                          // planes from 31 down, bit-reversed
+        int n = 0, pos = 9, p = 0;
+        // a plane with new ones at the start of w, for plane 31 - e (e < 32)
+        auto event = [&](int e) {
+            const uint32_t d = tab.d[n * 128 + (int)((uint32_t)w & 127u)];
             const int len = (int)((d >> 4) & 7u);
-            if (len > r) {                                         // the budget cuts this plane
-                if (n[b] < 4) X &= 7u;
-                pos[b] = END;
-            } else {
-                pos[b] += len;
-                n[b] = (int)(d >> 7);
-            }
-            u[b][0] |= (X & 1u) << k;
-            u[b][1] |= ((X >> 1) & 1u) << k;
-            u[b][2] |= ((X >> 2) & 1u) << k;
-            u[b][3] |= ((X >> 3) & 1u) << k;
-            more |= pos[b] < END;
-        }
-        if (!more) break;
-    }
+            const bool cut = len > END - pos;                      // the budget ends inside it
+            const uint32_t X = cut ? d & 7u : d & 15u;
 #pragma unroll
-    for (int b = 0; b < K; b++) {
-        if (!(w[b] & 1ull)) {
+            for (int i = 0; i < 4; i++) v[i] |= ((X >> i) & 1u) << e;
+            w = cut ? (T)0 : w >> len;
+            pos += len;
+            n = cut ? -1 : (int)(d >> 7);
+            p = e + 1;
+        };
+        if (w) {
+            const int e0 = Word1<RATE>::low(w);
+            w >>= e0;
+            pos += e0;
+            if (e0 < 32) event(e0);
+        }
+        if (n == 1) {
+            const T t = w & Word1<RATE>::kGroup1;
+            const int run = t ? Word1<RATE>::low(t) >> 1 : 32;
+            const T m = shl_any((T)1, 2 * run) - (T)1;
+            v[0] |= shl_any(Word1<RATE>::of_runs1(w & m), p);
+            w = shr_any(w, 2 * run);
+            pos += 2 * run;
+            if (p + run < 32 && t) event(p + run);
+            else n = -1;
+        }
+        if (n == 2) {
+            const T t = w & Word1<RATE>::kGroup2;
+            const int run = t ? (Word1<RATE>::low(t) * 43) >> 7 : 32;    // the group bits are at 3 i + 2
+            const T m = shl_any((T)1, 3 * run) - (T)1;
+            v[0] |= shl_any(Word1<RATE>::of_runs2(w & m), p);
+            v[1] |= shl_any(Word1<RATE>::of_runs2((w & m) >> 1), p);
+            w = shr_any(w, 3 * run);
+            pos += 3 * run;
+            if (p + run < 32 && t) event(p + run);
+            else n = -1;
+        }
+        if (n >= 3) {
+#pragma unroll
+            for (int i = 0; i < 4; i++) v[i] |= shl_any(Word1<RATE>::of_tail(w, i), p);
+        }
+        if (!(win[b] & 1ull)) {
             x[b][0] = x[b][1] = x[b][2] = x[b][3] = 0.0f;
             continue;
         }
-        const int e = (int)((w[b] >> 1) & 0xffu);
-        int32_t q0 = from_negabinary(u[b][0]), q1 = from_negabinary(u[b][1]);
-        int32_t q2 = from_negabinary(u[b][2]), q3 = from_negabinary(u[b][3]);
+        const int e = (int)((win[b] >> 1) & 0xffu);
+        int32_t q0 = from_negabinary(reverse32(v[0])), q1 = from_negabinary(reverse32(v[1]));
+        int32_t q2 = from_negabinary(reverse32(v[2])), q3 = from_negabinary(reverse32(v[3]));
         lift_inv(q0, q1, q2, q3);
         if (e >= 31) {
             const float sc = dequant_scale(e);
