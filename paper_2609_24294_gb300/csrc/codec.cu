@@ -525,10 +525,18 @@ int grid_for(K kernel, int64_t nunits, int warps = kWarps)
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 // Consecutive 32-block units per warp of the 3-D kernels, [encode][rate 16?];
-// 0 = default.  The default was picked by timing on GB300 (the autotuner can
-// override it); results never depend on it.
+// 0 = default: two, and one in launches of at most kFewUnits units per
+// resident warp.  A warp's units run one after the other, so where a launch is
+// little more than one wave of warps a second unit doubles its time (a 64 x 32
+// x 8 field: 18.4 us a kernel with two, 10.2 with one; 233 x 117 x 137: 36.9 /
+// 36.9 us against 26.6 / 28.7 compress / decompress), and one also ends a launch of
+// several waves more evenly (640 x 320 x 137, five waves: 69.6 / 77.8 against
+// 67.6 / 75.8); in long launches two save part of the per-CTA start-up
+// (twenty waves: 243 against 256 us).  The autotuner can override it; results
+// never depend on it.
 std::atomic<int> g_upw[2][2] = {{{0}, {0}}, {{0}, {0}}};
 constexpr int kDefaultUpw = 2;
+constexpr int kFewUnits = 8;
 
 // One launch of a 3-D codec kernel (either alignment instantiation): one
 // warp per upw consecutive units.
@@ -536,7 +544,11 @@ template <class In, class Out>
 void launch3(void (*kernel)(In, Out, LaunchGeom, int), int warps, int encode, int rate, LaunchGeom g,
              cudaStream_t st, In in, Out out, int layout)
 {
-    g.upw = units_per_warp(encode, rate);
+    g.upw = g_upw[encode ? 1 : 0][rate == 16 ? 1 : 0].load(std::memory_order_relaxed);
+    if (g.upw <= 0) {
+        const int64_t resident = (int64_t)num_sms() * occupancy((const void *)kernel, 32 * warps) * warps;
+        g.upw = g.nunits <= kFewUnits * resident ? 1 : kDefaultUpw;
+    }
     const int64_t per_cta = (int64_t)g.upw * warps;
     const int64_t grid = (g.nunits + per_cta - 1) / per_cta;
     kernel<<<(unsigned)grid, 32 * warps, 0, st>>>(in, out, g, layout);
