@@ -12,74 +12,30 @@
 // rate-16 stream, and the rate-16 decoder reads the same block from those L
 // bits followed by zeros (zeros after the last coded plane are empty planes).
 //
-// Encode: the rate-16 encoder writes every block to a 128-byte slot; one
-// thread per block walks its slot's planes down to kmin to find L; an
-// exclusive scan of the L (per 1024-block tile, then over the tiles) gives
-// every block's bit offset; one thread per block ORs its L bits into the
-// zeroed payload at that offset (words shared by neighbouring blocks take
-// atomic ORs).  Decode: the same scan, one thread per block copies its L bits
-// back into a zeroed slot, then the rate-16 decoder.
+// Encode: the rate-16 encoder writes every block to a 128-byte slot and, as it
+// walks the planes, its bit count L; an exclusive scan of the L (per 1024-block
+// tile, then over the tiles) gives every block's bit offset; one warp per 32
+// blocks shifts their bits together in shared memory and writes the payload
+// words that start in them, each once (the last with the leading bits of the
+// blocks that follow), so the payload needs no zeroing but its tail and no
+// atomics in global memory.  Decode: the same scan, then the rate-16
+// decoder, which cuts each block's bits out of the payload as it loads them.
+// What bounds it: the codec; the rest moves a slot once out and once in.  With a
+// parse of every slot for L, a zeroed payload filled by atomics, and slots
+// copied out for the decoder, compress, exchange and decompress of a 640 x 320 x
+// 137 field over 4 x 4 ranks at tolerance 1e-3 took 359, 97 and 215 us; now 155,
+// 27 and 146.
 #include <algorithm>
 #include <cmath>
 #include <vector>
 #include <cuda_runtime.h>
 
 #include "zfpx_internal.h"
-#include "zfpx_block.cuh"
 
 namespace zfpx {
 namespace {
 
-using namespace blk;
-
-constexpr int kTile = 1024;                  // blocks per scan tile (one CTA)
-constexpr int kSlotWords = 16;               // 1024 bits per block slot
-constexpr int kCutBits = 64 * kSlotWords;
-
-// Lowest plane kept: the accuracy rule, or 32 - prec in precision mode (prec > 0).
-__device__ __forceinline__ int acc_kmin(int emax, int minexp, int prec)
-{
-    if (prec > 0) return 32 - prec;
-    const int k = minexp - emax + 22;
-    return k < 0 ? 0 : (k > 32 ? 32 : k);
-}
-
-// Reader over one block's slot in global memory; bits past the slot read as 0.
-struct SlotReader {
-    const uint64_t *w;
-    int pos;
-    __device__ __forceinline__ uint64_t peek() const
-    {
-        const int i = pos >> 6, sh = pos & 63;
-        const uint64_t lo = i < kSlotWords ? __ldg(w + i) : 0ull;
-        const uint64_t hi = i + 1 < kSlotWords ? __ldg(w + i + 1) : 0ull;
-        return sh ? (lo >> sh) | (hi << (64 - sh)) : lo;
-    }
-    __device__ __forceinline__ void skip(int k) { pos += k; }
-};
-
-// L for every block: parse the slot's planes 31 .. kmin with the rate-16 budget.
-__global__ void __launch_bounds__(256) acc_lengths_kernel(const uint64_t *__restrict__ slots, int64_t nblocks,
-                                                          int minexp, int prec, uint16_t *__restrict__ lengths)
-{
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nblocks) return;
-    const uint64_t *w = slots + b * kSlotWords;
-    const uint64_t head = __ldg(w);
-    int L;
-    if (!(head & 1ull)) {
-        L = 1;
-    } else {
-        const int emax = (int)((head >> 1) & 0xffu) - 127;
-        const int kmin = acc_kmin(emax, minexp, prec);
-        SlotReader rd{w, 9};
-        int n = 0, R = kCutBits - 9;
-#pragma unroll 1
-        for (int k = 31; k >= kmin && R > 0; k--) (void)decode_plane<64>(rd, n, R);
-        L = kCutBits - R;
-    }
-    lengths[b] = (uint16_t)L;
-}
+constexpr int kTile = kAccTile;              // blocks per scan tile (one CTA)
 
 // Exclusive scan of the lengths inside each tile of kTile blocks; the tile's
 // total goes to totals[tile].
@@ -114,99 +70,170 @@ __global__ void __launch_bounds__(kTile) acc_scan_tiles_kernel(const uint16_t *_
     if (t == kTile - 1) totals[blockIdx.x] = warp_sum[kTile / 32 - 1];
 }
 
+// Exclusive sum over a CTA of kTile threads (`sums`: kTile / 32 shared values);
+// *total gets the sum of all.  Every thread calls it; sums may be reused after
+// the next barrier.
+__device__ __forceinline__ uint64_t cta_scan(uint64_t v, uint64_t *sums, uint64_t *total)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint64_t x = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint64_t y = __shfl_up_sync(0xffffffffu, x, d);
+        if (lane >= d) x += y;
+    }
+    if (lane == 31) sums[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        uint64_t s = sums[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint64_t y = __shfl_up_sync(0xffffffffu, s, d);
+            if (lane >= d) s += y;
+        }
+        sums[lane] = s;
+    }
+    __syncthreads();
+    *total = sums[kTile / 32 - 1];
+    return (wid ? sums[wid - 1] : 0ull) + x - v;
+}
+
 // Exclusive scan of the tile totals (one CTA, sequential over chunks of
 // kTile tiles); the grand total goes to *total_bits.
 __global__ void __launch_bounds__(kTile) acc_scan_totals_kernel(const uint64_t *__restrict__ totals, int64_t ntiles,
                                                                 uint64_t *__restrict__ tile_off,
                                                                 uint64_t *__restrict__ total_bits)
 {
-    __shared__ uint64_t warp_sum[kTile / 32];
-    __shared__ uint64_t carry;
-    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    if (t == 0) carry = 0;
-    __syncthreads();
+    __shared__ uint64_t sums[kTile / 32];
+    uint64_t carry = 0, all;
     for (int64_t base = 0; base < ntiles; base += kTile) {
-        const int64_t i = base + t;
-        const uint64_t v = i < ntiles ? totals[i] : 0ull;
-        uint64_t x = v;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint64_t y = __shfl_up_sync(0xffffffffu, x, d);
-            if (lane >= d) x += y;
-        }
-        if (lane == 31) warp_sum[wid] = x;
-        __syncthreads();
-        if (wid == 0) {
-            uint64_t s = warp_sum[lane];
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint64_t y = __shfl_up_sync(0xffffffffu, s, d);
-                if (lane >= d) s += y;
-            }
-            warp_sum[lane] = s;
-        }
-        __syncthreads();
-        const uint64_t c = carry;
-        if (i < ntiles) tile_off[i] = c + (wid ? warp_sum[wid - 1] : 0ull) + x - v;
-        __syncthreads();
-        if (t == 0) carry = c + warp_sum[kTile / 32 - 1];
+        const int64_t i = base + threadIdx.x;
+        const uint64_t before = cta_scan(i < ntiles ? totals[i] : 0ull, sums, &all);
+        if (i < ntiles) tile_off[i] = carry + before;
+        carry += all;
         __syncthreads();
     }
-    if (t == 0) *total_bits = carry;
+    if (threadIdx.x == 0) *total_bits = carry;
 }
 
-// Every block ORs its L bits into the zeroed payload at its bit offset.
-__global__ void __launch_bounds__(256) acc_pack_kernel(const uint64_t *__restrict__ slots, int64_t nblocks,
-                                                       const uint16_t *__restrict__ lengths,
-                                                       const uint32_t *__restrict__ local,
-                                                       const uint64_t *__restrict__ tile_off,
-                                                       unsigned long long *__restrict__ payload)
+// The block list a pack kernel walks: M messages in send order (msgs NULL: one
+// message, its slots from 0 on, its payload from word 0 on).
+struct AccList {
+    const AccMsg *msgs;
+    const int64_t *pay;        // first payload word of each message
+    const uint16_t *lengths;
+    const uint32_t *local;
+    const uint64_t *tile_off;
+    int M;
+    int64_t G;
+    __device__ __forceinline__ uint64_t bit(int64_t g) const { return tile_off[g / kTile] + local[g]; }
+    // the last message whose blocks start at or before g
+    __device__ __forceinline__ int message(int64_t g) const
+    {
+        int lo = 0, hi = M - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (msgs[mid].gb0 <= g) lo = mid; else hi = mid - 1;
+        }
+        return lo;
+    }
+    // block g's first bit in the payload and its slot's first byte
+    __device__ __forceinline__ void place(int64_t g, uint64_t &off, int64_t &slot) const
+    {
+        if (!msgs) {
+            off = bit(g);
+            slot = g * 128;
+            return;
+        }
+        const int m = message(g);
+        const AccMsg a = msgs[m];
+        off = (uint64_t)pay[m] * 64 + (bit(g) - bit(a.gb0));
+        slot = a.slot_send + (g - a.gb0) * 128;
+    }
+};
+
+// One warp per 32 consecutive blocks writes the payload words whose first bit
+// lies in them.  Block by block the lanes read the slot's 32 words, shift them
+// to the block's place in the warp's shared words and OR them in; the word the
+// last block ends in also takes the first bits of the blocks that follow, up to
+// 63 of them.  (Messages start on words, so every word's first bit is in some
+// block.)
+constexpr int kPackWarps = 4;
+constexpr int kPackWords = 32 * 32 + 4;       // 32-bit words: 32 blocks of at most 16 64-bit words, and the last word
+__global__ void __launch_bounds__(32 * kPackWarps) acc_pack_kernel(AccList P, const uint8_t *__restrict__ slots,
+                                                                   uint64_t *__restrict__ payload)
 {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nblocks) return;
-    const uint64_t off = tile_off[b / kTile] + local[b];
-    const int L = lengths[b];
-    const uint64_t *w = slots + b * kSlotWords;
-    const int sh = (int)(off & 63);
-    unsigned long long *d = payload + (off >> 6);
+    __shared__ __align__(8) uint32_t buf[kPackWarps][kPackWords];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t g0 = ((int64_t)blockIdx.x * kPackWarps + wid) * 32;
+    if (g0 >= P.G) return;
+    uint32_t *w = buf[wid];
+    for (int i = lane; i < kPackWords; i += 32) w[i] = 0u;
+    const int n = (int)min((int64_t)32, P.G - g0);
+    const int64_t g = g0 + min(lane, n - 1);
+    uint64_t off;
+    int64_t slot;
+    P.place(g, off, slot);
+    const int L = P.lengths[g];
+    const uint64_t first = __shfl_sync(0xffffffffu, off, 0), end = __shfl_sync(0xffffffffu, off + L, n - 1);
+    const uint64_t base = first & ~63ull;      // w[0] holds the payload's bits from here on
+    const uint32_t rel = (uint32_t)(off - base);
+    __syncwarp();
+    // eight blocks at a time, all their loads ahead of the shifting (past the
+    // warp's last block lengths are 0)
+    const int Lw = lane < n ? L : 0;
 #pragma unroll 1
-    for (int i = 0; 64 * i < L; i++) {
-        uint64_t v = __ldg(w + i);
-        const int rem = L - 64 * i;
-        if (rem < 64) v &= (1ull << rem) - 1ull;
-        if (!v) continue;
-        atomicOr(d + i, (unsigned long long)(v << sh));
-        if (sh && (v >> (64 - sh))) atomicOr(d + i + 1, (unsigned long long)(v >> (64 - sh)));
+    for (int b0 = 0; b0 < n; b0 += 8) {
+        uint32_t v[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            const int len = __shfl_sync(0xffffffffu, Lw, b0 + k) - 32 * lane;
+            const int64_t s = __shfl_sync(0xffffffffu, slot, b0 + k);
+            v[k] = len > 0 ? __ldg(reinterpret_cast<const uint32_t *>(slots + s) + lane) : 0u;
+            if (len > 0 && len < 32) v[k] &= (1u << len) - 1u;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            const uint32_t r = __shfl_sync(0xffffffffu, rel, b0 + k);
+            const uint64_t x = (uint64_t)v[k] << (r & 31u);
+            if ((uint32_t)x) atomicOr(w + (r >> 5) + lane, (uint32_t)x);
+            if ((uint32_t)(x >> 32)) atomicOr(w + (r >> 5) + lane + 1, (uint32_t)(x >> 32));
+        }
     }
+    // the words owned: those starting at or after `first`, up to the one `end` lies in
+    const uint64_t j0 = (first + 63) >> 6, j1 = (end + 63) >> 6;
+    if (j1 > j0 && (end & 63u)) {
+        const uint64_t wend = j1 * 64;
+        for (int64_t t = g0 + n + lane; ; t += 32) {
+            uint64_t o = wend;
+            int64_t sl = 0;
+            if (t < P.G) P.place(t, o, sl);
+            if (o < wend) {
+                uint64_t v = __ldg(reinterpret_cast<const uint64_t *>(slots + sl));
+                const int len = P.lengths[t];
+                if (len < 64) v &= (1ull << len) - 1ull;
+                v <<= o & 63u;
+                uint32_t *d = w + (uint32_t)((wend - 64 - base) >> 5);
+                if ((uint32_t)v) atomicOr(d, (uint32_t)v);
+                if ((uint32_t)(v >> 32)) atomicOr(d + 1, (uint32_t)(v >> 32));
+            }
+            if (!__all_sync(0xffffffffu, o < wend)) break;
+        }
+    }
+    __syncwarp();
+    const uint64_t *w64 = reinterpret_cast<const uint64_t *>(w);
+    for (uint64_t j = j0 + lane; j < j1; j += 32) payload[j] = w64[j - (base >> 6)];
 }
 
-// Every block copies its L bits back into a zeroed 1024-bit slot.
-__global__ void __launch_bounds__(256) acc_unpack_kernel(const uint64_t *__restrict__ payload, int64_t pwords,
-                                                         int64_t nblocks, const uint16_t *__restrict__ lengths,
-                                                         const uint32_t *__restrict__ local,
-                                                         const uint64_t *__restrict__ tile_off,
-                                                         uint64_t *__restrict__ slots)
+// Zeroes the payload's words from its end on: *count words (bits rounded up
+// to words where `bits` is set) up to `words`.
+__global__ void __launch_bounds__(256) acc_zero_tail_kernel(uint64_t *__restrict__ payload,
+                                                            const uint64_t *__restrict__ count, int bits, int64_t words)
 {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nblocks) return;
-    const uint64_t off = tile_off[b / kTile] + local[b];
-    const int L = min((int)lengths[b], kCutBits);
-    const int sh = (int)(off & 63);
-    const int64_t j0 = (int64_t)(off >> 6);
-    uint64_t *s = slots + b * kSlotWords;
-#pragma unroll
-    for (int i = 0; i < kSlotWords; i++) {
-        uint64_t v = 0;
-        const int rem = L - 64 * i;
-        if (rem > 0) {
-            const int64_t j = j0 + i;
-            const uint64_t lo = j < pwords ? __ldg(payload + j) : 0ull;
-            const uint64_t hi = (sh && j + 1 < pwords) ? __ldg(payload + j + 1) : 0ull;
-            v = sh ? (lo >> sh) | (hi << (64 - sh)) : lo;
-            if (rem < 64) v &= (1ull << rem) - 1ull;
-        }
-        s[i] = v;
-    }
+    const int64_t used = (int64_t)(bits ? (*count + 63) / 64 : *count);
+    for (int64_t i = used + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words;
+         i += (int64_t)gridDim.x * blockDim.x)
+        payload[i] = 0ull;
 }
 
 struct AccWork {
@@ -240,6 +267,16 @@ AccWork acc_carve(void *work, int64_t nb)
     return a;
 }
 
+int plan_geom(zfpx_plan p, LaunchGeom &g)
+{
+    DevTable *t = nullptr;
+    const int rc = get_table(p, 16, UNIT_BLOCKS32, &t);
+    if (rc) return rc;
+    g.msgs = t->d_msgs; g.nmsg = (int)p->msgs.size(); g.nunits = t->nunits;
+    for (int a = 0; a < 3; a++) { g.ss[a] = p->ss[a]; g.ds[a] = p->ds[a]; }
+    return ZFPX_OK;
+}
+
 int acc_scan(const AccWork &a, const uint16_t *lengths, uint64_t *total_bits, cudaStream_t st)
 {
     acc_scan_tiles_kernel<<<(unsigned)a.ntiles, kTile, 0, st>>>(lengths, a.nblocks, a.local, a.totals);
@@ -247,6 +284,30 @@ int acc_scan(const AccWork &a, const uint16_t *lengths, uint64_t *total_bits, cu
     acc_scan_totals_kernel<<<1, kTile, 0, st>>>(a.totals, a.ntiles, a.tile_off, total_bits);
     count_launch();
     return check_launch();
+}
+
+// Packs the slots of the listed blocks; *count (words, or bits) ends the payload.
+int acc_pack(const AccList &P, const uint8_t *slots, uint8_t *payload, const uint64_t *count, int bits, cudaStream_t st)
+{
+    const int64_t per_cta = 32 * kPackWarps;
+    acc_pack_kernel<<<(unsigned)((P.G + per_cta - 1) / per_cta), 32 * kPackWarps, 0, st>>>(
+        P, slots, reinterpret_cast<uint64_t *>(payload));
+    count_launch();
+    const int64_t words = P.G * 16, want = (words + 255) / 256;
+    acc_zero_tail_kernel<<<(unsigned)std::min<int64_t>(want, (int64_t)num_sms() * 8), 256, 0, st>>>(
+        reinterpret_cast<uint64_t *>(payload), count, bits, words);
+    count_launch();
+    return check_launch();
+}
+
+// Launch geometry of a raw array (its one-message table) for the rate-16 codec.
+int raw_geom(const int64_t n[3], const int64_t stride[3], const void *base, LaunchGeom &g, int &vec)
+{
+    zfpx_plan p = nullptr;
+    int rc = raw_plan(3, n, stride, &p);
+    if (!rc) rc = plan_geom(p, g);
+    if (!rc) vec = codec_vec_ok(base, stride, p) ? 1 : 0;
+    return rc;
 }
 
 bool aligned(const void *p, size_t a) { return ((uintptr_t)p % a) == 0; }
@@ -282,18 +343,15 @@ static int encode_variable(const float *d_in, const int64_t n[3], const int64_t 
     if (cap < (size_t)nb * 128 || work_bytes < acc_work_bytes(nb)) return ZFPX_ESIZE;
     cudaStream_t st = (cudaStream_t)stream;
     const AccWork a = acc_carve(d_work, nb);
-    int rc = zfpx_encode(3, 16, d_in, n, stride, reinterpret_cast<uint8_t *>(a.slots), (size_t)nb * 128, stream);
+    LaunchGeom g{};
+    int vec = 0, rc = raw_geom(n, stride, d_in, g, vec);
     if (rc) return rc;
-    const unsigned grid = (unsigned)((nb + 255) / 256);
-    acc_lengths_kernel<<<grid, 256, 0, st>>>(a.slots, nb, minexp, prec, d_lengths);
-    count_launch();
-    if ((rc = check_launch())) return rc;
+    if ((rc = launch_encode_lengths(d_in, reinterpret_cast<uint8_t *>(a.slots), g, vec,
+                                    AccEncode{d_lengths, nullptr, minexp, prec}, st)))
+        return rc;
     if ((rc = acc_scan(a, d_lengths, d_total_bits, st))) return rc;
-    if (cudaMemsetAsync(d_payload, 0, (size_t)nb * 128, st) != cudaSuccess) return ZFPX_ECUDA;
-    acc_pack_kernel<<<grid, 256, 0, st>>>(a.slots, nb, d_lengths, a.local, a.tile_off,
-                                          reinterpret_cast<unsigned long long *>(d_payload));
-    count_launch();
-    return check_launch();
+    return acc_pack(AccList{nullptr, nullptr, d_lengths, a.local, a.tile_off, 1, nb},
+                    reinterpret_cast<const uint8_t *>(a.slots), d_payload, d_total_bits, 1, st);
 }
 
 int zfpx_encode_accuracy(const float *d_in, const int64_t n[3], const int64_t stride[3], double tolerance,
@@ -326,13 +384,13 @@ int zfpx_decode_accuracy(const uint16_t *d_lengths, const uint8_t *d_payload, si
     if (work_bytes < acc_work_bytes(nb)) return ZFPX_ESIZE;
     cudaStream_t st = (cudaStream_t)stream;
     const AccWork a = acc_carve(d_work, nb);
-    int rc = acc_scan(a, d_lengths, a.total, st);
-    if (rc) return rc;
-    acc_unpack_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(
-        reinterpret_cast<const uint64_t *>(d_payload), (int64_t)(len / 8), nb, d_lengths, a.local, a.tile_off, a.slots);
-    count_launch();
-    if ((rc = check_launch())) return rc;
-    return zfpx_decode(3, 16, reinterpret_cast<const uint8_t *>(a.slots), (size_t)nb * 128, n, stride, d_out, stream);
+    LaunchGeom g{};
+    int vec = 0, rc = raw_geom(n, stride, d_out, g, vec);
+    if (rc || (rc = acc_scan(a, d_lengths, a.total, st))) return rc;
+    return launch_decode_payload(d_out, g, vec,
+                                 AccDecode{reinterpret_cast<const uint64_t *>(d_payload), (int64_t)(len / 8), d_lengths,
+                                           a.local, a.tile_off, nullptr, nullptr},
+                                 st);
 }
 
 }  // extern "C"
@@ -347,119 +405,58 @@ namespace zfpx {
 std::vector<int64_t> layout_offsets(const zfpx_plan_s *p, int rate, int layout, int64_t *total);
 namespace {
 
-// One message as the accuracy kernels see it (send-order index m).
-struct AccMsg {
-    int64_t gb0;        // first block in the send-order block list (and lengths array)
-    int64_t gr0;        // first block in the receive-order block list
-    int64_t nb;         // blocks
-    int64_t slot_send;  // byte offset of its rate-16 slots in the send layout
-    int64_t slot_recv;  // byte offset of its rate-16 slots in the receive layout
-};
-
 struct PlanAcc {
     const AccMsg *msgs;       // M, send order
     const int32_t *rorder;    // M: send index of the message at receive position r
-    const int64_t *rgb0;      // M: gr0 of the message at receive position r (ascending)
     int64_t *pay_send;        // M: payload word offset in the send buffer
     int64_t *pay_recv;        // M: payload word offset in the receive buffer
     int M;
     int64_t G;                // blocks in all messages
 };
 
-__device__ __forceinline__ int last_le(const int64_t *a, const AccMsg *m, int M, int64_t g, bool by_msgs)
+// Word counts and payload offsets of the messages: one CTA, kTile messages at a
+// time.  With `send` the counts come from the block scan of the send-order
+// lengths and are written to words[]; otherwise words[] is input.  *used (if
+// not NULL) gets the sum of the counts.
+__global__ void __launch_bounds__(kTile) pacc_messages_kernel(PlanAcc P, const uint32_t *__restrict__ local,
+                                                              const uint64_t *__restrict__ tile_off,
+                                                              const uint64_t *__restrict__ total,
+                                                              uint64_t *words, int send, uint64_t *used)
 {
-    int lo = 0, hi = M - 1;                  // last index whose start <= g (starts ascending)
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        const int64_t s = by_msgs ? m[mid].gb0 : a[mid];
-        if (s <= g) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ uint64_t goff(const uint32_t *local, const uint64_t *tile_off, int64_t G,
-                                         const uint64_t *total, int64_t g)
-{
-    return g < G ? tile_off[g / kTile] + local[g] : *total;
-}
-
-__global__ void __launch_bounds__(256) pacc_lengths_kernel(PlanAcc P, const uint8_t *__restrict__ slots, int minexp,
-                                                           int prec, uint16_t *__restrict__ lengths)
-{
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= P.G) return;
-    const int m = last_le(nullptr, P.msgs, P.M, g, true);
-    const AccMsg &a = P.msgs[m];
-    const uint64_t *w = reinterpret_cast<const uint64_t *>(slots + a.slot_send) + (g - a.gb0) * kSlotWords;
-    const uint64_t head = __ldg(w);
-    int L = 1;
-    if (head & 1ull) {
-        const int kmin = acc_kmin((int)((head >> 1) & 0xffu) - 127, minexp, prec);
-        SlotReader rd{w, 9};
-        int n = 0, R = kCutBits - 9;
-#pragma unroll 1
-        for (int k = 31; k >= kmin && R > 0; k--) (void)decode_plane<64>(rd, n, R);
-        L = kCutBits - R;
-    }
-    lengths[g] = (uint16_t)L;
-}
-
-// Word counts and payload offsets of the messages (one thread: M is a few
-// thousand at most).  With `send` the counts come from the block scan of the
-// send-order lengths and are written to words[]; otherwise words[] is input.
-__global__ void pacc_messages_kernel(PlanAcc P, const uint32_t *__restrict__ local,
-                                     const uint64_t *__restrict__ tile_off, const uint64_t *__restrict__ total,
-                                     uint64_t *__restrict__ words, int send)
-{
-    if (threadIdx.x || blockIdx.x) return;
-    int64_t o = 0;
-    for (int m = 0; m < P.M; m++) {
-        if (send) {
-            const AccMsg &a = P.msgs[m];
-            const uint64_t bits = goff(local, tile_off, P.G, total, a.gb0 + a.nb) - goff(local, tile_off, P.G, total, a.gb0);
-            words[m] = (bits + 63) / 64;
+    __shared__ uint64_t sums[kTile / 32];
+    auto bit = [&](int64_t g) { return g < P.G ? tile_off[g / kTile] + local[g] : *total; };
+    uint64_t carry = 0, all;
+    for (int base = 0; base < P.M; base += kTile) {
+        const int m = base + threadIdx.x;
+        uint64_t v = 0;
+        if (m < P.M) {
+            if (send) {
+                const AccMsg a = P.msgs[m];
+                v = (bit(a.gb0 + a.nb) - bit(a.gb0) + 63) / 64;
+                words[m] = v;
+            } else {
+                v = words[m];
+            }
         }
-        P.pay_send[m] = o;
-        o += (int64_t)words[m];
+        const uint64_t before = cta_scan(v, sums, &all);
+        if (m < P.M) P.pay_send[m] = (int64_t)(carry + before);
+        carry += all;
+        __syncthreads();                          // sums, and words[] for the next loop
     }
-    o = 0;
-    for (int r = 0; r < P.M; r++) {
-        const int m = P.rorder[r];
-        P.pay_recv[m] = o;
-        o += (int64_t)words[m];
-    }
-}
-
-__global__ void __launch_bounds__(256) pacc_pack_kernel(PlanAcc P, const uint8_t *__restrict__ slots,
-                                                        const uint16_t *__restrict__ lengths,
-                                                        const uint32_t *__restrict__ local,
-                                                        const uint64_t *__restrict__ tile_off,
-                                                        const uint64_t *__restrict__ total,
-                                                        unsigned long long *__restrict__ payload)
-{
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= P.G) return;
-    const int m = last_le(nullptr, P.msgs, P.M, g, true);
-    const AccMsg &a = P.msgs[m];
-    const uint64_t off = (uint64_t)P.pay_send[m] * 64 +
-                         (goff(local, tile_off, P.G, total, g) - goff(local, tile_off, P.G, total, a.gb0));
-    const int L = lengths[g];
-    const uint64_t *w = reinterpret_cast<const uint64_t *>(slots + a.slot_send) + (g - a.gb0) * kSlotWords;
-    const int sh = (int)(off & 63);
-    unsigned long long *d = payload + (off >> 6);
-#pragma unroll 1
-    for (int i = 0; 64 * i < L; i++) {
-        uint64_t v = __ldg(w + i);
-        const int rem = L - 64 * i;
-        if (rem < 64) v &= (1ull << rem) - 1ull;
-        if (!v) continue;
-        atomicOr(d + i, (unsigned long long)(v << sh));
-        if (sh && (v >> (64 - sh))) atomicOr(d + i + 1, (unsigned long long)(v >> (64 - sh)));
+    if (used && threadIdx.x == 0) *used = carry;
+    carry = 0;
+    for (int base = 0; base < P.M; base += kTile) {
+        const int r = base + threadIdx.x;
+        const int m = r < P.M ? P.rorder[r] : 0;
+        const uint64_t before = cta_scan(r < P.M ? words[m] : 0ull, sums, &all);
+        if (r < P.M) P.pay_recv[m] = (int64_t)(carry + before);
+        carry += all;
+        __syncthreads();
     }
 }
 
-// The all-to-all-v on one GPU: CTA m moves message m's payload words and its
-// block bit counts from the send to the receive buffers.
+// The all-to-all-v on one GPU: CTAs (m, *) move message m's payload words and
+// its block bit counts from the send to the receive buffers, in equal parts.
 __global__ void __launch_bounds__(256) pacc_exchange_kernel(PlanAcc P, const uint64_t *__restrict__ words,
                                                             const uint64_t *__restrict__ pay_in,
                                                             uint64_t *__restrict__ pay_out,
@@ -473,40 +470,10 @@ __global__ void __launch_bounds__(256) pacc_exchange_kernel(PlanAcc P, const uin
                            cap_words - max(P.pay_send[m], P.pay_recv[m]));
     const uint64_t *s = pay_in + P.pay_send[m];
     uint64_t *d = pay_out + P.pay_recv[m];
-    for (int64_t i = threadIdx.x; i < nw; i += blockDim.x) d[i] = __ldg(s + i);
-    for (int64_t i = threadIdx.x; i < a.nb; i += blockDim.x) len_out[a.gr0 + i] = len_in[a.gb0 + i];
-}
-
-__global__ void __launch_bounds__(256) pacc_unpack_kernel(PlanAcc P, const uint64_t *__restrict__ payload, int64_t pwords,
-                                                          const uint16_t *__restrict__ lengths,
-                                                          const uint32_t *__restrict__ local,
-                                                          const uint64_t *__restrict__ tile_off,
-                                                          const uint64_t *__restrict__ total, uint8_t *__restrict__ slots)
-{
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;     // receive-order block
-    if (g >= P.G) return;
-    const int r = last_le(P.rgb0, nullptr, P.M, g, false);
-    const int m = P.rorder[r];
-    const AccMsg &a = P.msgs[m];
-    const uint64_t off = (uint64_t)P.pay_recv[m] * 64 +
-                         (goff(local, tile_off, P.G, total, g) - goff(local, tile_off, P.G, total, a.gr0));
-    const int L = min((int)lengths[g], kCutBits);
-    const int sh = (int)(off & 63);
-    const int64_t j0 = (int64_t)(off >> 6);
-    uint64_t *s = reinterpret_cast<uint64_t *>(slots + a.slot_recv) + (g - a.gr0) * kSlotWords;
-#pragma unroll
-    for (int i = 0; i < kSlotWords; i++) {
-        uint64_t v = 0;
-        const int rem = L - 64 * i;
-        if (rem > 0) {
-            const int64_t j = j0 + i;
-            const uint64_t lo = j < pwords ? __ldg(payload + j) : 0ull;
-            const uint64_t hi = (sh && j + 1 < pwords) ? __ldg(payload + j + 1) : 0ull;
-            v = sh ? (lo >> sh) | (hi << (64 - sh)) : lo;
-            if (rem < 64) v &= (1ull << rem) - 1ull;
-        }
-        s[i] = v;
-    }
+    const int64_t t = (int64_t)blockIdx.y * blockDim.x + threadIdx.x, step = (int64_t)gridDim.y * blockDim.x;
+#pragma unroll 4
+    for (int64_t i = t; i < nw; i += step) d[i] = __ldg(s + i);
+    for (int64_t i = t; i < a.nb; i += step) len_out[a.gr0 + i] = len_in[a.gb0 + i];
 }
 
 struct PlanAccWork {
@@ -516,8 +483,7 @@ struct PlanAccWork {
     size_t bytes;
 };
 
-int64_t plan_blocks(const zfpx_plan_s *p, std::vector<AccMsg> *msgs, std::vector<int32_t> *rorder,
-                    std::vector<int64_t> *rgb0)
+int64_t plan_blocks(const zfpx_plan_s *p, std::vector<AccMsg> *msgs, std::vector<int32_t> *rorder)
 {
     const size_t M = p->msgs.size();
     auto c4 = [](int64_t v) { return (v + 3) / 4; };
@@ -530,7 +496,6 @@ int64_t plan_blocks(const zfpx_plan_s *p, std::vector<AccMsg> *msgs, std::vector
     }
     if (!msgs) return G;
     const std::vector<int64_t> so = layout_offsets(p, 16, ZFPX_LAYOUT_SEND, nullptr);
-    const std::vector<int64_t> ro = layout_offsets(p, 16, ZFPX_LAYOUT_RECV, nullptr);
     std::vector<int32_t> ord(M);
     for (size_t i = 0; i < M; i++) ord[i] = (int32_t)i;
     std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) {
@@ -539,17 +504,15 @@ int64_t plan_blocks(const zfpx_plan_s *p, std::vector<AccMsg> *msgs, std::vector
     });
     msgs->assign(M, AccMsg{});
     rorder->assign(ord.begin(), ord.end());
-    rgb0->assign(M, 0);
     int64_t g = 0;
     for (size_t i = 0; i < M; i++) {
         (*msgs)[i].gb0 = g; (*msgs)[i].nb = nb[i];
-        (*msgs)[i].slot_send = so[i]; (*msgs)[i].slot_recv = ro[i];
+        (*msgs)[i].slot_send = so[i];
         g += nb[i];
     }
     g = 0;
     for (size_t r = 0; r < M; r++) {
         (*msgs)[ord[r]].gr0 = g;
-        (*rgb0)[r] = g;
         g += nb[ord[r]];
     }
     return G;
@@ -559,7 +522,7 @@ size_t plan_acc_bytes(const zfpx_plan_s *p, int64_t G)
 {
     const size_t M = p->msgs.size();
     return align256((size_t)buffer_bytes(p, 16)) + acc_work_bytes(G) - align256((size_t)G * 128) +
-           align256(M * sizeof(AccMsg)) + align256(M * 4) + 3 * align256(M * 8);
+           align256(M * sizeof(AccMsg)) + align256(M * 4) + 2 * align256(M * 8);
 }
 
 // Carves the scratch and uploads the message tables (pageable copies: the
@@ -568,8 +531,7 @@ int plan_acc_setup(const zfpx_plan_s *p, void *work, size_t work_bytes, cudaStre
 {
     std::vector<AccMsg> msgs;
     std::vector<int32_t> rorder;
-    std::vector<int64_t> rgb0;
-    const int64_t G = plan_blocks(p, &msgs, &rorder, &rgb0);
+    const int64_t G = plan_blocks(p, &msgs, &rorder);
     const size_t M = msgs.size();
     if (work_bytes < plan_acc_bytes(p, G)) return ZFPX_ESIZE;
     char *c = static_cast<char *>(work);
@@ -583,18 +545,14 @@ int plan_acc_setup(const zfpx_plan_s *p, void *work, size_t work_bytes, cudaStre
     w->scan.total = reinterpret_cast<uint64_t *>(c); c += 256;
     AccMsg *dm = reinterpret_cast<AccMsg *>(c); c += align256(M * sizeof(AccMsg));
     int32_t *dr = reinterpret_cast<int32_t *>(c); c += align256(M * 4);
-    int64_t *dg = reinterpret_cast<int64_t *>(c); c += align256(M * 8);
     w->P.pay_send = reinterpret_cast<int64_t *>(c); c += align256(M * 8);
     w->P.pay_recv = reinterpret_cast<int64_t *>(c); c += align256(M * 8);
-    w->P.msgs = dm; w->P.rorder = dr; w->P.rgb0 = dg; w->P.M = (int)M; w->P.G = G;
+    w->P.msgs = dm; w->P.rorder = dr; w->P.M = (int)M; w->P.G = G;
     if (M && (cudaMemcpyAsync(dm, msgs.data(), M * sizeof(AccMsg), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-              cudaMemcpyAsync(dr, rorder.data(), M * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-              cudaMemcpyAsync(dg, rgb0.data(), M * 8, cudaMemcpyHostToDevice, st) != cudaSuccess))
+              cudaMemcpyAsync(dr, rorder.data(), M * 4, cudaMemcpyHostToDevice, st) != cudaSuccess))
         return ZFPX_ECUDA;
     return ZFPX_OK;
 }
-
-unsigned grid256(int64_t n) { return (unsigned)std::max<int64_t>(1, (n + 255) / 256); }
 
 }  // namespace
 }  // namespace zfpx
@@ -603,13 +561,13 @@ extern "C" {
 
 size_t zfpx_plan_accuracy_blocks(zfpx_plan p)
 {
-    return p ? (size_t)plan_blocks(p, nullptr, nullptr, nullptr) : 0;
+    return p ? (size_t)plan_blocks(p, nullptr, nullptr) : 0;
 }
 
 size_t zfpx_plan_accuracy_workspace_bytes(zfpx_plan p)
 {
     if (!p || p->dims != 3) return 0;
-    return plan_acc_bytes(p, plan_blocks(p, nullptr, nullptr, nullptr));
+    return plan_acc_bytes(p, plan_blocks(p, nullptr, nullptr));
 }
 
 static int pack_compress_variable(zfpx_plan p, int minexp, int prec, const float *d_src, uint16_t *d_lengths,
@@ -619,7 +577,7 @@ static int pack_compress_variable(zfpx_plan p, int minexp, int prec, const float
     if (!p || !d_src || !d_lengths || !d_payload || !d_msg_words || !d_work || p->dims != 3) return ZFPX_EINVAL;
     if (!aligned(d_payload, 8) || !aligned(d_work, 256) || !aligned(d_lengths, 2) || !aligned(d_msg_words, 8))
         return ZFPX_EINVAL;
-    const int64_t G = plan_blocks(p, nullptr, nullptr, nullptr);
+    const int64_t G = plan_blocks(p, nullptr, nullptr);
     if (cap < (size_t)G * 128) return ZFPX_ESIZE;
     cudaStream_t st = (cudaStream_t)stream;
     PlanAccWork w;
@@ -627,18 +585,19 @@ static int pack_compress_variable(zfpx_plan p, int minexp, int prec, const float
     if (rc) return rc;
     if (G == 0)                                    // every message empty
         return cudaMemsetAsync(d_msg_words, 0, p->msgs.size() * 8, st) == cudaSuccess ? ZFPX_OK : ZFPX_ECUDA;
-    if ((rc = zfpx_pack_compress(p, 16, d_src, w.slots, (size_t)buffer_bytes(p, 16), ZFPX_LAYOUT_SEND, stream)))
+    LaunchGeom g{};
+    if ((rc = plan_geom(p, g))) return rc;
+    if ((rc = launch_encode_lengths(d_src, w.slots, g, codec_vec_ok(d_src, p->ss, p) ? 1 : 0,
+                                    AccEncode{d_lengths, w.P.msgs, minexp, prec}, st)))
         return rc;
-    pacc_lengths_kernel<<<grid256(G), 256, 0, st>>>(w.P, w.slots, minexp, prec, d_lengths);
+    if ((rc = acc_scan(w.scan, d_lengths, w.scan.total, st))) return rc;
+    // the sum of the word counts, where the payload ends, in the scratch after the total
+    uint64_t *used = w.scan.total + 1;
+    pacc_messages_kernel<<<1, kTile, 0, st>>>(w.P, w.scan.local, w.scan.tile_off, w.scan.total, d_msg_words, 1, used);
     count_launch();
-    if ((rc = check_launch()) || (rc = acc_scan(w.scan, d_lengths, w.scan.total, st))) return rc;
-    pacc_messages_kernel<<<1, 32, 0, st>>>(w.P, w.scan.local, w.scan.tile_off, w.scan.total, d_msg_words, 1);
-    count_launch();
-    if (cudaMemsetAsync(d_payload, 0, (size_t)G * 128, st) != cudaSuccess) return ZFPX_ECUDA;
-    pacc_pack_kernel<<<grid256(G), 256, 0, st>>>(w.P, w.slots, d_lengths, w.scan.local, w.scan.tile_off,
-                                                 w.scan.total, reinterpret_cast<unsigned long long *>(d_payload));
-    count_launch();
-    return check_launch();
+    if ((rc = check_launch())) return rc;
+    return acc_pack(AccList{w.P.msgs, w.P.pay_send, d_lengths, w.scan.local, w.scan.tile_off, w.P.M, G}, w.slots,
+                    d_payload, used, 0, st);
 }
 
 int zfpx_pack_compress_accuracy(zfpx_plan p, double tolerance, const float *d_src, uint16_t *d_lengths,
@@ -668,15 +627,18 @@ int zfpx_exchange_accuracy(zfpx_plan p, const uint64_t *d_msg_words, const uint1
     if (!p || !d_msg_words || !d_len_send || !d_pay_send || !d_len_recv || !d_pay_recv || !d_work || p->dims != 3)
         return ZFPX_EINVAL;
     if (!aligned(d_pay_send, 8) || !aligned(d_pay_recv, 8) || !aligned(d_work, 256)) return ZFPX_EINVAL;
-    const int64_t G = plan_blocks(p, nullptr, nullptr, nullptr);
+    const int64_t G = plan_blocks(p, nullptr, nullptr);
     if (cap < (size_t)G * 128) return ZFPX_ESIZE;
     cudaStream_t st = (cudaStream_t)stream;
     PlanAccWork w;
     int rc = plan_acc_setup(p, d_work, work_bytes, st, &w);
     if (rc || w.P.M == 0) return rc;
-    pacc_messages_kernel<<<1, 32, 0, st>>>(w.P, nullptr, nullptr, nullptr, const_cast<uint64_t *>(d_msg_words), 0);
+    pacc_messages_kernel<<<1, kTile, 0, st>>>(w.P, nullptr, nullptr, nullptr, const_cast<uint64_t *>(d_msg_words), 0,
+                                              nullptr);
     count_launch();
-    pacc_exchange_kernel<<<(unsigned)w.P.M, 256, 0, st>>>(w.P, d_msg_words,
+    // about eight CTAs per SM over all messages
+    const unsigned parts = (unsigned)std::max<int64_t>(1, std::min<int64_t>(64, (int64_t)num_sms() * 8 / w.P.M));
+    pacc_exchange_kernel<<<dim3((unsigned)w.P.M, parts), 256, 0, st>>>(w.P, d_msg_words,
                                                            reinterpret_cast<const uint64_t *>(d_pay_send),
                                                            reinterpret_cast<uint64_t *>(d_pay_recv), d_len_send,
                                                            d_len_recv, (int64_t)(cap / 8));
@@ -690,20 +652,21 @@ int zfpx_decompress_unpack_accuracy(zfpx_plan p, const uint64_t *d_msg_words, co
 {
     if (!p || !d_msg_words || !d_len_recv || !d_pay_recv || !d_dst || !d_work || p->dims != 3) return ZFPX_EINVAL;
     if (!aligned(d_pay_recv, 8) || !aligned(d_work, 256) || !aligned(d_len_recv, 2)) return ZFPX_EINVAL;
-    const int64_t G = plan_blocks(p, nullptr, nullptr, nullptr);
+    const int64_t G = plan_blocks(p, nullptr, nullptr);
     cudaStream_t st = (cudaStream_t)stream;
     PlanAccWork w;
     int rc = plan_acc_setup(p, d_work, work_bytes, st, &w);
     if (rc || G == 0) return rc;
-    pacc_messages_kernel<<<1, 32, 0, st>>>(w.P, nullptr, nullptr, nullptr, const_cast<uint64_t *>(d_msg_words), 0);
+    pacc_messages_kernel<<<1, kTile, 0, st>>>(w.P, nullptr, nullptr, nullptr, const_cast<uint64_t *>(d_msg_words), 0,
+                                              nullptr);
     count_launch();
     if ((rc = acc_scan(w.scan, d_len_recv, w.scan.total, st))) return rc;
-    pacc_unpack_kernel<<<grid256(G), 256, 0, st>>>(w.P, reinterpret_cast<const uint64_t *>(d_pay_recv),
-                                                   (int64_t)(len / 8), d_len_recv, w.scan.local, w.scan.tile_off,
-                                                   w.scan.total, w.slots);
-    count_launch();
-    if ((rc = check_launch())) return rc;
-    return zfpx_decompress_unpack(p, 16, w.slots, (size_t)buffer_bytes(p, 16), d_dst, ZFPX_LAYOUT_RECV, stream);
+    LaunchGeom g{};
+    if ((rc = plan_geom(p, g))) return rc;
+    return launch_decode_payload(d_dst, g, codec_vec_ok(d_dst, p->ds, p) ? 1 : 0,
+                                 AccDecode{reinterpret_cast<const uint64_t *>(d_pay_recv), (int64_t)(len / 8), d_len_recv,
+                                           w.scan.local, w.scan.tile_off, w.P.msgs, w.P.pay_recv},
+                                 st);
 }
 
 }  // extern "C"

@@ -103,9 +103,10 @@ struct UnitRange {
 // so full rows move as 16-byte loads and stores.  Otherwise a separate
 // instantiation reads and writes the rows of x-complete blocks as four scalar
 // accesses each, unrolled, keeping the vector kernel's code as it is.
-template <int RATE, bool VEC>
+// LEN: the variable-rate modes, which also want every block's bit count (acc).
+template <int RATE, bool VEC, bool LEN>
 __global__ void __launch_bounds__(32 * kEnc3Warps<RATE>, kEnc3MinBlocks<RATE, VEC>)
-encode3_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchGeom g, int layout)
+encode3_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchGeom g, int layout, AccEncode acc)
 {
     __shared__ enc3::Shared<RATE> sh[kEnc3Warps<RATE>];
     __shared__ enc3::Expand expand;
@@ -177,16 +178,73 @@ encode3_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchG
                 for (int r = 0; r < 64; r++) x[r] = t[r];
             }
         }
-        enc3::encode<RATE>(x, valid, v, lane);
+        const int len = enc3::encode<RATE, LEN>(x, valid, v, lane, enc3::PlaneCut{acc.minexp, acc.prec});
+        if (LEN && valid) acc.lengths[(acc.msgs ? acc.msgs[walk.mi].gb0 : 0) + b0 + lane] = (uint16_t)len;
         __syncwarp();
         enc3::store_stream<RATE>(v, lane, valid, out + boff + (b0 + lane) * RATE * 8);
         __syncwarp();
     }
 }
 
-template <int RATE, bool VEC>
+// Cuts a unit's nact blocks, from block b0 of message mi on, out of the payload
+// into the lanes' tile columns: 1024 bits each, those past a block's length 0.
+__device__ __forceinline__ void load_payload(const AccDecode &acc, int mi, int64_t b0, int nact, int lane,
+                                             uint32_t *t32, uint64_t *stage)
+{
+    const int64_t gr0 = acc.msgs ? acc.msgs[mi].gr0 : 0;
+    const int64_t gl = gr0 + b0 + (lane < nact ? lane : nact - 1);
+    auto bit = [&](int64_t q) { return acc.tile_off[q / kAccTile] + acc.local[q]; };
+    const uint64_t off = (acc.pay ? (uint64_t)acc.pay[mi] * 64 : 0ull) + (bit(gl) - bit(gr0));
+    const int L = min((int)acc.lengths[gl], 1024);
+    const int64_t j0 = (int64_t)(__shfl_sync(0xffffffffu, off, 0) >> 6);
+    const int64_t j1 = (int64_t)(__shfl_sync(0xffffffffu, off + (uint64_t)L + 63, nact - 1) >> 6);
+    if (j1 - j0 > 32 * 16 + 1) {                                 // lengths above 1024 bits: not the encoder's
+        if (lane < nact) {
+            auto word = [&](int64_t j) { return j < acc.pwords ? __ldg(acc.payload + j) : 0ull; };
+#pragma unroll 1
+            for (int i = 0; i < 16; i++) {
+                const int64_t j = (int64_t)(off >> 6) + i;
+                const int sh = (int)(off & 63), rem = L - 64 * i;
+                uint64_t v = rem > 0 ? (sh ? (word(j) >> sh) | (word(j + 1) << (64 - sh)) : word(j)) : 0ull;
+                if (rem > 0 && rem < 64) v &= (1ull << rem) - 1ull;
+                t32[(2 * i) * 32 + lane] = (uint32_t)v;
+                t32[(2 * i + 1) * 32 + lane] = (uint32_t)(v >> 32);
+            }
+        }
+        return;
+    }
+    const int nw = (int)(j1 - j0);
+    for (int i = lane; i <= nw; i += 32) {                       // one word more, for the last funnel
+        const int64_t j = j0 + i;
+        stage[i] = i < nw && j < acc.pwords ? __ldg(acc.payload + j) : 0ull;
+    }
+    __syncwarp();
+    const uint32_t *s32 = reinterpret_cast<const uint32_t *>(stage);
+    const int p = (int)(off - (uint64_t)j0 * 64);
+    const int w = p >> 5, sh = p & 31;
+    uint32_t a = s32[w];
+#pragma unroll
+    for (int i = 0; i < 32; i++) {
+        const int rem = L - 32 * i;
+        uint32_t v = 0;
+        if (rem > 0) {
+            const uint32_t b = s32[w + i + 1];
+            v = __funnelshift_r(a, b, sh);
+            if (rem < 32) v &= (1u << rem) - 1u;
+            a = b;
+        }
+        t32[i * 32 + lane] = v;
+    }
+    __syncwarp();                                                // the planes go over the staged words next
+}
+
+// PAY: the variable-rate modes, whose blocks lie back to back in a payload at
+// the bit offsets that the scan of their lengths gives (acc); a unit's bits are
+// one run of words, copied to shared memory (the planes' space, not yet in
+// use) in whole and cut into the lanes' columns from there.
+template <int RATE, bool VEC, bool PAY>
 __global__ void __launch_bounds__(32 * kDec3Warps<RATE>, kDec3MinBlocks<RATE>)
-decode3_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchGeom g, int layout)
+decode3_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchGeom g, int layout, AccDecode acc)
 {
     __shared__ uint32_t stile[kDec3Warps<RATE>][(2 * RATE + kTileZeroRows<RATE>) * 32];
     __shared__ uint64_t splanes[kDec3Warps<RATE>][32 * 32];
@@ -208,17 +266,20 @@ decode3_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchG
         const int nx = m.nx, ny = m.ny, nz = m.nz, bxn = m.bx, byn = m.by;
         const int64_t b0 = (c - unit0) * 32;
         const int nact = (int)min((int64_t)32, nblocks - b0);
+        if (PAY) load_payload(acc, walk.mi, b0, nact, lane, t32, splanes[wid]);
         if (lane < nact) {
             const int b = (int)b0 + lane;
-            // this lane's block: RATE / 2 16-byte loads into its own tile column
-            const uint4 *src4 = reinterpret_cast<const uint4 *>(in + boff) + (int64_t)b * (RATE / 2);
+            if (!PAY) {
+                // this lane's block: RATE / 2 16-byte loads into its own tile column
+                const uint4 *src4 = reinterpret_cast<const uint4 *>(in + boff) + (int64_t)b * (RATE / 2);
 #pragma unroll
-            for (int i = 0; i < RATE / 2; i++) {
-                const uint4 v = __ldg(src4 + i);
-                t32[(4 * i) * 32 + lane] = v.x;
-                t32[(4 * i + 1) * 32 + lane] = v.y;
-                t32[(4 * i + 2) * 32 + lane] = v.z;
-                t32[(4 * i + 3) * 32 + lane] = v.w;
+                for (int i = 0; i < RATE / 2; i++) {
+                    const uint4 v = __ldg(src4 + i);
+                    t32[(4 * i) * 32 + lane] = v.x;
+                    t32[(4 * i + 1) * 32 + lane] = v.y;
+                    t32[(4 * i + 2) * 32 + lane] = v.z;
+                    t32[(4 * i + 3) * 32 + lane] = v.w;
+                }
             }
             const int t = (int)divu((uint32_t)b, m.bxm, m.bxl), bxi = b - t * bxn;
             const int bzi = (int)divu((uint32_t)t, m.bym, m.byl), byi = t - bzi * byn;
@@ -540,9 +601,9 @@ constexpr int kFewUnits = 8;
 
 // One launch of a 3-D codec kernel (either alignment instantiation): one
 // warp per upw consecutive units.
-template <class In, class Out>
-void launch3(void (*kernel)(In, Out, LaunchGeom, int), int warps, int encode, int rate, LaunchGeom g,
-             cudaStream_t st, In in, Out out, int layout)
+template <class In, class Out, class Acc>
+void launch3(void (*kernel)(In, Out, LaunchGeom, int, Acc), int warps, int encode, int rate, LaunchGeom g,
+             cudaStream_t st, In in, Out out, int layout, const Acc &acc = Acc{})
 {
     g.upw = g_upw[encode ? 1 : 0][rate == 16 ? 1 : 0].load(std::memory_order_relaxed);
     if (g.upw <= 0) {
@@ -551,7 +612,7 @@ void launch3(void (*kernel)(In, Out, LaunchGeom, int), int warps, int encode, in
     }
     const int64_t per_cta = (int64_t)g.upw * warps;
     const int64_t grid = (g.nunits + per_cta - 1) / per_cta;
-    kernel<<<(unsigned)grid, 32 * warps, 0, st>>>(in, out, g, layout);
+    kernel<<<(unsigned)grid, 32 * warps, 0, st>>>(in, out, g, layout, acc);
 }
 
 // vec: rows start on 16 bytes wherever a block starts (x0 multiple of 4).
@@ -574,10 +635,10 @@ int launch_encode(int dims, int rate, const float *src, uint8_t *out, const Laun
     if (g.nunits == 0) return ZFPX_OK;
     if (dims == 3) {
         if (rate == 8)
-            launch3(vec ? encode3_kernel<8, true> : encode3_kernel<8, false>, kEnc3Warps<8>, 1, 8, g, st, src, out,
+            launch3(vec ? encode3_kernel<8, true, false> : encode3_kernel<8, false, false>, kEnc3Warps<8>, 1, 8, g, st, src, out,
                     layout);
         else
-            launch3(vec ? encode3_kernel<16, true> : encode3_kernel<16, false>, kEnc3Warps<16>, 1, 16, g, st, src, out,
+            launch3(vec ? encode3_kernel<16, true, false> : encode3_kernel<16, false, false>, kEnc3Warps<16>, 1, 16, g, st, src, out,
                     layout);
     } else if (dims == 2) {
         if (rate == 8) encode2_kernel<8><<<grid_for(encode2_kernel<8>, g.nunits), kThreads, 0, st>>>(src, out, g, layout, vec);
@@ -596,10 +657,10 @@ int launch_decode(int dims, int rate, const uint8_t *in, float *dst, const Launc
     if (g.nunits == 0) return ZFPX_OK;
     if (dims == 3) {
         if (rate == 8)
-            launch3(vec ? decode3_kernel<8, true> : decode3_kernel<8, false>, kDec3Warps<8>, 0, 8, g, st, in, dst,
+            launch3(vec ? decode3_kernel<8, true, false> : decode3_kernel<8, false, false>, kDec3Warps<8>, 0, 8, g, st, in, dst,
                     layout);
         else
-            launch3(vec ? decode3_kernel<16, true> : decode3_kernel<16, false>, kDec3Warps<16>, 0, 16, g, st, in, dst,
+            launch3(vec ? decode3_kernel<16, true, false> : decode3_kernel<16, false, false>, kDec3Warps<16>, 0, 16, g, st, in, dst,
                     layout);
     } else if (dims == 2) {
         if (rate == 8) decode2_kernel<8><<<grid_for(decode2_kernel<8>, g.nunits), kThreads, 0, st>>>(in, dst, g, layout, vec);
@@ -608,6 +669,25 @@ int launch_decode(int dims, int rate, const uint8_t *in, float *dst, const Launc
         if (rate == 8) decode1_kernel<8><<<grid_for(decode1_kernel<8>, g.nunits), kThreads, 0, st>>>(in, dst, g, layout, vec);
         else decode1_kernel<16><<<grid_for(decode1_kernel<16>, g.nunits), kThreads, 0, st>>>(in, dst, g, layout, vec);
     }
+    count_launch();
+    return check_launch();
+}
+
+int launch_encode_lengths(const float *src, uint8_t *slots, const LaunchGeom &g, int vec, const AccEncode &a,
+                          cudaStream_t st)
+{
+    if (g.nunits == 0) return ZFPX_OK;
+    launch3(vec ? encode3_kernel<16, true, true> : encode3_kernel<16, false, true>, kEnc3Warps<16>, 1, 16, g, st, src,
+            slots, (int)ZFPX_LAYOUT_SEND, a);
+    count_launch();
+    return check_launch();
+}
+
+int launch_decode_payload(float *dst, const LaunchGeom &g, int vec, const AccDecode &a, cudaStream_t st)
+{
+    if (g.nunits == 0) return ZFPX_OK;
+    launch3(vec ? decode3_kernel<16, true, true> : decode3_kernel<16, false, true>, kDec3Warps<16>, 0, 16, g, st,
+            (const uint8_t *)nullptr, dst, (int)ZFPX_LAYOUT_RECV, a);
     count_launch();
     return check_launch();
 }
@@ -690,6 +770,7 @@ namespace zfpx {
 namespace {
 std::mutex g_raw_mu;
 std::map<std::tuple<int, int, int64_t, int64_t, int64_t, int64_t, int64_t, int64_t>, zfpx_plan> g_raw_plans;
+}  // namespace
 
 int raw_plan(int dims, const int64_t n[3], const int64_t s[3], zfpx_plan *out)
 {
@@ -710,7 +791,6 @@ int raw_plan(int dims, const int64_t n[3], const int64_t s[3], zfpx_plan *out)
     g_raw_plans[key] = *out;
     return ZFPX_OK;
 }
-}  // namespace
 }  // namespace zfpx
 
 extern "C" {

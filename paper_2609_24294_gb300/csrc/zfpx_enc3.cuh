@@ -105,6 +105,18 @@ __device__ __forceinline__ void load_expand(Expand &tab)
 }
 __device__ __forceinline__ void wait_expand() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Lowest bit plane a block of exponent e_max keeps in the variable-rate modes:
+// the accuracy rule, or 32 - prec in precision mode (prec > 0).
+struct PlaneCut {
+    int minexp, prec;
+    __device__ __forceinline__ int kmin(int emax) const
+    {
+        if (prec > 0) return 32 - prec;
+        const int k = minexp - emax + 22;
+        return k < 0 ? 0 : (k > 32 ? 32 : k);
+    }
+};
+
 // One warp's shared memory: tile (kWords<RATE> * 32 words, or more), planes
 // (32 * 32), spos (32 * 32).
 struct View {
@@ -170,8 +182,11 @@ __device__ __forceinline__ void chunk(uint32_t &zl, uint32_t &zh, int &A, uint32
     A += 8 + popc32(c);
 }
 
-template <int RATE>
-__device__ __forceinline__ void encode(const float (&x)[64], bool valid, const View &sh, int lane)
+// LEN: also returns how many bits the block's planes 31 .. kmin take (at most
+// 64 RATE; 1 for a zero block), kmin by `cut` from the block's exponent; planes
+// below kmin may be left out of the stream.
+template <int RATE, bool LEN = false>
+__device__ __forceinline__ int encode(const float (&x)[64], bool valid, const View &sh, int lane, PlaneCut cut = {})
 {
     constexpr int kSeq[64] = ZFPX_SEQ3;
     constexpr int END = 64 * RATE;
@@ -245,8 +260,9 @@ __device__ __forceinline__ void encode(const float (&x)[64], bool valid, const V
     uint64_t lm = 0;                                   // low n bits
     const uint32_t tb = smem(tile), xb = smem(sh.expand), list0 = smem(planes + 31 * 32);
     uint32_t list = list0;                             // where the next entry goes
+    const int kmin = LEN ? cut.kmin(E - 126) : 0;
 #pragma unroll 1
-    for (int k = act ? 31 : -1; k >= 0; k--) {
+    for (int k = act ? 31 : -1; k >= kmin; k--) {
         if (k == kLow - 1) finish_low();
         const uint64_t X = planes[32 * k];
         const uint64_t Y = X & ~lm, V = X & lm;
@@ -280,10 +296,14 @@ __device__ __forceinline__ void encode(const float (&x)[64], bool valid, const V
     __syncwarp();                                      // the lanes go on together
     if (n1 == 65) pos -= 2;                            // coefficient 63's one is implied: no value or group bit
 
-    // ---- phase B
+    int len = 0;
+    if (LEN) len = act ? min(END, pos + (n1 == 65 ? 64 * max(0, kB - kmin + 1) : 0)) : 1;
+
+    // ---- phase B: planes kB, kB - 1, ... verbatim from bit pos
     if (n1 == 65 && pos < END) {
         const uint32_t s = (uint32_t)pos & 31u;
         const int w0 = pos >> 5;
+        // the lowest plane read here: kB - m for the m with w0 + 2 m < 2 RATE
         if (!low_done && kB - ((2 * RATE - w0 + 1) / 2 - 1) < kLow) finish_low();
         uint32_t prev = 0;
 #pragma unroll 1
@@ -321,6 +341,7 @@ __device__ __forceinline__ void encode(const float (&x)[64], bool valid, const V
             chunk(zl, zh, A, 0u, tb, xb, last);
         }
     }
+    return len;
 }
 
 // Copies this lane's 2 RATE stream words to dst (16-byte aligned, the

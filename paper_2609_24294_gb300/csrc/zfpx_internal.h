@@ -103,6 +103,39 @@ int64_t host_table(const zfpx_plan_s *p, int rate, UnitKind kind, const std::vec
 // Uploads a host table into a new device allocation (t->d_msgs, freed by the owner).
 int upload_table(const std::vector<MsgDev> &h, int64_t units, DevTable *t);
 
+// One message of a plan in the variable-rate modes (send-order index).
+struct AccMsg {
+    int64_t gb0;        // first block in the send-order block list (and lengths array)
+    int64_t gr0;        // first block in the receive-order block list
+    int64_t nb;         // blocks
+    int64_t slot_send;  // byte offset of its rate-16 slots in the send layout
+};
+// Where the variable-rate kernels find a table's messages; a NULL array stands
+// for one message that starts at 0.
+struct AccEncode {
+    uint16_t *lengths;        // bits per block, send order
+    const AccMsg *msgs;
+    int minexp, prec;         // the plane cut (prec > 0: precision mode)
+};
+struct AccDecode {
+    const uint64_t *payload;  // 64-bit words
+    int64_t pwords;
+    const uint16_t *lengths;  // receive order
+    const uint32_t *local;    // exclusive scan of the lengths: tile_off[g / kAccTile] + local[g]
+    const uint64_t *tile_off;
+    const AccMsg *msgs;
+    const int64_t *pay;       // first payload word of each message (send-order index)
+};
+constexpr int kAccTile = 1024;               // blocks per scan tile
+
+// The rate-16 3-D codec of the variable-rate modes over a table: encode into
+// 128-byte slots with every block's bit count, decode straight from the payload.
+int launch_encode_lengths(const float *src, uint8_t *slots, const LaunchGeom &g, int vec, const AccEncode &a,
+                          cudaStream_t st);
+int launch_decode_payload(float *dst, const LaunchGeom &g, int vec, const AccDecode &a, cudaStream_t st);
+// The one-message plan of a raw array (cached by shape).
+int raw_plan(int dims, const int64_t n[3], const int64_t s[3], zfpx_plan *out);
+
 // Kernel launchers over a table (geometry g: table, units, view strides).
 // vec: every row the kernel touches starts on 16 bytes.
 int launch_encode(int dims, int rate, const float *src, uint8_t *out, const LaunchGeom &g, int layout, int vec,

@@ -69,3 +69,58 @@ def test_default_units_per_warp_either_side_of_the_rule(rate):
                 z.zfpx_set_units_per_warp(0, rate, 0)
         for s, d in outs[1:]:
             assert torch.equal(s, outs[0][0]) and torch.equal(d, outs[0][1])
+
+
+# payloads whose words hold many blocks (1 and 9 bits each), end inside a word
+# and in the middle of a warp's 32 blocks, blocks cut at 1024 bits beside zero
+# blocks, and messages of one block: the payload written word by word against the
+# oracle's bit string, and the tail zeroed
+@pytest.mark.parametrize("blocks", [1, 31, 32, 33, 130, 1025])
+@pytest.mark.parametrize("kind", ["tiny", "mixed", "full"])
+def test_variable_rate_payload_words(blocks, kind):
+    r = np.random.default_rng(blocks)
+    x = r.standard_normal((4, 4, 4 * blocks)).astype(np.float32)
+    keep = {"tiny": r.random(blocks) < 0.02, "mixed": r.random(blocks) < 0.5, "full": np.ones(blocks, bool)}[kind]
+    x *= np.repeat(np.where(keep, 1.0, np.where(r.random(blocks) < 0.5, 0.0, 1e-6)), 4).astype(np.float32)
+    tol = 1e-9 if kind == "full" else 1e-2
+    n = (4 * blocks, 4, 4)
+    xd = torch.from_numpy(x).cuda()
+    lens = torch.zeros(blocks, dtype=torch.int16, device="cuda")
+    pay = torch.full((z.zfpx_accuracy_max_payload_bytes(n),), 255, dtype=torch.uint8, device="cuda")
+    total = torch.zeros(1, dtype=torch.int64, device="cuda")
+    work = torch.zeros(z.zfpx_accuracy_workspace_bytes(n), dtype=torch.uint8, device="cuda")
+    z.zfpx_encode_accuracy(xd, tol, lens, pay, total, work)
+    rl, rp, rt = oc.encode_accuracy(x, tol)
+    assert np.array_equal(lens.cpu().numpy().view(np.uint16), rl) and int(total) == rt
+    got = pay.cpu().numpy()                            # the oracle's payload ends with its last byte
+    assert np.array_equal(got[:len(rp)], rp) and not got[len(rp):].any()
+    d = torch.full(x.shape, float("nan"), device="cuda")
+    z.zfpx_decode_accuracy(lens, pay, d, work)
+    rd = np.empty_like(x)
+    oc.decode_accuracy(rl, rp, rd)
+    assert np.array_equal(d.cpu().numpy().view(np.uint32), rd.view(np.uint32))
+
+
+@pytest.mark.parametrize("shape,pr,pc", [((13, 9, 7), 3, 2), ((40, 24, 16), 10, 4), ((9, 5, 2), 2, 3)])
+def test_variable_rate_messages_of_few_blocks(shape, pr, pc):
+    x = np.random.default_rng(7).standard_normal(shape[::-1]).astype(np.float32)
+    x[:, :, : shape[0] // 2] = 0.0
+    xd = torch.from_numpy(x).cuda()
+    plan = z.Plan.for_fields(xd, pr, pc, 0, 3)
+    acc = z.AccuracyTransposition(plan)
+    acc.pay_send.fill_(255)
+    out = torch.full_like(xd, float("nan"))
+    acc.compress(xd, 1e-3)
+    acc.exchange()
+    acc.decompress(out)
+    for i, (ranks, (x0, nx, y0, ny, z0, nz)) in enumerate(plan.messages()):
+        box = x[z0:z0 + nz, y0:y0 + ny, x0:x0 + nx]
+        bits = 0
+        if box.size:
+            rl, rp, bits = oc.encode_accuracy(np.ascontiguousarray(box), 1e-3)
+            rd = np.empty(box.shape, dtype=np.float32)
+            oc.decode_accuracy(rl, rp, rd)
+            got = out[z0:z0 + nz, y0:y0 + ny, x0:x0 + nx].cpu().numpy()
+            assert np.array_equal(got.view(np.uint32), rd.view(np.uint32))
+        assert int(acc.words[i]) == (bits + 63) // 64
+    assert not acc.pay_send[8 * int(acc.words.sum()):].any()
