@@ -54,12 +54,20 @@ template <int RATE>
 constexpr int kDec3MinBlocks = RATE == 8 ? 5 : 6;
 
 // ----------------------------------------------------------------- message walk
+// The last message whose units start at or before u, by the whole warp: every
+// round the lanes look at 32 messages spread over the range that is left, so 512
+// messages take two rounds of loads where halving takes nine, each waiting for
+// the one before at the start of every warp.
 __device__ __forceinline__ int find_msg(const MsgDev *msgs, int nmsg, int64_t u)
 {
-    int lo = 0, hi = nmsg - 1;               // last message with unit0 <= u
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (msgs[mid].unit0 <= u) lo = mid; else hi = mid - 1;
+    const int lane = threadIdx.x & 31;
+    int lo = 0, n = nmsg;
+    while (n > 1) {
+        const int step = (n + 31) >> 5;
+        const bool before = lane * step < n && msgs[lo + lane * step].unit0 <= u;
+        const int k = __popc(__ballot_sync(0xffffffffu, before)) - 1;    // msgs[lo] starts at or before u
+        lo += k * step;
+        n = min(step, n - k * step);
     }
     return lo;
 }
@@ -590,14 +598,14 @@ bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 // resident warp.  A warp's units run one after the other, so where a launch is
 // little more than one wave of warps a second unit doubles its time (a 64 x 32
 // x 8 field: 18.4 us a kernel with two, 10.2 with one; 233 x 117 x 137: 36.9 /
-// 36.9 us against 26.6 / 28.7 compress / decompress), and one also ends a launch of
-// several waves more evenly (640 x 320 x 137, five waves: 69.6 / 77.8 against
-// 67.6 / 75.8); in long launches two save part of the per-CTA start-up
-// (twenty waves: 243 against 256 us).  The autotuner can override it; results
-// never depend on it.
+// 36.9 us against 26.6 / 26.6 compress / decompress), and one also ends a launch of a
+// few waves more evenly (640 x 320 x 137 over 4 x 4 ranks, five waves: 73.7 /
+// 75.8 against 71.7 / 73.7); in longer launches two halve the start-up of the
+// warps (message search, tables; eight waves: 158 / 166 us against 174 / 188).
+// The autotuner can override it; results never depend on it.
 std::atomic<int> g_upw[2][2] = {{{0}, {0}}, {{0}, {0}}};
 constexpr int kDefaultUpw = 2;
-constexpr int kFewUnits = 8;
+constexpr int kFewUnits = 6;
 
 // One launch of a 3-D codec kernel (either alignment instantiation): one
 // warp per upw consecutive units.

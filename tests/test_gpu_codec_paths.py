@@ -51,7 +51,7 @@ def test_units_at_the_edges(blocks, rate):
 @pytest.mark.parametrize("rate", [8, 16])
 def test_default_units_per_warp_either_side_of_the_rule(rate):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    for per_sm in (8 * 15, 8 * 21):                    # fewer and more than eight units per resident warp
+    for per_sm in (6 * 15, 6 * 21):                    # fewer and more than six units per resident warp
         y = (sms * per_sm * 32 + 63) // 64             # 64 blocks a row of blocks
         x = torch.randn((4, 4 * y, 256), device="cuda", generator=torch.Generator("cuda").manual_seed(per_sm))
         outs = []
@@ -124,3 +124,28 @@ def test_variable_rate_messages_of_few_blocks(shape, pr, pc):
             assert np.array_equal(got.view(np.uint32), rd.view(np.uint32))
         assert int(acc.words[i]) == (bits + 63) // 64
     assert not acc.pay_send[8 * int(acc.words.sum()):].any()
+
+
+# message counts around the powers of the 32-way message search, messages of one
+# block each, and empty ones (more ranks than values)
+@pytest.mark.parametrize("pr,pc", [(1, 1), (1, 5), (2, 4), (1, 6), (11, 3), (8, 12), (31, 6)])
+@pytest.mark.parametrize("dims", [1, 2, 3])
+def test_message_search(pr, pc, dims):
+    x = np.random.default_rng(pr * pc).standard_normal((5, 33, 44)).astype(np.float32)
+    xd = torch.from_numpy(x).cuda()
+    plan = z.Plan.for_fields(xd, pr, pc, 0, dims)
+    s = torch.zeros(max(1, plan.buffer_bytes(8)), dtype=torch.uint8, device="cuda")
+    d = torch.full_like(xd, float("nan"))
+    z.zfpx_pack_compress(plan, 8, xd, s)
+    z.zfpx_decompress_unpack(plan, 8, s, d, layout=z.LAYOUT_SEND)
+    got, vals = s.cpu().numpy(), d.cpu().numpy()
+    for (src, dst, _, _), (x0, nx, y0, ny, z0, nz) in plan.messages():
+        box = np.ascontiguousarray(x[z0:z0 + nz, y0:y0 + ny, x0:x0 + nx])
+        if not box.size:
+            continue
+        ref = oc.encode_array(dims, 8, box)
+        off = plan.message_offset(8, z.LAYOUT_SEND, src, dst)
+        assert np.array_equal(got[off:off + len(ref)], ref)
+        rd = np.empty_like(box)
+        oc.decode_array(dims, 8, ref, rd)
+        assert np.array_equal(vals[z0:z0 + nz, y0:y0 + ny, x0:x0 + nx].view(np.uint32), rd.view(np.uint32))
