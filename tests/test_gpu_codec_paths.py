@@ -149,3 +149,28 @@ def test_message_search(pr, pc, dims):
         rd = np.empty_like(box)
         oc.decode_array(dims, 8, ref, rd)
         assert np.array_equal(vals[z0:z0 + nz, y0:y0 + ny, x0:x0 + nx].view(np.uint32), rd.view(np.uint32))
+
+
+# parts that close in the first, second and third 32-bit window, run through a
+# whole window, end in its last bit or at the implied coefficient: streams of long
+# runs of ones and zeros
+@pytest.mark.parametrize("rate", [8, 16])
+def test_streams_of_long_runs(rate):
+    r = np.random.default_rng(rate)
+    n = (4 * 512, 4, 4)
+    bits = []
+    for _ in range(512):
+        b = np.zeros(64 * rate, np.uint8)
+        p, v = 9, 1
+        while p < len(b):
+            q = p + int(r.choice([1, 2, 3, 7, 31, 32, 33, 63, 64, 65]))
+            b[p:q] = v
+            p, v = q, 1 - v
+        b[:9] = 1, *r.integers(0, 2, 8)
+        bits.append(b)
+    s = np.packbits(np.concatenate(bits), bitorder="little")
+    d = torch.full((4, 4, n[0]), float("nan"), device="cuda")
+    z.zfpx_decode(3, rate, torch.from_numpy(s).cuda(), d)
+    rd = np.empty((4, 4, n[0]), dtype=np.float32)
+    oc.decode_array(3, rate, s, rd)
+    assert np.array_equal(d.cpu().numpy().view(np.uint32), rd.view(np.uint32))
