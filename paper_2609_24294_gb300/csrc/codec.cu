@@ -27,6 +27,7 @@
 #include "zfpx_block.cuh"
 #include "zfpx_smem.cuh"
 #include "zfpx_enc3.cuh"
+#include "zfpx_enc2.cuh"
 
 namespace zfpx {
 namespace {
@@ -457,63 +458,61 @@ decode1_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchG
 // ================================================================= 2-D kernels
 // Blocks of 4 x 4 values over axes 0 and 1 of one level; one lane per block,
 // a warp takes 32 consecutive blocks of one message (units split statically
-// over the warps).  A block's stream is RATE / 4 64-bit words, staged in a
-// swizzled [word][lane] shared tile and moved with coalesced 8-byte accesses.
+// over the warps).  Each lane moves its own stream with 16-byte accesses.
 template <int RATE>
 __global__ void __launch_bounds__(kThreads)
 encode2_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchGeom g, int layout, int vec)
 {
-    constexpr int NW = RATE / 4;
-    __shared__ uint64_t smem[kWarps][(NW + 2) * 32];
-    __shared__ uint32_t splanes[kWarps][32 * 32];
+    __shared__ enc2::Shared<RATE> sh[kWarps];
+    __shared__ enc3::Expand expand;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint64_t *wsm = smem[wid];
-    SmemPlanes16 pl{splanes[wid], lane};
+    const enc2::View v = sh[wid].view(expand);
+    enc3::load_expand(expand);
     const int64_t W = (int64_t)gridDim.x * kWarps;
     const int64_t gw = (int64_t)blockIdx.x * kWarps + wid;
     int64_t c = gw * g.nunits / W;
     const int64_t c1 = (gw + 1) * g.nunits / W;
-    if (c >= c1) return;
+#pragma unroll
+    for (int w = 0; w < enc2::kWords<RATE>; w++) v.tile[32 * w + lane] = 0u;
     MsgWalk walk;
-    walk.start(g.msgs, g.nmsg, c);
+    if (c < c1) walk.start(g.msgs, g.nmsg, c);
+    enc3::wait_expand();
+    __syncthreads();
     for (; c < c1; c++) {
         walk.advance(c);
         const MsgDev &m = g.msgs[walk.mi];
         const int64_t b0 = (c - m.unit0) * 32;
         const int nact = (int)min((int64_t)32, m.nblocks - b0);
+        const bool valid = lane < nact;
         const int64_t boff = layout ? m.off[1] : m.off[0];
-        if (lane < nact) {
-            const int nx = m.nx, ny = m.ny, bxn = m.bx, byn = m.by;
-            const int b = (int)b0 + lane;
-            const int t = (int)divu((uint32_t)b, m.bxm, m.bxl), bxi = b - t * bxn;
-            const int z = (int)divu((uint32_t)t, m.bym, m.byl), byi = t - z * byn;
-            const int x0 = 4 * bxi, y0 = 4 * byi;
-            const float *base = src + m.src_off + (int64_t)z * g.ss[2];
-            float x[16];
+        float x[16];
+        {
+            // lanes past the unit's last block load that block and code nothing
+            const int nx = m.nx, ny = m.ny;
+            const uint32_t b = (uint32_t)b0 + (uint32_t)(valid ? lane : nact - 1);
+            const uint32_t t = divu(b, m.bxm, m.bxl), z = divu(t, m.bym, m.byl);
+            const int x0 = 4 * (int)(b - t * (uint32_t)m.bx), y0 = 4 * (int)(t - z * (uint32_t)m.by);
+            const float *base = src + m.src_off + (int64_t)z * g.ss[2] + (int64_t)y0 * g.ss[1];
             if (vec && x0 + 4 <= nx) {
                 // four 16-byte row loads (rows past the box repeat its last row)
+                const float *row = base + x0;
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
-                    const float4 f = __ldg(reinterpret_cast<const float4 *>(
-                        base + (int64_t)min(y0 + j, ny - 1) * g.ss[1] + x0));
+                    const float4 f = __ldg(reinterpret_cast<const float4 *>(row));
                     x[4 * j] = f.x; x[4 * j + 1] = f.y; x[4 * j + 2] = f.z; x[4 * j + 3] = f.w;
+                    if (y0 + j + 1 < ny) row += g.ss[1];
                 }
             } else {
 #pragma unroll
                 for (int r = 0; r < 16; r++) {
                     const int i = r & 3, j = r >> 2;
-                    x[r] = __ldg(base + (int64_t)min(y0 + j, ny - 1) * g.ss[1] + (int64_t)min(x0 + i, nx - 1) * g.ss[0]);
+                    x[r] = __ldg(base + (int64_t)min(j, ny - 1 - y0) * g.ss[1] + (int64_t)min(x0 + i, nx - 1) * g.ss[0]);
                 }
             }
-            SmemWriter<NW> wr{wsm, 0ull, 0, 0, lane};
-            encode_block2<RATE>(x, wr, pl);
         }
+        enc2::encode<RATE>(x, valid, v, lane);
         __syncwarp();
-        uint64_t *dst = reinterpret_cast<uint64_t *>(out + boff) + b0 * NW;
-        for (int idx = lane; idx < nact * NW; idx += 32) {
-            const int l = idx / NW, w = idx % NW;
-            dst[idx] = wsm[w * 32 + (l ^ w)];
-        }
+        enc2::store_stream<RATE>(v, lane, valid, out + boff + (b0 + lane) * (2 * RATE));
         __syncwarp();
     }
 }
@@ -522,16 +521,14 @@ template <int RATE>
 __global__ void __launch_bounds__(kThreads)
 decode2_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchGeom g, int layout, int vec)
 {
-    constexpr int NW = RATE / 4;              // 64-bit words per block
-    constexpr int ZR = 3;                     // zero rows after the stream
-    __shared__ uint32_t stile[kWarps][(2 * NW + ZR) * 32];
-    __shared__ uint32_t splanes[kWarps][32 * 32];
+    constexpr int NW = RATE / 2;              // 32-bit words per block
+    __shared__ uint32_t stile[kWarps][(NW + 1) * 32];
+    __shared__ uint32_t splanes[kWarps][16 * 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t *t32 = stile[wid];
     SmemPlanes16 pl{splanes[wid], lane};
     const StreamTile tile{t32, lane};
-#pragma unroll
-    for (int r = 0; r < ZR; r++) t32[(2 * NW + r) * 32 + lane] = 0u;
+    t32[NW * 32 + lane] = 0u;                 // a zero word after the stream
     const int64_t W = (int64_t)gridDim.x * kWarps;
     const int64_t gw = (int64_t)blockIdx.x * kWarps + wid;
     int64_t c = gw * g.nunits / W;
@@ -545,13 +542,13 @@ decode2_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchG
         const int64_t b0 = (c - m.unit0) * 32;
         const int nact = (int)min((int64_t)32, m.nblocks - b0);
         if (lane >= nact) continue;
-        const int nx = m.nx, ny = m.ny, bxn = m.bx, byn = m.by;
+        const int nx = m.nx, ny = m.ny;
         const int64_t boff = layout ? m.off[1] : m.off[0];
-        const int b = (int)b0 + lane;
-        // this lane's block: NW / 2 16-byte loads into its own tile column
-        const uint4 *src4 = reinterpret_cast<const uint4 *>(in + boff) + (int64_t)b * (NW / 2);
+        const uint32_t b = (uint32_t)b0 + lane;
+        // this lane's block: 16-byte loads into its own tile column
+        const uint4 *src4 = reinterpret_cast<const uint4 *>(in + boff) + (int64_t)b * (NW / 4);
 #pragma unroll
-        for (int i = 0; i < NW / 2; i++) {
+        for (int i = 0; i < NW / 4; i++) {
             const uint4 v = __ldg(src4 + i);
             t32[(4 * i) * 32 + lane] = v.x;
             t32[(4 * i + 1) * 32 + lane] = v.y;
@@ -560,22 +557,22 @@ decode2_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchG
         }
         float v[16];
         decode_block2_tile<RATE>(tile, v, pl);
-        const int t = (int)divu((uint32_t)b, m.bxm, m.bxl), bxi = b - t * bxn;
-        const int z = (int)divu((uint32_t)t, m.bym, m.byl), byi = t - z * byn;
-        const int x0 = 4 * bxi, y0 = 4 * byi;
-        float *base = dstf + m.dst_off + (int64_t)z * g.ds[2];
+        const uint32_t t = divu(b, m.bxm, m.bxl), z = divu(t, m.bym, m.byl);
+        const int x0 = 4 * (int)(b - t * (uint32_t)m.bx), y0 = 4 * (int)(t - z * (uint32_t)m.by);
+        float *base = dstf + m.dst_off + (int64_t)z * g.ds[2] + (int64_t)y0 * g.ds[1];
         if (vec && x0 + 4 <= nx) {
+            float *row = base + x0;
 #pragma unroll
-            for (int j = 0; j < 4; j++)
+            for (int j = 0; j < 4; j++) {
                 if (y0 + j < ny)
-                    *reinterpret_cast<float4 *>(base + (int64_t)(y0 + j) * g.ds[1] + x0) =
-                        make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    *reinterpret_cast<float4 *>(row) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                row += g.ds[1];
+            }
         } else {
 #pragma unroll
             for (int r = 0; r < 16; r++) {
                 const int i = r & 3, j = r >> 2;
-                if (x0 + i < nx && y0 + j < ny)
-                    base[(int64_t)(y0 + j) * g.ds[1] + (int64_t)(x0 + i) * g.ds[0]] = v[r];
+                if (x0 + i < nx && y0 + j < ny) base[(int64_t)j * g.ds[1] + (int64_t)(x0 + i) * g.ds[0]] = v[r];
             }
         }
     }

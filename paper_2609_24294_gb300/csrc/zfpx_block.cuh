@@ -927,109 +927,97 @@ ZFPX_HD void encode_block2(const float (&x)[16], Writer &wr, Planes &pl)
     if (cacc) wr.orw(cw, cacc);
 }
 
-// Reader over a stream tile: peek() = the 64 bits from the current position.
-template <class Tile>
-struct TileReader {
-    const Tile &t;
-    int pos;
-    ZFPX_HD uint64_t peek() const { return tile_peek(t, pos); }
-    ZFPX_HD void skip(int k) { pos += k; }
-};
+// Planes k and k + 16 of a 2-D block as the halves of one word.
+template <class Planes>
+ZFPX_HD uint32_t plane_pair(const Planes &pl, int k)
+{
+    return pl.load_half(k, 0) | (pl.load_half(k + 16, 0) << 16);
+}
+
+// The bit planes of 16 words as 16 pairs and back: afterwards bit i of the low
+// (high) half of w[k] is what bit k (k + 16) of w[i] was.
+ZFPX_HD void transpose16_pairs(uint32_t (&w)[32])
+{
+    tstage<8, 0, 16>(w);
+    tstage<4, 0, 16>(w);
+    tstage<2, 0, 16>(w);
+    tstage<1, 0, 16>(w);
+}
 
 // Decodes one 2-D block from this lane's stream tile (2 RATE / 4 words of 32
-// bits, then at least two zero words).  Planes below the last one the budget
-// reached stay zero.
+// bits, then at least one zero word).  With 16 coefficients a plane takes at most
+// 31 bits (n verbatim bits, the group bit, and a value and a group bit for
+// each of the rest but the implied last one), so one 32-bit window holds it.
+// Issue-bound; with 64-bit windows and 32-word transposes decompressing a 1280
+// x 640 x 37 field level by level over 4 x 4 ranks took 182 us at rate 8 and 201
+// at rate 16, now 127 and 139.
 template <int RATE, class Tile, class Planes>
 ZFPX_HD void decode_block2_tile(const Tile &tile, float (&x)[16], Planes &pl)
 {
     constexpr int kSeq[16] = ZFPX_SEQ2;
-    const uint64_t head = tile_peek(tile, 0);
-    if (!(head & 1ull)) {
+    constexpr int END = 16 * RATE;
+    const uint32_t head = tile_peek32(tile, 0);
+    if (!(head & 1u)) {
 #pragma unroll
         for (int i = 0; i < 16; i++) x[i] = 0.0f;
         return;
     }
     const int e = (int)((head >> 1) & 0xffu);
-    // Plane by plane from one 64-bit window: n verbatim bits, the first group
-    // bit, and a group-tested part of at most 16 - n value bits and 15 group
-    // bits, 48 bits in all.  The tile is zero past the budget, so a part the
-    // budget cuts reads on as zeros: no one and no closing 0 appear there,
-    // and only the implied one of coefficient 15 needs the check that its
-    // bits fit (the 3-D decoder's reading, with 16 coefficients).
-    constexpr int END = 16 * RATE;
-    int pos = 9, n = 0, kmin = 32;
+    // The tile is zero past the budget, so a part the budget cuts reads on as
+    // zeros: no one and no closing 0 appear there, and only the implied one of
+    // coefficient 15 needs the check that its bits fit (the 3-D decoder's
+    // reading, with 16 coefficients).
+    int pos = 9, n = 0, k = 31;
     uint32_t lm = 0;                                             // low n bits
+    bool cut = false;
 #pragma unroll 1
-    for (int k = 31; k >= 0 && pos < END; k--) {
-        kmin = k;
+    for (; k >= 0 && n < 16 && pos < END && !cut; k--) {
         const int rem = END - pos;
-        const uint64_t w = tile_peek(tile, pos);
-        if (n >= 16) {                                           // verbatim plane
-            pl.store_half(k, 0, (uint32_t)w & (rem < 16 ? (1u << rem) - 1u : 0xffffu));
-            pos += 16;
-            continue;
-        }
-        uint32_t X = (uint32_t)w & lm;
-        if (rem <= n) { pl.store_half(k, 0, (uint32_t)w & ((1u << rem) - 1u)); break; }   // cut in the verbatim bits
+        const uint32_t W = tile_peek32(tile, pos);
+        uint32_t X = W & lm;
         pos += n + 1;
-        if (!(w & (uint64_t)(lm + 1u))) { pl.store_half(k, 0, X); continue; }           // group empty
-        uint64_t term;
-        uint64_t V = group_values<uint64_t>(w >> (n + 1), term);
-        const uint64_t below = term ? (term & (0ull - term)) - 1ull : ~0ull;   // bits before the closing 0
-        const int T = popc64(below);
-        // the t-th one, at offset p, is coefficient n + p - t: take the ones
-        // lowest first, shifting the rest down by one after each
-        int t = 0;
-        uint64_t nw = 0;
-        V &= below;
-        while (V) {
-            const uint64_t b = V & (0ull - V);
-            nw |= b;
-            V = (V ^ b) >> 1;
-            t++;
-        }
-        // ones past coefficient 14 lie beyond a part that ends at the implied one
-        const uint64_t keep = (1ull << (15 - n)) - 1ull;
-        const bool over = (nw & ~keep) != 0ull;
-        if (over) {
+        if (rem > n && (W & (lm + 1u))) {                        // the group bit
+            uint32_t term;
+            const uint32_t val = group_values<uint32_t>(W >> (n + 1), term);
+            const uint32_t below = (term - 1u) & ~term;          // the bits before the closing 0 (all: none)
+            const uint32_t V = val & below;
+            uint32_t nw = drop_group_bits<uint32_t>(V);
+            // ones past coefficient 14 lie beyond a part that ends at the implied one
+            const uint32_t keep = (1u << (15 - n)) - 1u;
+            const bool over = (nw & ~keep) != 0u;
             nw &= keep;
-            t = popc64(nw);
+            X |= nw << n;
+            if (!over && term) {                                 // closed by a 0 below coefficient 15
+                const int T = popc32(below);
+                n += T - popc32(V) + 1;
+                lm = (1u << n) - 1u;
+                pos += T + 1;
+            } else {
+                const int E = 15 - n + popc32(nw);               // the part ends at the implied one
+                if (E > END - pos) {
+                    cut = true;
+                } else {
+                    X |= 0x8000u;
+                    n = 16;
+                }
+                pos += E;
+            }
         }
-        X |= (uint32_t)nw << n;
-        if (!over && term) {                                     // closed by a 0 below coefficient 15
-            pl.store_half(k, 0, X);
-            n += T - t + 1;
-            lm = (1u << n) - 1u;
-            pos += T + 1;
-            continue;
-        }
-        const int E = 15 - n + t;                                // the part ends at the implied one
-        if (E > END - pos) { pl.store_half(k, 0, X); break; }
-        pl.store_half(k, 0, X | 0x8000u);
-        pos += E;
-        n = 16;
-        lm = 0xffffu;
+        pl.store_half(k, 0, X);                                  // past the budget W and so X is 0
     }
-    // Planes below kmin are zero; when planes 0..15 are zero in every lane of
-    // the warp, the transpose stages below 16 skip them.
+    // every coefficient significant: the planes that the budget still holds, verbatim
+#pragma unroll 1
+    for (; k >= 0 && pos < END && !cut; k--, pos += 16) pl.store_half(k, 0, tile_peek32(tile, pos) & 0xffffu);
+#pragma unroll 1
+    for (; k >= 0; k--) pl.store_half(k, 0, 0u);
+    // u ^ 0xAA..A of the negabinary map as the complement of the odd planes
     uint32_t w[32];
-#ifdef __CUDA_ARCH__
-    const bool low_zero = __all_sync(__activemask(), kmin >= 16);
-#else
-    const bool low_zero = kmin >= 16;
-#endif
-    if (low_zero) {
 #pragma unroll
-        for (int k = 16; k < 32; k++) w[k] = k >= kmin ? pl.load_half(k, 0) : 0u;
-        transpose32_zero_low<16>(w);
-    } else {
-#pragma unroll
-        for (int k = 0; k < 32; k++) w[k] = k >= kmin ? pl.load_half(k, 0) : 0u;
-        transpose32(w);
-    }
+    for (int i = 0; i < 16; i++) w[i] = i & 1 ? ~plane_pair(pl, i) : plane_pair(pl, i);
+    transpose16_pairs(w);
     int32_t q[16];
 #pragma unroll
-    for (int t = 0; t < 16; t++) q[kSeq[t]] = from_negabinary(w[t]);
+    for (int t = 0; t < 16; t++) q[kSeq[t]] = (int32_t)(w[t] - 0xAAAAAAAAu);
     xform2_inv(q);
     if (e >= 31) {
         const float sc = dequant_scale(e);

@@ -7,49 +7,6 @@
 
 namespace zfpx {
 
-// Writer into this lane's column of a [word][lane] tile of RATE + 2 64-bit
-// words (RATE stream words, two slack words past the budget), XOR-swizzled (word w of lane l at w * 32 + (l ^ w)) so that both the
-// per-lane writes and the warp's coalesced copy-out spread over the banks.
-// put(bits, len): 1 <= len <= 64, bits < 2^len; zeros(len): len >= 0;
-// finish(): flush and zero-fill to RATE words; orw(i, v): OR v into word i
-// (only after finish()).
-template <int RATE>
-struct SmemWriter {
-    uint64_t *sm;
-    uint64_t acc;
-    int nb, w, lane;
-    __device__ __forceinline__ uint64_t &word(int i) const { return sm[i * 32 + (lane ^ i)]; }
-    __device__ __forceinline__ void put(uint64_t bits, int len)
-    {
-        acc |= bits << nb;
-        int t = nb + len;
-        if (t >= 64) {
-            word(w) = acc;
-            w++;
-            acc = nb ? (bits >> (64 - nb)) : 0ull;
-            t -= 64;
-        }
-        nb = t;
-    }
-    __device__ __forceinline__ void zeros(int len)
-    {
-        int t = nb + len;
-        while (t >= 64) {
-            word(w) = acc;
-            w++;
-            acc = 0ull;
-            t -= 64;
-        }
-        nb = t;
-    }
-    __device__ __forceinline__ void finish()
-    {
-        if (nb > 0) { word(w) = acc; w++; }
-        for (; w < RATE; w++) word(w) = 0ull;
-    }
-    __device__ __forceinline__ void orw(int i, uint64_t v) const { word(i) |= v; }
-};
-
 // Bit planes of one block in this lane's column of a [plane][lane] tile
 // (a warp touches 32 consecutive words: conflict-free).
 struct SmemPlanes {
@@ -68,14 +25,17 @@ struct SmemPlanes {
     }
 };
 
-// 32-bit bit planes (2-D blocks: 16 coefficients) in this lane's column of a
-// [plane][lane] tile; the same interface as the low half of SmemPlanes.
+// The 32 16-bit planes of a 2-D block in this lane's column of a [word][lane]
+// tile of 16 words: word k holds planes k and k + 16 as halves.
 struct SmemPlanes16 {
     uint32_t *sm;
     int lane;
-    __device__ __forceinline__ void store_half(int k, int, uint32_t v) { sm[k * 32 + lane] = v; }
-    __device__ __forceinline__ uint32_t load_half(int k, int) const { return sm[k * 32 + lane]; }
+    __device__ __forceinline__ void store_half(int k, int, uint32_t v)
+    {
+        reinterpret_cast<uint16_t *>(sm)[2 * ((k & 15) * 32 + lane) + (k >> 4)] = (uint16_t)v;
+    }
 };
+__device__ __forceinline__ uint32_t plane_pair(const SmemPlanes16 &pl, int k) { return pl.sm[k * 32 + pl.lane]; }
 
 // Stream tile of one warp: 32-bit words in a [word][lane] layout (word i of
 // lane l at i * 32 + l), so every lane reads its own column without bank

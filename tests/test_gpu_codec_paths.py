@@ -174,3 +174,30 @@ def test_streams_of_long_runs(rate):
     rd = np.empty((4, 4, n[0]), dtype=np.float32)
     oc.decode_array(3, rate, s, rd)
     assert np.array_equal(d.cpu().numpy().view(np.uint32), rd.view(np.uint32))
+
+
+# 2-D blocks: extents around a block and a unit, padded rows (element loads),
+# planes in both halves of a word, blocks cut inside the verbatim, group-tested
+# and all-significant planes at both budgets
+@pytest.mark.parametrize("shape", [(1, 1, 1), (3, 5, 7), (2, 4, 128), (1, 33, 132), (5, 64, 260)])
+@pytest.mark.parametrize("rate", [8, 16])
+def test_blocks_2d(shape, rate):
+    r = np.random.default_rng(sum(shape))
+    for x in (r.standard_normal(shape), np.ldexp(r.choice([-1.0, 1.0], shape), -r.integers(0, 33, shape)),
+              np.cumsum(r.standard_normal(shape), 2) + 250.0, np.ldexp(r.standard_normal(shape), -120 - r.integers(0, 8, shape))):
+        round_trip(x.astype(np.float32), 2, rate)
+
+
+@pytest.mark.parametrize("rate", [8, 16])
+def test_random_streams_2d(rate):
+    r = np.random.default_rng(rate)
+    n = (4 * 256, 8, 2)
+    s = r.integers(0, 256, z.zfpx_stream_bytes(2, rate, n), dtype=np.uint8)
+    s[:: 2 * rate] |= 1                                # every block non-zero
+    half = len(s) // 2                                 # half of them with long runs
+    s[:half] = np.where(r.random(half) < 0.7, 0, s[:half]) | (np.arange(half) % (2 * rate) == 0)
+    d = torch.full((2, 8, n[0]), float("nan"), device="cuda")
+    z.zfpx_decode(2, rate, torch.from_numpy(s).cuda(), d)
+    rd = np.empty((2, 8, n[0]), dtype=np.float32)
+    oc.decode_array(2, rate, s, rd)
+    assert np.array_equal(d.cpu().numpy().view(np.uint32), rd.view(np.uint32))
