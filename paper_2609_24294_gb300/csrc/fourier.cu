@@ -56,6 +56,23 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 3) rfft_lon_kernel(const float
     }
 }
 
+// Rows of N = 64 R1 (rfft_row64), one warp per row.  The bound leaves 102
+// registers, which both passes fit, and 20 warps per SM.
+constexpr int kRow64Warps = 4;
+template <int R1>
+__global__ void __launch_bounds__(32 * kRow64Warps, 5)
+rfft_lon64_kernel(const float *__restrict__ in, float *__restrict__ re, float *__restrict__ im,
+                  const float2 *__restrict__ tw, FftGeom g)
+{
+    __shared__ float2 buf[kRow64Warps][row64_values(R1)];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int64_t gr = (int64_t)blockIdx.x * kRow64Warps + wid; gr < g.nrows; gr += (int64_t)gridDim.x * kRow64Warps) {
+        const int64_t y = gr % g.ny, z = gr / g.ny;
+        rfft_row64<R1>(reinterpret_cast<const float2 *>(in + z * g.is2 + y * g.is1), buf[wid], tw, tw + g.N, g.K, lane,
+                       re + z * g.os2 + y * g.os1, im + z * g.os2 + y * g.os1);
+    }
+}
+
 // e^{-2 pi i t / N}, t < N, per (device, N); built once, never freed.
 std::mutex g_tw_mu;
 std::map<std::pair<int, int>, float2 *> g_tw;
@@ -68,15 +85,18 @@ int twiddles_impl(int N, const float2 **out)
     auto key = std::make_pair(dev, N);
     auto it = g_tw.find(key);
     if (it != g_tw.end()) { *out = it->second; return ZFPX_OK; }
-    std::vector<float2> h(N);
+    const int r1 = N % 64 == 0 && row64_radix(N / 64) ? N / 64 : 0;
+    std::vector<float2> h(N + 32 * r1);
     const double two_pi = 6.283185307179586476925286766559;
     for (int t = 0; t < N; t++) {
         const double a = two_pi * (double)t / (double)N;
         h[t] = make_float2((float)std::cos(a), (float)-std::sin(a));
     }
+    for (int s = 0; s < r1; s++)
+        for (int k = 0; k < 32; k++) h[N + 32 * s + k] = h[2 * k * s];       // w_H = w_N^2; 2 k s < N
     float2 *d = nullptr;
-    if (cudaMalloc(&d, sizeof(float2) * N) != cudaSuccess) return ZFPX_ECUDA;
-    if (cudaMemcpy(d, h.data(), sizeof(float2) * N, cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (cudaMalloc(&d, sizeof(float2) * h.size()) != cudaSuccess) return ZFPX_ECUDA;
+    if (cudaMemcpy(d, h.data(), sizeof(float2) * h.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaFree(d);
         return ZFPX_ECUDA;
     }
@@ -107,6 +127,7 @@ int fft_twiddles(int N, const float2 **out) { return twiddles_impl(N, out); }
 bool fft_plan_half(int H, FftGeom &g)
 {
     if (!factor_half_impl(H, g)) return false;
+    g.r1 = H % 32 == 0 && row64_radix(H / 32) ? H / 32 : 0;
     for (int s = 0, r = H; s < g.nst; s++) {
         g.rp[s] = make_fastdiv((uint32_t)(r / g.radix[s]));
         r /= g.radix[s];
@@ -139,6 +160,19 @@ int zfpx_rfft_lon(const float *d_in, const int64_t n[3], const int64_t stride[3]
     const float2 *tw = nullptr;
     int rc = fft_twiddles(g.N, &tw);
     if (rc) return rc;
+    if (g.r1) {
+        void (*k64)(const float *, float *, float *, const float2 *, FftGeom) = nullptr;
+        switch (g.r1) {
+#define ZFPX_FFT_CASE(R) case R: k64 = rfft_lon64_kernel<R>; break;
+            ZFPX_FFT_ROW64_RADICES(ZFPX_FFT_CASE)
+#undef ZFPX_FFT_CASE
+        }
+        const int64_t groups = (g.nrows + kRow64Warps - 1) / kRow64Warps;
+        const int64_t cap = (int64_t)num_sms() * occupancy((const void *)k64, 32 * kRow64Warps);
+        k64<<<(unsigned)std::min<int64_t>(groups, cap), 32 * kRow64Warps, 0, (cudaStream_t)stream>>>(d_in, d_re, d_im, tw, g);
+        count_launch();
+        return check_launch();
+    }
     const size_t smem = 2 * sizeof(float2) * (size_t)warps * g.H;
     if (cudaFuncSetAttribute(rfft_lon_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return ZFPX_ECUDA;

@@ -46,6 +46,14 @@ constexpr int kRows = 16;                      // rows per unit
 template <int RATE>
 constexpr int dec_smem_bytes() { return (2 * RATE + kTileZeroRows<RATE>) * 32 * 4 + 32 * 32 * 8; }
 
+// One copy of each length's transform for both rates' kernels.
+template <int R1>
+__device__ __noinline__ void row64_call(const float2 *src, float2 *buf, const float2 *__restrict__ tw,
+                                        const float2 *__restrict__ tw2, int K, int lane, float *ore, float *oim)
+{
+    fft::rfft_row64<R1>(src, buf, tw, tw2, K, lane, ore, oim);
+}
+
 template <int RATE>
 __global__ void __launch_bounds__(32 * kWarps)
 decode_rfft_kernel(const uint8_t *__restrict__ in, const FusedMsg *__restrict__ msgs, const FusedUnit *__restrict__ units,
@@ -114,11 +122,17 @@ decode_rfft_kernel(const uint8_t *__restrict__ in, const FusedMsg *__restrict__ 
             const int k = r >> 2, j = r & 3;
             if (k >= U.nzr || j >= U.nyr) continue;
             const float2 *src = reinterpret_cast<const float2 *>(rows + (size_t)r * NP);
-            fft::load_row_async(X, src, fg.H, lane);
-            fft::wait_rows();
-            __syncwarp();
             const int64_t o = (int64_t)(U.z0 + k) * os2 + (int64_t)(U.y0 + j) * os1;
-            fft::rfft_row(X, Y, tw, fg, lane, re + o, im + o);
+            switch (fg.r1) {
+#define ZFPX_FFT_CASE(R) case R: row64_call<R>(src, X, tw, tw + fg.N, fg.K, lane, re + o, im + o); break;
+                ZFPX_FFT_ROW64_RADICES(ZFPX_FFT_CASE)
+#undef ZFPX_FFT_CASE
+            default:
+                fft::load_row_async(X, src, fg.H, lane);
+                fft::wait_rows();
+                __syncwarp();
+                fft::rfft_row(X, Y, tw, fg, lane, re + o, im + o);
+            }
         }
         __syncthreads();
     }
