@@ -7,13 +7,21 @@
 // planes 63 .. 0 cut at exactly 64 r bits; decode x = q 2^(e_max - 62)
 // rounded once to nearest even.
 //
-// One lane per block, 32 consecutive blocks per warp, one warp per CTA.  A
-// block's 64 int64 values live in the lane's registers (128 of them) through
-// the gather, quantisation, transform and negabinary map; the 64 bit planes
-// come from four 32x32 register transposes (low / high 32 coefficients x low
-// / high 32 bits) and wait in shared memory ([plane][lane]) for the coder,
-// which writes the lane's column of a [word][lane] stream tile.  Rates 1 .. 32
-// bits per value.
+// One lane per block, 32 consecutive blocks per warp.  A block's 64 int64
+// values live in the lane's registers (128 of them) through the gather,
+// quantisation, transform and negabinary map; the bit planes come from 32x32
+// register transposes (low / high 32 coefficients x low / high 32 bits) and wait
+// in shared memory ([plane][lane]) for the coder, the float32 encoder's
+// (enc3::code), which writes the lane's column of a [word][lane] stream tile.  The
+// low 32 planes are transposed only where a budget reaches them (from about 24
+// bits per value on); until then the encoder parks the coefficients' low words
+// in their slots, and the decoder knows them to be zero.  Rates 1 .. 32 bits
+// per value.
+// What bounds it: latency at ten to twelve warps per SM (registers and shared
+// memory), and the int64 arithmetic.  With all four transposes, a per-lane coder
+// that wrote bit by bit through 64-bit words and 64-bit index divisions, a 640 x
+// 320 x 91 field took 175 / 153 us to encode / decode at rate 8, 207 / 182 at 16
+// and 235 / 219 at 32, now 128 / 129, 139 / 161 and 164 / 217.
 #include <algorithm>
 #include <climits>
 #include <cuda_runtime.h>
@@ -21,6 +29,7 @@
 #include "zfpx_internal.h"
 #include "zfpx_block.cuh"
 #include "zfpx_smem.cuh"
+#include "zfpx_enc3.cuh"
 
 namespace zfpx {
 namespace {
@@ -28,36 +37,12 @@ namespace {
 using namespace blk;
 
 constexpr int kMaxRate = 32;
-constexpr int kF64MinCtas = 10;         // one-warp CTAs per SM the registers are budgeted for
+constexpr int kEncWarps = 2;            // the encoder's warps share its table
+constexpr int kF64MinWarps = 10;        // warps per SM the registers are budgeted for
 constexpr uint64_t kNega64 = 0xAAAAAAAAAAAAAAAAull;
 
 __device__ __forceinline__ int64_t add64(int64_t a, int64_t b) { return (int64_t)((uint64_t)a + (uint64_t)b); }
 __device__ __forceinline__ int64_t sub64(int64_t a, int64_t b) { return (int64_t)((uint64_t)a - (uint64_t)b); }
-
-// Writer into this lane's column of a [word][lane] tile of nwords + 2 words.
-struct VarWriter {
-    uint64_t *sm;
-    uint64_t acc;
-    int nb, w, lane, nwords;
-    __device__ __forceinline__ uint64_t &word(int i) const { return sm[i * 32 + lane]; }
-    __device__ __forceinline__ void put(uint64_t bits, int len)
-    {
-        acc |= bits << nb;
-        int t = nb + len;
-        if (t >= 64) {
-            word(w) = acc;
-            w++;
-            acc = nb ? (bits >> (64 - nb)) : 0ull;
-            t -= 64;
-        }
-        nb = t;
-    }
-    __device__ __forceinline__ void finish()
-    {
-        if (nb > 0) { word(w) = acc; w++; }
-        for (; w < nwords; w++) word(w) = 0ull;
-    }
-};
 
 // One lane's stream in a [64-bit word][lane] tile; peek(pos) = the 64 stream
 // bits from bit pos on (reads words pos / 64 and pos / 64 + 1).
@@ -84,6 +69,8 @@ struct Tile64As32 {
 struct Geom64 {
     int64_t n[3], s[3];
     int64_t bx, by, nblocks, nunits;
+    uint32_t bxm, bym;      // 32-bit divisors of bx and by (used while the block count fits)
+    int32_t bxl, byl;
     int rate;
     int vec;        // unit x stride, even y and z strides, 16-byte aligned base: rows of a block are
                     // two 16-byte moves each
@@ -91,6 +78,13 @@ struct Geom64 {
 
 __device__ __forceinline__ void block_origin(const Geom64 &g, int64_t b, int64_t &x0, int64_t &y0, int64_t &z0)
 {
+    if (g.nblocks <= INT_MAX) {
+        const uint32_t t = divu((uint32_t)b, g.bxm, g.bxl), z = divu(t, g.bym, g.byl);
+        x0 = 4 * (int64_t)((uint32_t)b - t * (uint32_t)g.bx);
+        y0 = 4 * (int64_t)(t - z * (uint32_t)g.by);
+        z0 = 4 * (int64_t)z;
+        return;
+    }
     const int64_t t = b / g.bx;
     x0 = 4 * (b - t * g.bx);
     y0 = 4 * (t % g.by);
@@ -98,10 +92,11 @@ __device__ __forceinline__ void block_origin(const Geom64 &g, int64_t b, int64_t
 }
 
 // exponent: 0 for a zero block, else e_max + 1023 (1 .. 2046)
-__device__ __forceinline__ int block_exponent(uint64_t amax)
+// from the high word of the largest magnitude
+__device__ __forceinline__ int block_exponent(uint32_t amax_hi)
 {
-    const int E = (int)(amax >> 52);
-    if (E == 2047 || amax < 0x0008000000000000ull) return 0;     // non-finite, or below 2^-1023
+    const int E = (int)(amax_hi >> 20);
+    if (E == 2047 || amax_hi < 0x00080000u) return 0;            // non-finite, or below 2^-1023
     return E == 0 ? 1 : E + 1;                                   // frexp exponent + 1023
 }
 
@@ -115,15 +110,17 @@ __device__ __forceinline__ int block_exponent(uint64_t amax)
 // q = trunc(x 2^(62 - e_max)), e = e_max + 1023 the block's exponent: x =
 // +-M 2^(E - 1075) with E the biased exponent (taken as 1 for subnormals) and
 // M the significand (with the implicit bit for normals), so |q| is M shifted
-// left by E + 10 - e (at most 10 within the block whose maximum set e) or
-// right by its negative.
+// left by E + 10 - e (at most 10, in the value whose exponent set e): M 2^10
+// shifted right by e - E.
 __device__ __forceinline__ int64_t quantize64(uint64_t bits, int e)
 {
-    const int E = (int)((bits >> 52) & 0x7ffu);
-    const uint64_t M = (bits & 0x000fffffffffffffull) | (E ? 0x0010000000000000ull : 0ull);
-    const int t = (E ? E : 1) + 10 - e;
-    const uint64_t a = t >= 0 ? (M << t) : (t > -64 ? (M >> -t) : 0ull);
-    return (bits >> 63) ? (int64_t)(0ull - a) : (int64_t)a;
+    const uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
+    const int E = (int)((hi >> 20) & 0x7ffu);
+    const uint32_t m = (hi & 0x000fffffu) | (E ? 0x00100000u : 0u);
+    const uint64_t M = ((uint64_t)__funnelshift_l(lo, m, 10) << 32) | (lo << 10);
+    const uint64_t a = shr_any(M, e - (E ? E : 1));
+    const uint64_t s = (uint64_t)(int64_t)((int32_t)hi >> 31);   // all ones for a negative value
+    return (int64_t)((a ^ s) - s);
 }
 
 // x = q 2^(e - 1085) rounded once to nearest even, for e >= 63, where every
@@ -194,97 +191,129 @@ __device__ __forceinline__ void xform3_inv64(int64_t (&v)[64])
             lift_inv64r(v[16 * k + 4 * j], v[16 * k + 4 * j + 1], v[16 * k + 4 * j + 2], v[16 * k + 4 * j + 3]);
 }
 
-// Shared memory of one warp: the 64 bit planes ([plane][lane]) and the stream
-// tile ([64-bit word][lane], rate words and two zero words).
-__host__ __device__ constexpr size_t f64_smem_bytes(int rate) { return (size_t)(64 + rate + 2) * 32 * 8; }
-
-__global__ void __launch_bounds__(32, kF64MinCtas) encode_f64_kernel(const double *__restrict__ src,
-                                                                     uint8_t *__restrict__ out, Geom64 g)
+// Shared memory of one decoder warp: the 64 bit planes ([plane][lane]) and the
+// stream tile ([64-bit word][lane], rate words and two zero words); of an
+// encoder CTA: per warp the planes and the stream tile ([32-bit word][lane], 2
+// rate words and four slack words), and the table.
+__host__ __device__ constexpr size_t f64_dec_smem_bytes(int rate) { return (size_t)(64 + rate + 2) * 32 * 8; }
+__host__ __device__ constexpr size_t f64_enc_smem_bytes(int rate)
 {
-    extern __shared__ uint64_t sm64[];
-    uint64_t *stile = sm64 + 64 * 32;
-    const int lane = threadIdx.x;
-    SmemPlanes pl{sm64, lane};
+    return sizeof(enc3::Expand) + (size_t)kEncWarps * (64 * 32 * 8 + (size_t)(2 * rate + 4) * 32 * 4);
+}
+
+__global__ void __launch_bounds__(32 * kEncWarps, kF64MinWarps / kEncWarps)
+encode_f64_kernel(const double *__restrict__ src, uint8_t *__restrict__ out, Geom64 g)
+{
+    extern __shared__ __align__(16) uint64_t sm64[];
+    enc3::Expand &expand = *reinterpret_cast<enc3::Expand *>(sm64);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = 2 * g.rate;
+    uint64_t *wplanes = sm64 + sizeof(enc3::Expand) / 8 + (size_t)wid * (64 * 32 + (size_t)(nw + 4) * 16);
+    uint32_t *tile = reinterpret_cast<uint32_t *>(wplanes + 64 * 32) + lane;
+    uint64_t *planes = wplanes + lane;                          // plane k at planes[32 k]
+    uint32_t *p32 = reinterpret_cast<uint32_t *>(planes);        // half h of plane k at p32[64 k + h]
     constexpr int kSeq[64] = ZFPX_SEQ3;
-    for (int64_t u = blockIdx.x; u < g.nunits; u += gridDim.x) {
+    enc3::load_expand(expand);
+    for (int w = 0; w < nw + 4; w++) tile[32 * w] = 0u;
+    enc3::wait_expand();
+    __syncthreads();
+    const bool out16 = (g.rate & 1) == 0 && !((uintptr_t)out & 15u);
+    for (int64_t u = (int64_t)blockIdx.x * kEncWarps + wid; u < g.nunits; u += (int64_t)gridDim.x * kEncWarps) {
         const int64_t b0 = u * 32;
         const int nact = (int)min((int64_t)32, g.nblocks - b0);
-        if (lane < nact) {
-            int64_t x0, y0, z0;
-            block_origin(g, b0 + lane, x0, y0, z0);
-            int64_t v[64];
-            if (g.vec && x0 + 4 <= g.n[0] && y0 + 4 <= g.n[1] && z0 + 4 <= g.n[2]) {
-                // an interior block: two 16-byte loads per row
+        const bool valid = lane < nact;
+        int64_t x0, y0, z0;
+        // lanes past the unit's last block load that block and code nothing
+        block_origin(g, b0 + (valid ? lane : nact - 1), x0, y0, z0);
+        int64_t v[64];
+        if (g.vec && x0 + 4 <= g.n[0] && y0 + 4 <= g.n[1] && z0 + 4 <= g.n[2]) {
+            // an interior block: two 16-byte loads per row
+            const double *p = src + z0 * g.s[2] + y0 * g.s[1] + x0;
 #pragma unroll
-                for (int k = 0; k < 4; k++)
+            for (int k = 0; k < 4; k++) {
+                const double *row = p;
 #pragma unroll
-                    for (int j = 0; j < 4; j++) {
-                        const double2 *row = reinterpret_cast<const double2 *>(src + (z0 + k) * g.s[2] +
-                                                                               (y0 + j) * g.s[1] + x0);
-                        const double2 a = __ldg(row), b = __ldg(row + 1);
-                        v[16 * k + 4 * j] = __double_as_longlong(a.x);
-                        v[16 * k + 4 * j + 1] = __double_as_longlong(a.y);
-                        v[16 * k + 4 * j + 2] = __double_as_longlong(b.x);
-                        v[16 * k + 4 * j + 3] = __double_as_longlong(b.y);
-                    }
-            } else {
-                // edge blocks and other layouts: element loads, the last row, level
-                // and point repeated past the array's end, through a local array
-                // kept rolled so the hot path's code stays compact
-                int64_t t[64];
-#pragma unroll 1
-                for (int r = 0; r < 64; r++) {
-                    const int i = r & 3, j = (r >> 2) & 3, k = r >> 4;
-                    t[r] = __double_as_longlong(__ldg(src + min(z0 + k, g.n[2] - 1) * g.s[2] +
-                                                      min(y0 + j, g.n[1] - 1) * g.s[1] +
-                                                      min(x0 + i, g.n[0] - 1) * g.s[0]));
+                for (int j = 0; j < 4; j++) {
+                    const double2 a = __ldg(reinterpret_cast<const double2 *>(row));
+                    const double2 b = __ldg(reinterpret_cast<const double2 *>(row) + 1);
+                    v[16 * k + 4 * j] = __double_as_longlong(a.x);
+                    v[16 * k + 4 * j + 1] = __double_as_longlong(a.y);
+                    v[16 * k + 4 * j + 2] = __double_as_longlong(b.x);
+                    v[16 * k + 4 * j + 3] = __double_as_longlong(b.y);
+                    row += g.s[1];
                 }
-#pragma unroll
-                for (int r = 0; r < 64; r++) v[r] = t[r];
+                p += g.s[2];
             }
-            uint64_t amax = 0;
-#pragma unroll
+        } else {
+            // edge blocks and other layouts: element loads, the last row, level
+            // and point repeated past the array's end, through a local array
+            // kept rolled so the hot path's code stays compact
+            int64_t t[64];
+#pragma unroll 1
             for (int r = 0; r < 64; r++) {
-                const uint64_t a = (uint64_t)v[r] & 0x7fffffffffffffffull;
-                amax = a > amax ? a : amax;
+                const int i = r & 3, j = (r >> 2) & 3, k = r >> 4;
+                t[r] = __double_as_longlong(__ldg(src + min(z0 + k, g.n[2] - 1) * g.s[2] +
+                                                  min(y0 + j, g.n[1] - 1) * g.s[1] +
+                                                  min(x0 + i, g.n[0] - 1) * g.s[0]));
             }
-            const int e = block_exponent(amax);
-            VarWriter wr{stile, 0ull, 0, 0, lane, g.rate};
-            if (!e) {
-                wr.finish();
-            } else {
 #pragma unroll
-                for (int r = 0; r < 64; r++) v[r] = quantize64((uint64_t)v[r], e);
-                xform3_fwd64(v);
+            for (int r = 0; r < 64; r++) v[r] = t[r];
+        }
+        uint32_t amax = 0;                                       // high word of the largest magnitude
 #pragma unroll
-                for (int r = 0; r < 64; r++) v[r] = (int64_t)(((uint64_t)v[r] + kNega64) ^ kNega64);
-                // the 64 planes by quadrant: bits 32 hb .. 32 hb + 31 of the
-                // coefficients 32 ch .. 32 ch + 31 in coding order.  The loop over
-                // ch stays rolled (a select picks the coefficient): half the code
-                // of four unrolled quadrants, which the instruction cache holds
-                // better beside the unrolled lifting
+        for (int r = 0; r < 64; r++) amax = max(amax, (uint32_t)((uint64_t)v[r] >> 32) & 0x7fffffffu);
+        const int e = block_exponent(amax);
+        const bool act = valid && e;
 #pragma unroll
-                for (int hb = 0; hb < 2; hb++)
+        for (int r = 0; r < 64; r++) v[r] = quantize64((uint64_t)v[r], e);
+        xform3_fwd64(v);
+        // negabinary: the add here, the xor as the complement of the odd planes
+#pragma unroll
+        for (int r = 0; r < 64; r++) v[r] = (int64_t)((uint64_t)v[r] + kNega64);
+        // planes 32 .. 63 from the high words of the coefficients in coding
+        // order; the low words wait in the slots of planes 0 .. 31.  The loop over
+        // the coefficients' halves stays rolled (a select picks the coefficient):
+        // half the code, which the instruction cache holds better beside the
+        // unrolled lifting
 #pragma unroll 1
-                    for (int ch = 0; ch < 2; ch++) {
-                        uint32_t w[32];
+        for (int ch = 0; ch < 2; ch++) {
+            uint32_t w[32];
 #pragma unroll
-                        for (int t = 0; t < 32; t++)
-                            w[t] = (uint32_t)((uint64_t)(ch ? v[kSeq[32 + t]] : v[kSeq[t]]) >> (32 * hb));
-                        transpose32(w);
+            for (int t = 0; t < 32; t++) {
+                const uint64_t c = (uint64_t)(ch ? v[kSeq[32 + t]] : v[kSeq[t]]);
+                w[t] = (uint32_t)(c >> 32);
+                p32[64 * t + ch] = (uint32_t)c;
+            }
+            transpose32(w);
 #pragma unroll
-                        for (int k = 0; k < 32; k++) pl.store_half(32 * hb + k, ch, w[k]);
-                    }
-                wr.put(1ull | ((uint64_t)e << 1), 12);
-                int n = 0, R = 64 * g.rate - 12;
+            for (int k = 0; k < 32; k++) p32[64 * (32 + k) + ch] = k & 1 ? ~w[k] : w[k];
+        }
+        auto finish_low = [&]() {
 #pragma unroll 1
-                for (int k = 63; k >= 0 && R > 0; k--) code_plane<64>(wr, pl.load(k), n, R);
-                wr.finish();
+            for (int ch = 0; ch < 2; ch++) {
+                uint32_t w[32];
+#pragma unroll
+                for (int t = 0; t < 32; t++) w[t] = p32[64 * t + ch];
+                transpose32(w);
+#pragma unroll
+                for (int k = 0; k < 32; k++) p32[64 * k + ch] = k & 1 ? ~w[k] : w[k];
+            }
+        };
+        if (act) tile[0] = 1u | ((uint32_t)e << 1);
+        enc3::code<false>(enc3::smem(tile), enc3::smem(expand.e), planes, 63, 12, 64 * g.rate, 0, act, 32, finish_low);
+        __syncwarp();
+        uint8_t *dst = out + (b0 + lane) * (int64_t)g.rate * 8;
+        if (out16) {
+            for (int i = 0; i < nw; i += 4) {
+                const uint4 c = make_uint4(tile[32 * i], tile[32 * (i + 1)], tile[32 * (i + 2)], tile[32 * (i + 3)]);
+                if (valid) *reinterpret_cast<uint4 *>(dst + 4 * i) = c;
+            }
+        } else {
+            for (int i = 0; i < nw; i += 2) {
+                const uint2 c = make_uint2(tile[32 * i], tile[32 * (i + 1)]);
+                if (valid) *reinterpret_cast<uint2 *>(dst + 4 * i) = c;
             }
         }
-        __syncwarp();
-        uint64_t *dst = reinterpret_cast<uint64_t *>(out) + b0 * g.rate;
-        for (int idx = lane; idx < nact * g.rate; idx += 32) dst[idx] = stile[(idx % g.rate) * 32 + idx / g.rate];
+        for (int w = 0; w < nw + 4; w++) tile[32 * w] = 0u;
         __syncwarp();
     }
 }
@@ -329,8 +358,8 @@ __device__ __forceinline__ double dequantize64(int64_t q, int e)
     return __longlong_as_double((long long)(m | sign));
 }
 
-__global__ void __launch_bounds__(32, kF64MinCtas) decode_f64_kernel(const uint8_t *__restrict__ in,
-                                                                     double *__restrict__ dst, Geom64 g)
+__global__ void __launch_bounds__(32, kF64MinWarps) decode_f64_kernel(const uint8_t *__restrict__ in,
+                                                                      double *__restrict__ dst, Geom64 g)
 {
     extern __shared__ uint64_t sm64[];
     uint64_t *tile = sm64 + 64 * 32;
@@ -361,26 +390,42 @@ __global__ void __launch_bounds__(32, kF64MinCtas) decode_f64_kernel(const uint8
             // parser read past the budget without a test
             const Tile64As32 t32{reinterpret_cast<const uint32_t *>(tile), lane};
             const int kmin = parse_planes64<true>(t32, 12, 64 * g.rate, 63, pl);
-#pragma unroll 1
-            for (int k = 0; k < kmin; k++) pl.store(k, 0ull);
+            // planes below kmin are zero; the negabinary xor is the complement of
+            // the odd planes
             int64_t v[64];
 #pragma unroll
-            for (int hb = 0; hb < 2; hb++)
+            for (int ch = 0; ch < 2; ch++) {
+                uint32_t w[32];
+#pragma unroll
+                for (int k = 0; k < 32; k++) {
+                    const uint32_t c = 32 + k >= kmin ? pl.load_half(32 + k, ch) : 0u;
+                    w[k] = k & 1 ? ~c : c;
+                }
+                transpose32(w);
+#pragma unroll
+                for (int t = 0; t < 32; t++) v[kSeq[32 * ch + t]] = (int64_t)((uint64_t)w[t] << 32);
+            }
+            if (__all_sync(__activemask(), kmin >= 32)) {
+                // no low plane in any lane: every low word is M - M = 0
+#pragma unroll
+                for (int r = 0; r < 64; r++) v[r] = sub64(v[r], (int64_t)(kNega64 & 0xffffffff00000000ull));
+            } else {
 #pragma unroll
                 for (int ch = 0; ch < 2; ch++) {
                     uint32_t w[32];
 #pragma unroll
-                    for (int k = 0; k < 32; k++) w[k] = pl.load_half(32 * hb + k, ch);
+                    for (int k = 0; k < 32; k++) {
+                        const uint32_t c = k >= kmin ? pl.load_half(k, ch) : 0u;
+                        w[k] = k & 1 ? ~c : c;
+                    }
                     transpose32(w);
-                    // w[t] = bits 32 hb .. 32 hb + 31 of coefficient 32 ch + t
 #pragma unroll
                     for (int t = 0; t < 32; t++) {
                         int64_t &c = v[kSeq[32 * ch + t]];
-                        c = hb ? (int64_t)(((uint64_t)c & 0xffffffffull) | ((uint64_t)w[t] << 32)) : (int64_t)w[t];
+                        c = sub64((int64_t)((uint64_t)c | w[t]), (int64_t)kNega64);
                     }
                 }
-#pragma unroll
-            for (int r = 0; r < 64; r++) v[r] = sub64((int64_t)((uint64_t)v[r] ^ kNega64), (int64_t)kNega64);
+            }
             xform3_inv64(v);
             if (e >= 63) {
 #pragma unroll
@@ -429,17 +474,20 @@ Geom64 make_geom(const int64_t n[3], const int64_t s[3], int rate, const void *b
     for (int a = 0; a < 3; a++) { g.n[a] = n[a]; g.s[a] = s[a]; }
     g.bx = (n[0] + 3) / 4; g.by = (n[1] + 3) / 4;
     g.nblocks = g.bx * g.by * ((n[2] + 3) / 4);
+    block_divisor((uint32_t)std::min<int64_t>(g.bx, INT_MAX), g.bxm, g.bxl);
+    block_divisor((uint32_t)std::min<int64_t>(g.by, INT_MAX), g.bym, g.byl);
     g.nunits = (g.nblocks + 31) / 32;
     g.rate = rate;
     return g;
 }
 
-unsigned grid_f64(const void *fn, int64_t nunits, size_t smem)
+unsigned grid_f64(const void *fn, int warps, int64_t nunits, size_t smem)
 {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * warps, smem) != cudaSuccess || per_sm < 1)
+        per_sm = 1;
     const int64_t cap = (int64_t)num_sms() * per_sm;
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(nunits, cap));
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((nunits + warps - 1) / warps, cap));
 }
 
 // Dynamic shared memory above 48 KB is opted into per kernel.
@@ -478,11 +526,11 @@ int zfpx_encode_f64(int rate, const double *d_in, const int64_t n[3], const int6
     if (((uintptr_t)d_out & 7u) || ((uintptr_t)d_in & 7u)) return ZFPX_EINVAL;
     if (cap < zfpx_stream_bytes_f64(rate, n)) return ZFPX_ESIZE;
     const Geom64 g = make_geom(n, stride, rate, d_in);
-    const size_t smem = f64_smem_bytes(rate);
+    const size_t smem = f64_enc_smem_bytes(rate);
     const int rc = f64_prepare((const void *)encode_f64_kernel, smem);
     if (rc) return rc;
-    encode_f64_kernel<<<grid_f64((const void *)encode_f64_kernel, g.nunits, smem), 32, smem, (cudaStream_t)stream>>>(
-        d_in, d_out, g);
+    encode_f64_kernel<<<grid_f64((const void *)encode_f64_kernel, kEncWarps, g.nunits, smem), 32 * kEncWarps, smem,
+                        (cudaStream_t)stream>>>(d_in, d_out, g);
     count_launch();
     return check_launch();
 }
@@ -494,10 +542,10 @@ int zfpx_decode_f64(int rate, const uint8_t *d_in, size_t len, const int64_t n[3
     if (((uintptr_t)d_out & 7u) || ((uintptr_t)d_in & 7u)) return ZFPX_EINVAL;
     if (len < zfpx_stream_bytes_f64(rate, n)) return ZFPX_ESIZE;
     const Geom64 g = make_geom(n, stride, rate, d_out);
-    const size_t smem = f64_smem_bytes(rate);
+    const size_t smem = f64_dec_smem_bytes(rate);
     const int rc = f64_prepare((const void *)decode_f64_kernel, smem);
     if (rc) return rc;
-    decode_f64_kernel<<<grid_f64((const void *)decode_f64_kernel, g.nunits, smem), 32, smem, (cudaStream_t)stream>>>(
+    decode_f64_kernel<<<grid_f64((const void *)decode_f64_kernel, 1, g.nunits, smem), 32, smem, (cudaStream_t)stream>>>(
         d_in, d_out, g);
     count_launch();
     return check_launch();

@@ -163,6 +163,11 @@ __device__ __forceinline__ void red_or(uint32_t a, uint32_t v)
     asm volatile("red.shared.or.b32 [%0+%2], %1;" ::"r"(a), "r"(v), "n"(OFF) : "memory");
 }
 
+__device__ __forceinline__ void store_word(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
 // One step of a group-tested part: the code of the next eight coefficients
 // (the low bits of zh:zl, shifted out) ORed into the lane's stream after bit A,
 // with e0 at bit A itself (the plane's group bit ahead of its first eight);
@@ -180,6 +185,108 @@ __device__ __forceinline__ void chunk(uint32_t &zl, uint32_t &zh, int &A, uint32
     red_or<0>(w, e << s);
     red_or<128>(w, shr(e, 32u - s));
     A += 8 + popc32(c);
+}
+
+// The coder: bit planes ktop, ktop - 1, ... (plane k at planes[32 k]) into the
+// lane's stream at shared address tb from bit pos on, cut at bit END; lanes that
+// are not `act` code nothing.  finish_low() is called before the first plane
+// below kLow is read.  LEN: returns how many bits of the stream planes ktop ..
+// kmin take (END at most; 1 for an inactive lane, the zero block's bit);
+// planes below kmin may then be left out of it.  Every lane of the warp calls it.
+template <bool LEN, class FinishLow>
+__device__ __forceinline__ int code(uint32_t tb, uint32_t xb, uint64_t *planes, int ktop, int pos, const int END,
+                                    int kmin, bool act, const int kLow, FinishLow &&finish_low)
+{
+    // ---- phase A: planes while n < 64
+    int n1 = 1, kB = -1;                               // n + 1
+    uint64_t lm = 0;                                   // low n bits
+    bool low_done = false;
+    const uint32_t list0 = smem(planes + 32 * ktop);
+    uint32_t list = list0;                             // where the next entry goes
+#pragma unroll 1
+    for (int k = act ? ktop : -1; k >= kmin; k--) {
+        if (k == kLow - 1) {
+            finish_low();
+            low_done = true;
+        }
+        const uint64_t X = planes[32 * k];
+        const uint64_t Y = X & ~lm, V = X & lm;
+        const uint32_t vl = (uint32_t)V, vh = (uint32_t)(V >> 32), s = (uint32_t)pos & 31u;
+        const uint32_t w = tb + 4u * (uint32_t)(pos & ~31);
+        red_or<0>(w, vl << s);
+        red_or<128>(w, funnel(vl, vh, s));
+        red_or<256>(w, funnel(vh, 0u, s));
+        // the group bit and the first eight coefficients of the group-tested
+        // part now (the next eight too where more than 52 remain), the rest
+        // listed; without new ones all of it is zeros
+        const bool any = Y != 0;
+        const uint64_t Z = Y >> (n1 - 1);
+        uint32_t zl = (uint32_t)Z, zh = (uint32_t)(Z >> 32);
+        int A = pos + n1 - 1;                          // the group bit
+        if (any) {
+            const int lead = 63 - highest_set64(Y);
+            lm = ~0ull >> lead;
+            n1 = 65 - lead;
+        }
+        pos += popc64(Y) + n1;
+        const uint32_t last = n1 == 65 ? 1024u : 512u;
+        chunk(zl, zh, A, any ? 1u : 0u, tb, xb, last);
+        if (zh >> 20) chunk(zl, zh, A, 0u, tb, xb, last);
+        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(list), "r"(zl),
+                     "r"(zh | (n1 == 65 ? 1u << 20 : 0u) | ((uint32_t)A << 21)) : "memory");
+        if ((zl | zh) && A < END) list -= 256;
+        kB = k - 1;
+        if (n1 == 65 || pos >= END) break;
+    }
+    __syncwarp();                                      // the lanes go on together
+    if (n1 == 65) pos -= 2;                            // coefficient 63's one is implied: no value or group bit
+
+    int len = 0;
+    if (LEN) len = act ? min(END, pos + (n1 == 65 ? 64 * max(0, kB - kmin + 1) : 0)) : 1;
+
+    // ---- phase B: planes kB, kB - 1, ... verbatim from bit pos
+    if (n1 == 65 && pos < END) {
+        const uint32_t s = (uint32_t)pos & 31u;
+        const int w0 = pos >> 5, nw = END >> 5;
+        // the lowest plane read here: kB - m for the m with w0 + 2 m < nw
+        if (!low_done && kB - ((nw - w0 + 1) / 2 - 1) < kLow) finish_low();
+        uint32_t prev = 0;
+#pragma unroll 1
+        for (int wa = w0; wa < nw; wa += 2) {
+            const uint64_t X = kB >= 0 ? planes[32 * kB] : 0ull;
+            const uint32_t xl = (uint32_t)X, xh = (uint32_t)(X >> 32);
+            if (wa == w0) red_or<0>(tb + 128u * wa, xl << s);
+            else store_word(tb + 128u * wa, funnel(prev, xl, s));
+            store_word(tb + 128u * (wa + 1), funnel(xl, xh, s));
+            prev = xh;
+            kB--;
+        }
+    }
+    __syncwarp();
+
+    // ---- the list: eight coefficients per step, each lane through its own
+    // entries; a lane without any ORs zeros
+    {
+        uint32_t next = list0, zl = 0, zh = 0, last = 512u;
+        int A = 0;
+#pragma unroll 1
+        while (__any_sync(0xffffffffu, (zl | zh) != 0 || next != list)) {
+            if ((zl | zh) == 0 && next != list) {
+                asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(zl), "=r"(zh) : "r"(next));
+                next -= 256;
+                A = (int)(zh >> 21);
+                last = zh & (1u << 20) ? 1024u : 512u;
+                zh &= (1u << 20) - 1u;
+            }
+            if (A >= END) {                            // positions only grow: nothing later is sent
+                zl = zh = 0;
+                next = list;
+                A = 0;
+            }
+            chunk(zl, zh, A, 0u, tb, xb, last);
+        }
+    }
+    return len;
 }
 
 // LEN: also returns how many bits the block's planes 31 .. kmin take (at most
@@ -236,7 +343,6 @@ __device__ __forceinline__ int encode(const float (&x)[64], bool valid, const Vi
 #pragma unroll
         for (int k = 0; k < 32; k++) p32[64 * k + half] = k >= kLow && (k & 1) ? ~lo[k] : lo[k];
     }
-    bool low_done = false;
     auto finish_low = [&]() {
         uint32_t a[32], b[32];
 #pragma unroll
@@ -251,97 +357,9 @@ __device__ __forceinline__ int encode(const float (&x)[64], bool valid, const Vi
             const uint32_t c = i & 1 ? 0xffffffffu : 0u;
             planes[32 * i] = ((uint64_t)(b[i] ^ c) << 32) | (a[i] ^ c);
         }
-        low_done = true;
     };
     if (act) tile[0] = 1u | ((uint32_t)(E + 1) << 1);
-
-    // ---- phase A: planes while n < 64
-    int n1 = 1, pos = 9, kB = -1;                      // n + 1
-    uint64_t lm = 0;                                   // low n bits
-    const uint32_t tb = smem(tile), xb = smem(sh.expand), list0 = smem(planes + 31 * 32);
-    uint32_t list = list0;                             // where the next entry goes
-    const int kmin = LEN ? cut.kmin(E - 126) : 0;
-#pragma unroll 1
-    for (int k = act ? 31 : -1; k >= kmin; k--) {
-        if (k == kLow - 1) finish_low();
-        const uint64_t X = planes[32 * k];
-        const uint64_t Y = X & ~lm, V = X & lm;
-        const uint32_t vl = (uint32_t)V, vh = (uint32_t)(V >> 32), s = (uint32_t)pos & 31u;
-        const uint32_t w = tb + 4u * (uint32_t)(pos & ~31);
-        red_or<0>(w, vl << s);
-        red_or<128>(w, funnel(vl, vh, s));
-        red_or<256>(w, funnel(vh, 0u, s));
-        // the group bit and the first eight coefficients of the group-tested
-        // part now (the next eight too where more than 53 remain), the rest
-        // listed; without new ones all of it is zeros
-        const bool any = Y != 0;
-        const uint64_t Z = Y >> (n1 - 1);
-        uint32_t zl = (uint32_t)Z, zh = (uint32_t)(Z >> 32);
-        int A = pos + n1 - 1;                          // the group bit
-        if (any) {
-            const int lead = 63 - highest_set64(Y);
-            lm = ~0ull >> lead;
-            n1 = 65 - lead;
-        }
-        pos += popc64(Y) + n1;
-        const uint32_t last = n1 == 65 ? 1024u : 512u;
-        chunk(zl, zh, A, any ? 1u : 0u, tb, xb, last);
-        if (zh >> 21) chunk(zl, zh, A, 0u, tb, xb, last);
-        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(list), "r"(zl),
-                     "r"(zh | (n1 == 65 ? 1u << 21 : 0u) | ((uint32_t)A << 22)) : "memory");
-        if ((zl | zh) && A < END) list -= 256;
-        kB = k - 1;
-        if (n1 == 65 || pos >= END) break;
-    }
-    __syncwarp();                                      // the lanes go on together
-    if (n1 == 65) pos -= 2;                            // coefficient 63's one is implied: no value or group bit
-
-    int len = 0;
-    if (LEN) len = act ? min(END, pos + (n1 == 65 ? 64 * max(0, kB - kmin + 1) : 0)) : 1;
-
-    // ---- phase B: planes kB, kB - 1, ... verbatim from bit pos
-    if (n1 == 65 && pos < END) {
-        const uint32_t s = (uint32_t)pos & 31u;
-        const int w0 = pos >> 5;
-        // the lowest plane read here: kB - m for the m with w0 + 2 m < 2 RATE
-        if (!low_done && kB - ((2 * RATE - w0 + 1) / 2 - 1) < kLow) finish_low();
-        uint32_t prev = 0;
-#pragma unroll 1
-        for (int wa = w0; wa < 2 * RATE; wa += 2) {
-            const uint64_t X = kB >= 0 ? planes[32 * kB] : 0ull;
-            const uint32_t xl = (uint32_t)X, xh = (uint32_t)(X >> 32);
-            if (wa == w0) red_or<0>(tb + 128u * wa, xl << s);
-            else tile[32 * wa] = funnel(prev, xl, s);
-            tile[32 * (wa + 1)] = funnel(xl, xh, s);
-            prev = xh;
-            kB--;
-        }
-    }
-    __syncwarp();
-
-    // ---- the list: eight coefficients per step, each lane through its own
-    // entries; a lane without any ORs zeros
-    {
-        uint32_t next = list0, zl = 0, zh = 0, last = 512u;
-        int A = 0;
-#pragma unroll 1
-        while (__any_sync(0xffffffffu, (zl | zh) != 0 || next != list)) {
-            if ((zl | zh) == 0 && next != list) {
-                asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(zl), "=r"(zh) : "r"(next));
-                next -= 256;
-                A = (int)(zh >> 22);
-                last = zh & (1u << 21) ? 1024u : 512u;
-                zh &= (1u << 21) - 1u;
-            }
-            if (A >= END) {                            // positions only grow: nothing later is sent
-                zl = zh = 0;
-                next = list;
-                A = 0;
-            }
-            chunk(zl, zh, A, 0u, tb, xb, last);
-        }
-    }
-    return len;
+    return code<LEN>(smem(tile), smem(sh.expand), planes, 31, 9, END, LEN ? cut.kmin(E - 126) : 0, act, kLow, finish_low);
 }
 
 // Copies this lane's 2 RATE stream words to dst (16-byte aligned, the

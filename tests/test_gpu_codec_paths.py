@@ -201,3 +201,29 @@ def test_random_streams_2d(rate):
     rd = np.empty((2, 8, n[0]), dtype=np.float32)
     oc.decode_array(2, rate, s, rd)
     assert np.array_equal(d.cpu().numpy().view(np.uint32), rd.view(np.uint32))
+
+
+# float64: coefficients that become significant in every one of the 64 planes, so
+# that the low 32 planes are reached in phase A (sparse blocks, any rate), in the
+# verbatim planes (rates from about 24 on) or not at all; odd rates and streams on
+# 8 bytes; a unit with one block
+@pytest.mark.parametrize("rate", [1, 3, 8, 15, 16, 24, 31, 32])
+@pytest.mark.parametrize("shape,offset", [((4, 4, 4), 0), ((5, 9, 132), 8)])
+def test_float64_planes(rate, shape, offset):
+    r = np.random.default_rng(rate)
+    n = tuple(reversed(shape))
+    nb = z.zfpx_stream_bytes_f64(rate, n)
+    for x in (np.ldexp(r.choice([-1.0, 1.0], shape) * r.choice([1.0, 1.25, 1.999], shape), -r.integers(0, 65, shape)),
+              np.full(shape, 3.0) + np.ldexp(r.standard_normal(shape), -r.integers(30, 60)),
+              np.cumsum(r.standard_normal(shape), 2) + 250.0,
+              np.ldexp(r.standard_normal(shape), -1010 - r.integers(0, 20, shape)),
+              np.where(r.random(shape) < 0.02, np.inf, r.standard_normal(shape))):
+        s = torch.zeros(nb + 16, dtype=torch.uint8, device="cuda")[offset:offset + nb]
+        xd, d = torch.from_numpy(x).cuda(), torch.full(shape, float("nan"), dtype=torch.float64, device="cuda")
+        z.zfpx_encode_f64(rate, xd, s)
+        ref = oc.encode_array_f64(rate, x)
+        assert np.array_equal(s.cpu().numpy(), ref)
+        z.zfpx_decode_f64(rate, s, d)
+        rd = np.empty(shape)
+        oc.decode_array_f64(rate, ref, rd)
+        assert np.array_equal(d.cpu().numpy().view(np.uint64), rd.view(np.uint64))
