@@ -37,18 +37,16 @@ using namespace blk;
 constexpr int kWarps = 4;
 constexpr int kThreads = 32 * kWarps;
 // Launch shapes of the 3-D kernels, chosen by measurement on GB300: encoder
-// CTAs of 2 warps, nine to an SM at rate 8 and eight at rate 16, what the
-// shared memory allows (where rows don't start on 16 bytes eight at both, which
-// leaves the four scalar loads per row their registers: 194 us against 209 for
-// a 1000 x 501 x 91 field on 3 x 3 ranks); decoder CTAs of 4 warps, except the
-// rate-16 decoder, whose 3-warp CTAs fit six to an SM (two zero rows after its
-// stream tile make the shared memory fit); the rate-8 decoder is compiled for
-// five resident CTAs, which its shared memory allows and capping its registers
-// to match pays for.
+// CTAs of 2 warps, eight to an SM (the shared memory of a ninth is there at rate
+// 8, but five warps on a scheduler leave 96 registers and a few spills: 287 us
+// against 274 for a 1280 x 640 x 137 field over 8 x 8 ranks); decoder CTAs of 4
+// warps, except the rate-16 decoder, whose 3-warp CTAs fit six to an SM (two zero
+// rows after its stream tile make the shared memory fit); the rate-8 decoder is
+// compiled for five resident CTAs, which its shared memory allows and capping its
+// registers to match pays for (four: 10 % slower).
 template <int RATE>
 constexpr int kEnc3Warps = 2;
-template <int RATE, bool VEC>
-constexpr int kEnc3MinBlocks = RATE == 8 && VEC ? 9 : 8;
+constexpr int kEnc3MinBlocks = 8;
 template <int RATE>
 constexpr int kDec3Warps = RATE == 16 ? 3 : 4;
 template <int RATE>
@@ -106,15 +104,117 @@ struct UnitRange {
     }
 };
 
+// ----------------------------------------------------------------- rows of a 3-D block
+// Rows that don't start on 16 bytes (a longitude split 3, 6, 7 ... ways, a padded
+// row pitch): with unit x stride and even y and z strides every row of a
+// message starts alike, on 8 bytes or 4 past them, and moves as two 8-byte
+// accesses or as 4 + 8 + 4 bytes.  Any other layout moves value by value.
+enum RowKind { ROWS_8 = 0, ROWS_4_8_4 = 1, ROWS_ANY = 2 };
+__device__ __forceinline__ int row_kind(const void *first, const int64_t *s)
+{
+    if (s[0] != 1 || ((s[1] | s[2]) & 1)) return ROWS_ANY;
+    return ((uintptr_t)first >> 2) & 1 ? ROWS_4_8_4 : ROWS_8;
+}
+
+// The 64 values of the block at p (rows past the end of the box repeat its
+// last row); every row complete in x.
+template <int KIND>
+__device__ __forceinline__ void load_rows(const float *p, const int64_t *s, int ny, int nz, float (&x)[64])
+{
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const float *row = p;
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            float *v = x + 16 * k + 4 * j;
+            if (KIND == ROWS_8) {
+                const float2 a = __ldg(reinterpret_cast<const float2 *>(row));
+                const float2 b = __ldg(reinterpret_cast<const float2 *>(row) + 1);
+                v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+            } else if (KIND == ROWS_4_8_4) {
+                const float2 b = __ldg(reinterpret_cast<const float2 *>(row + 1));
+                v[0] = __ldg(row); v[1] = b.x; v[2] = b.y; v[3] = __ldg(row + 3);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; i++) v[i] = __ldg(row + (int64_t)i * s[0]);
+            }
+            if (j + 1 < ny) row += s[1];
+        }
+        if (k + 1 < nz) p += s[2];
+    }
+}
+
+// The same with partial rows (nx < 4 values, the last one repeated): four
+// values at a time through the lane's column of `stage` (64 rows of 32 floats),
+// kept rolled so that the complete blocks' code stays compact.
+__device__ __forceinline__ void load_edge(const float *p, const int64_t *s, int nx, int ny, int nz, float *stage,
+                                          float (&x)[64])
+{
+#pragma unroll 1
+    for (int r = 0; r < 16; r++) {
+        const float *row = p + (int64_t)min(r >> 2, nz - 1) * s[2] + (int64_t)min(r & 3, ny - 1) * s[1];
+#pragma unroll
+        for (int i = 0; i < 4; i++) stage[32 * (4 * r + i)] = __ldg(row + (int64_t)min(i, nx - 1) * s[0]);
+    }
+#pragma unroll
+    for (int r = 0; r < 64; r++) x[r] = stage[32 * r];
+}
+
+// The inverses: only rows inside the box are written.
+template <int KIND>
+__device__ __forceinline__ void store_rows(float *p, const int64_t *s, int ny, int nz, const float (&x)[64])
+{
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            float *row = p + (int64_t)k * s[2] + (int64_t)j * s[1];
+            const float *v = x + 16 * k + 4 * j;
+            if (k < nz && j < ny) {
+                if (KIND == ROWS_8) {
+                    reinterpret_cast<float2 *>(row)[0] = make_float2(v[0], v[1]);
+                    reinterpret_cast<float2 *>(row)[1] = make_float2(v[2], v[3]);
+                } else if (KIND == ROWS_4_8_4) {
+                    row[0] = v[0];
+                    *reinterpret_cast<float2 *>(row + 1) = make_float2(v[1], v[2]);
+                    row[3] = v[3];
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; i++) row[(int64_t)i * s[0]] = v[i];
+                }
+            }
+        }
+    }
+}
+__device__ __forceinline__ void store_edge(float *p, const int64_t *s, int nx, int ny, int nz, float *stage,
+                                           const float (&x)[64])
+{
+#pragma unroll
+    for (int r = 0; r < 64; r++) stage[32 * r] = x[r];
+#pragma unroll 1
+    for (int r = 0; r < 16; r++) {
+        if ((r >> 2) >= nz || (r & 3) >= ny) continue;
+        float *row = p + (int64_t)(r >> 2) * s[2] + (int64_t)(r & 3) * s[1];
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+            if (i < nx) row[(int64_t)i * s[0]] = stage[32 * (4 * r + i)];
+    }
+}
+
 // ================================================================= 3-D kernels
 // VEC: every block's rows start on 16 bytes (the view's row and level strides
 // and every message's x origin are multiples of 4 values, the base aligned),
 // so full rows move as 16-byte loads and stores.  Otherwise a separate
-// instantiation reads and writes the rows of x-complete blocks as four scalar
-// accesses each, unrolled, keeping the vector kernel's code as it is.
+// instantiation moves the rows by their kind (load_rows), keeping the vector
+// kernel's code as it is.  Blocks partial in x go through load_edge in both.
+// Four scalar accesses per row and partial blocks value by value through a local
+// array took 5760 (compress) and 5130 (decompress) warp instructions per 32
+// blocks of a 1000 x 501 x 91 field on 3 x 3 ranks, against 3540 and 4040 for
+// aligned rows: 192 / 174 us at rate 8, now 172 / 131; a 233 x 117 x 137 array of
+// aligned rows, one partial block in 59, went from 26.6 / 26.6 to 22.5 / 20.5 us.
 // LEN: the variable-rate modes, which also want every block's bit count (acc).
 template <int RATE, bool VEC, bool LEN>
-__global__ void __launch_bounds__(32 * kEnc3Warps<RATE>, kEnc3MinBlocks<RATE, VEC>)
+__global__ void __launch_bounds__(32 * kEnc3Warps<RATE>, kEnc3MinBlocks)
 encode3_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchGeom g, int layout, AccEncode acc)
 {
     __shared__ enc3::Shared<RATE> sh[kEnc3Warps<RATE>];
@@ -161,30 +261,17 @@ encode3_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchG
                     }
                     if (z0 + k + 1 < nz) p += g.ss[2];
                 }
-            } else if (!VEC && x0 + 4 <= nx) {
-                // rows not on 16 bytes: four scalar loads per row
-#pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    const int64_t zo = (int64_t)min(z0 + k, nz - 1) * g.ss[2];
-#pragma unroll
-                    for (int j = 0; j < 4; j++) {
-                        const float *row = base + zo + (int64_t)min(y0 + j, ny - 1) * g.ss[1] + (int64_t)x0 * g.ss[0];
-#pragma unroll
-                        for (int i = 0; i < 4; i++) x[16 * k + 4 * j + i] = __ldg(row + (int64_t)i * g.ss[0]);
-                    }
-                }
             } else {
-                // partial in x: element loads through a local
-                // array, kept rolled so the hot path's code stays compact
-                float t[64];
-#pragma unroll 1
-                for (int r = 0; r < 64; r++) {
-                    const int i = r & 3, j = (r >> 2) & 3, k = r >> 4;
-                    t[r] = __ldg(base + (int64_t)min(z0 + k, nz - 1) * g.ss[2] +
-                                 (int64_t)min(y0 + j, ny - 1) * g.ss[1] + (int64_t)min(x0 + i, nx - 1) * g.ss[0]);
-                }
-#pragma unroll
-                for (int r = 0; r < 64; r++) x[r] = t[r];
+                const float *p = base + (int64_t)z0 * g.ss[2] + (int64_t)y0 * g.ss[1] + (int64_t)x0 * g.ss[0];
+                const int kind = VEC ? ROWS_ANY : row_kind(base, g.ss);
+                if (x0 + 4 > nx)
+                    load_edge(p, g.ss, nx - x0, ny - y0, nz - z0, reinterpret_cast<float *>(v.planes) + lane, x);
+                else if (!VEC && kind == ROWS_8)
+                    load_rows<ROWS_8>(p, g.ss, ny - y0, nz - z0, x);
+                else if (!VEC && kind == ROWS_4_8_4)
+                    load_rows<ROWS_4_8_4>(p, g.ss, ny - y0, nz - z0, x);
+                else if (!VEC)
+                    load_rows<ROWS_ANY>(p, g.ss, ny - y0, nz - z0, x);
             }
         }
         const int len = enc3::encode<RATE, LEN>(x, valid, v, lane, enc3::PlaneCut{acc.minexp, acc.prec});
@@ -307,29 +394,17 @@ decode3_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchG
                                                                            v[16 * k + 4 * j + 2], v[16 * k + 4 * j + 3]);
                     }
                 }
-            } else if (!VEC && x0 + 4 <= nx) {
-                // rows not on 16 bytes: four scalar stores per row
-#pragma unroll
-                for (int k = 0; k < 4; k++) {
-#pragma unroll
-                    for (int j = 0; j < 4; j++) {
-                        float *row = base + (int64_t)(z0 + k) * g.ds[2] + (int64_t)(y0 + j) * g.ds[1] + (int64_t)x0 * g.ds[0];
-                        if (z0 + k < nz && y0 + j < ny) {
-#pragma unroll
-                            for (int i = 0; i < 4; i++) row[(int64_t)i * g.ds[0]] = v[16 * k + 4 * j + i];
-                        }
-                    }
-                }
             } else {
-                float t[64];
-#pragma unroll
-                for (int r = 0; r < 64; r++) t[r] = v[r];
-#pragma unroll 1
-                for (int r = 0; r < 64; r++) {
-                    const int i = r & 3, j = (r >> 2) & 3, k = r >> 4;
-                    if (x0 + i < nx && y0 + j < ny && z0 + k < nz)
-                        base[(int64_t)(z0 + k) * g.ds[2] + (int64_t)(y0 + j) * g.ds[1] + (int64_t)(x0 + i) * g.ds[0]] = t[r];
-                }
+                float *p = base + (int64_t)z0 * g.ds[2] + (int64_t)y0 * g.ds[1] + (int64_t)x0 * g.ds[0];
+                const int kind = VEC ? ROWS_ANY : row_kind(base, g.ds);
+                if (x0 + 4 > nx)
+                    store_edge(p, g.ds, nx - x0, ny - y0, nz - z0, reinterpret_cast<float *>(splanes[wid]) + lane, v);
+                else if (!VEC && kind == ROWS_8)
+                    store_rows<ROWS_8>(p, g.ds, ny - y0, nz - z0, v);
+                else if (!VEC && kind == ROWS_4_8_4)
+                    store_rows<ROWS_4_8_4>(p, g.ds, ny - y0, nz - z0, v);
+                else if (!VEC)
+                    store_rows<ROWS_ANY>(p, g.ds, ny - y0, nz - z0, v);
             }
         }
         __syncwarp();

@@ -227,3 +227,38 @@ def test_float64_planes(rate, shape, offset):
         rd = np.empty(shape)
         oc.decode_array_f64(rate, ref, rd)
         assert np.array_equal(d.cpu().numpy().view(np.uint64), rd.view(np.uint64))
+
+
+# rows of every kind -- on 16, 8 and 4 bytes, rows that start alike and rows that
+# don't (odd row pitch), values apart -- with every remainder of the x extent, one
+# and several messages, both directions, nothing written outside the view
+@pytest.mark.parametrize("rate", [8, 16])
+@pytest.mark.parametrize("start,pitch,step", [(0, 0, 1), (0, 2, 1), (1, 2, 1), (2, 2, 1), (3, 1, 1), (1, 3, 1), (1, 2, 2)])
+@pytest.mark.parametrize("nx", [4, 37, 42, 131])
+def test_row_kinds(nx, start, pitch, step, rate):
+    r = np.random.default_rng(nx)
+    ny, nz = 9, 6
+    width = start + step * nx + pitch
+    width += width & 1 if pitch == 2 else 0            # even row pitch: rows start alike
+    a = torch.from_numpy(r.standard_normal((nz, ny, width)).astype(np.float32)).cuda()
+    o = torch.full((nz, ny, width), 7.0, device="cuda")
+    src, dst = (t[:, :, start:start + step * nx:step] for t in (a, o))
+    x = np.ascontiguousarray(src.cpu().numpy())
+    for pr, pc in ((1, 1), (2, 3)):
+        plan = z.Plan.for_fields(src, pr, pc, 0, 3, dst=dst)
+        s = torch.zeros(plan.buffer_bytes(rate), dtype=torch.uint8, device="cuda")
+        o.fill_(7.0)
+        z.zfpx_pack_compress(plan, rate, src, s)
+        z.zfpx_decompress_unpack(plan, rate, s, dst, layout=z.LAYOUT_SEND)
+        got, full = s.cpu().numpy(), o.cpu().numpy()
+        vals = full[:, :, start:start + step * nx:step]
+        for (sr, ds, _, _), (x0, mx, y0, my, z0, mz) in plan.messages():
+            box = np.ascontiguousarray(x[z0:z0 + mz, y0:y0 + my, x0:x0 + mx])
+            ref = oc.encode_array(3, rate, box)
+            off = plan.message_offset(rate, z.LAYOUT_SEND, sr, ds)
+            assert np.array_equal(got[off:off + len(ref)], ref)
+            rd = np.empty_like(box)
+            oc.decode_array(3, rate, ref, rd)
+            assert np.array_equal(vals[z0:z0 + mz, y0:y0 + my, x0:x0 + mx].view(np.uint32), rd.view(np.uint32))
+        full[:, :, start:start + step * nx:step] = 7.0
+        assert (full == 7.0).all()
