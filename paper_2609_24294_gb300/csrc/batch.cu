@@ -111,8 +111,11 @@ __device__ __forceinline__ void fill_plane4(const BatchGeom &bg, Tab &tab)
 
 // Work distribution of the batch kernels.  A batch with no more units than
 // the grid has warps gives each warp one unit.  Otherwise each (dims, rate)
-// group is a queue of units claimed upc at a time (one atomic add per claim)
-// by whole warps.  A CTA starts on
+// group is a queue of units claimed by whole warps, at most upc at a time (one
+// atomic add per claim) and towards the queue's end fewer, down to one, so that
+// no warp holds several units while others find the queues empty: ten percent of
+// a launch of fifty units per warp (965 us against 911 and 887 with claims of
+// one, three 3-D and six 1-D fields on a grid of 1280 rows).  A CTA starts on
 // its home group -- the SMs are split between groups in proportion to their
 // work, so an SM mostly runs one kind's code and keeps it in its instruction
 // cache -- and then helps the other groups until every queue is empty.
@@ -123,12 +126,16 @@ __device__ __forceinline__ void for_each_unit(const BatchGeom &bg, int lane, Fn 
 {
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const bool single = bg.nunits <= nwarps;                     // a small batch: one unit per warp, no claims
-    const uint32_t C = (uint32_t)bg.upc;
     int gi = 0, tried = 1;                                       // the group in work, groups seen so far
-    uint32_t u = 0;                                              // the unit inside it
-    auto claim = [&]() {
+    uint32_t u = 0, C = 1;                                       // the claim: first unit inside the group, units
+    // units to claim once unit `seen` has been reached: half a warp's share of what is left
+    auto size = [&](uint32_t seen) {
+        const int64_t share = (bg.groups[gi].n - (int64_t)seen) / (2 * nwarps);
+        return (uint32_t)max((int64_t)1, min(share, (int64_t)bg.upc));
+    };
+    auto claim = [&](uint32_t units) {
         uint32_t v = 0;
-        if (lane == 0) v = atomicAdd(bg.ctr + gi, C);
+        if (lane == 0) v = atomicAdd(bg.ctr + gi, units);
         return v;
     };
     if (single) {
@@ -142,16 +149,19 @@ __device__ __forceinline__ void for_each_unit(const BatchGeom &bg, int lane, Fn 
         asm volatile("mov.u32 %0, %%nsmid;" : "=r"(nsmid));
         const float x = ((float)smid + 0.5f) / (float)nsmid;
         while (gi + 1 < bg.ngroups && x >= bg.groups[gi].cum1) gi++;
-        u = __shfl_sync(0xffffffffu, claim(), 0);
+        C = size(0);
+        u = __shfl_sync(0xffffffffu, claim(C), 0);
     }
     for (;;) {
         while (!single && (int64_t)u >= bg.groups[gi].n) {       // this queue is empty: the next group's
             if (tried++ == bg.ngroups) return;
             gi = gi + 1 == bg.ngroups ? 0 : gi + 1;
-            u = __shfl_sync(0xffffffffu, claim(), 0);
+            C = 1;                                               // likely near its end by now
+            u = __shfl_sync(0xffffffffu, claim(C), 0);
         }
         const GroupDev G = bg.groups[gi];
-        const uint32_t next = single ? 0u : claim();             // claimed ahead: its latency hides behind fn
+        const uint32_t nextC = single ? 1u : size(u);
+        const uint32_t next = single ? 0u : claim(nextC);        // claimed ahead: its latency hides behind fn
         // the claim's units in order; a unit's item is the last one starting at or before it
         const uint32_t ue = single ? u + 1 : (uint32_t)min((int64_t)u + C, G.n);
         int ii = item_of_unit(bg.items, bg.nitems, G.u0 + u);
@@ -162,6 +172,7 @@ __device__ __forceinline__ void for_each_unit(const BatchGeom &bg, int lane, Fn 
         }
         if (single) return;
         u = __shfl_sync(0xffffffffu, next, 0);
+        C = nextC;
     }
 }
 
@@ -527,10 +538,24 @@ int64_t field_stream_bytes(const GridHost &g, const zfpx_field &F, int r0, int r
 }
 
 // Blocks of one work unit: 32 for 3-D items (one per lane), 32 lb1 for 1-D.
-constexpr int kDefaultLb1 = 16;
 constexpr int kMaxLb1 = 64;
 constexpr int kDefaultUpc = 4;
 constexpr int kMaxUpc = 64;
+// lb1 where the caller has set none: about four units per resident warp over the
+// batch's 1-D blocks, from kLoads1 (a lane's blocks in lockstep: fewer cost the
+// same) to 16.  A lone small batch of 1-D fields ends 4 us earlier than with 16
+// (23.6 -> 19.5 us for three fields on a grid of 122 rows).
+int auto_lb1(const GridHost &g, const zfpx_field *fields, int nfields)
+{
+    int64_t blocks = 0;
+    for (int f = 0; f < nfields; f++) {
+        const zfpx_field &F = fields[f];
+        const int r1 = (F.row0 == 0 && F.row1 == 0) ? g.nrows : F.row1;
+        if (F.dims == 1) blocks += F.nlev * (g.rpre[r1] - g.rpre[F.row0]);
+    }
+    const int64_t per = blocks / (32ll * num_sms() * 16 * 4);
+    return (int)std::max<int64_t>(kLoads1, std::min<int64_t>(per, 16));
+}
 inline int64_t unit_blocks(int dims, int lb1) { return dims == 3 ? 32 : 32 * (int64_t)lb1; }
 
 // Field and item descriptors of a set of fields whose streams start at the
@@ -650,6 +675,10 @@ int launch_batch(const BatchGeom &g, int warps, int ctas_per_sm, bool encode, co
                  cudaStream_t st)
 {
     if (g.nunits == 0) return ZFPX_OK;
+    // where the caller has set none: CTAs of two warps, sixteen warps to an SM, for
+    // batches that fill the device (885 / 867 us against 911 / 879 with three), else
+    // three, which spread a small batch's units better over the schedulers
+    if (!warps) warps = g.nunits > (int64_t)num_sms() * 15 ? 2 : 3;
     if (!batch_warps_ok(warps)) return ZFPX_EINVAL;
     const void *fn = warps == 2 ? batch_kernel<2>(encode) : warps == 3 ? batch_kernel<3>(encode)
                    : warps == 8 ? batch_kernel<8>(encode) : batch_kernel<4>(encode);
@@ -675,8 +704,9 @@ struct zfpx_batch_s {
     int64_t total = 0;
     int nitems = 0;
     int64_t nunits = 0;
-    int warps = 3, ctas_per_sm = 0;     // 0 = as many as fit
-    int lb1 = zfpx::kDefaultLb1;        // 1-D blocks per lane of a unit
+    int warps = 0, ctas_per_sm = 0;     // 0 = the library's choice, as many as fit
+    int lb1 = 0;                        // 1-D blocks per lane of a unit; 0 = the library's choice
+    int lb1_used = 0;                   // what the tables were built with
     int upc = zfpx::kDefaultUpc;        // units per work claim
     zfpx::FieldDevB *d_fields = nullptr;
     zfpx::ItemDevB *d_items = nullptr;
@@ -703,8 +733,9 @@ static int batch_work(zfpx_batch b)
 {
     std::vector<FieldDevB> fd;
     std::vector<ItemDevB> items;
-    build_work(b->grid, b->fields.data(), b->field_off.data(), (int)b->fields.size(), b->lb1, fd, items, b->nunits,
-               b->groups);
+    b->lb1_used = b->lb1 ? b->lb1 : auto_lb1(b->grid, b->fields.data(), (int)b->fields.size());
+    build_work(b->grid, b->fields.data(), b->field_off.data(), (int)b->fields.size(), b->lb1_used, fd, items,
+               b->nunits, b->groups);
     b->nitems = (int)items.size();
     cudaFree(b->d_fields);
     cudaFree(b->d_items);
@@ -777,10 +808,10 @@ int zfpx_batch_set_claim_units(zfpx_batch b, int units_per_claim)
 int zfpx_batch_set_unit_blocks(zfpx_batch b, int blocks_per_lane_1d)
 {
     if (!b || blocks_per_lane_1d < 1 || blocks_per_lane_1d > kMaxLb1) return ZFPX_EINVAL;
-    if (blocks_per_lane_1d == b->lb1) return ZFPX_OK;
+    b->lb1 = blocks_per_lane_1d;
+    if (blocks_per_lane_1d == b->lb1_used) return ZFPX_OK;
     // the tables in use by launches still in flight stay valid until they finish
     if (cudaDeviceSynchronize() != cudaSuccess) return ZFPX_ECUDA;
-    b->lb1 = blocks_per_lane_1d;
     return batch_work(b);
 }
 
@@ -789,7 +820,7 @@ static int batch_geom(zfpx_batch b, bool encode, cudaStream_t st, BatchGeom &g)
 {
     uint32_t *ctr = b->d_ctr + (encode ? 0 : kMaxGroups);
     if (cudaMemsetAsync(ctr, 0, kMaxGroups * sizeof(uint32_t), st) != cudaSuccess) return ZFPX_ECUDA;
-    g = make_geom(b->d_fields, b->d_items, b->grid.dev(), b->nitems, b->nunits, b->groups, b->lb1, b->upc, ctr);
+    g = make_geom(b->d_fields, b->d_items, b->grid.dev(), b->nitems, b->nunits, b->groups, b->lb1_used, b->upc, ctr);
     return ZFPX_OK;
 }
 
@@ -903,8 +934,8 @@ struct zfpx_server_s {
     int next_slot = 0;
     int64_t next_id = 1;
     int max_batch = 64;
-    int warps = 3, ctas_per_sm = 0;
-    int lb1 = zfpx::kDefaultLb1;
+    int warps = 0, ctas_per_sm = 0;     // 0 = the library's choice
+    int lb1 = 0;
     int upc = zfpx::kDefaultUpc;
     int min_batch = 1;                  // batching window: launch at min_batch waiting requests
     double max_wait_s = 0.0;            // ... or once the oldest has waited this long
@@ -1073,7 +1104,8 @@ int zfpx_server_pump(zfpx_server s, int *launched)
     std::vector<ItemDevB> items;
     std::vector<GroupDev> groups;
     int64_t units = 0;
-    build_work(s->grid, fields.data(), soff.data(), (int)fields.size(), s->lb1, fd, items, units, groups);
+    const int lb1 = s->lb1 ? s->lb1 : auto_lb1(s->grid, fields.data(), (int)fields.size());
+    build_work(s->grid, fields.data(), soff.data(), (int)fields.size(), lb1, fd, items, units, groups);
     // descriptors: fields, items, then zeroed work counters (encode, decode)
     const size_t fbytes = fd.size() * sizeof(FieldDevB);
     const size_t ioff = (fbytes + 255) / 256 * 256;
@@ -1088,8 +1120,8 @@ int zfpx_server_pump(zfpx_server s, int *launched)
     uint32_t *ctr = reinterpret_cast<uint32_t *>(sl.d_desc + coff);
     const FieldDevB *dfd = reinterpret_cast<const FieldDevB *>(sl.d_desc);
     const ItemDevB *dit = reinterpret_cast<const ItemDevB *>(sl.d_desc + ioff);
-    const BatchGeom ge = make_geom(dfd, dit, s->grid.dev(), (int)items.size(), units, groups, s->lb1, s->upc, ctr);
-    const BatchGeom gd = make_geom(dfd, dit, s->grid.dev(), (int)items.size(), units, groups, s->lb1, s->upc,
+    const BatchGeom ge = make_geom(dfd, dit, s->grid.dev(), (int)items.size(), units, groups, lb1, s->upc, ctr);
+    const BatchGeom gd = make_geom(dfd, dit, s->grid.dev(), (int)items.size(), units, groups, lb1, s->upc,
                                    ctr + kMaxGroups);
     int rc = launch_batch(ge, s->warps, s->ctas_per_sm, true, nullptr, s->d_arena, sl.stream);
     if (!rc) rc = launch_batch(gd, s->warps, s->ctas_per_sm, false, s->d_arena, nullptr, sl.stream);

@@ -262,3 +262,33 @@ def test_row_kinds(nx, start, pitch, step, rate):
             assert np.array_equal(vals[z0:z0 + mz, y0:y0 + my, x0:x0 + mx].view(np.uint32), rd.view(np.uint32))
         full[:, :, start:start + step * nx:step] = 7.0
         assert (full == 7.0).all()
+
+
+# batches on both sides of the claim path (fewer and more units than the grid has
+# warps) and of the library's own launch shape, unit size and claims: every choice
+# gives the bytes and values of the one-warp-per-unit settings
+@pytest.mark.parametrize("N,nlev,nsingle", [(8, 1, 1), (24, 5, 3), (160, 9, 2), (320, 8, 4)])
+def test_batch_defaults(N, nlev, nsingle):
+    north = 20 + 4 * np.arange(N)
+    lens = np.concatenate([north, north[::-1]]).tolist()
+    g = torch.Generator("cuda").manual_seed(N)
+    fields = []
+    for k, (lev, dims) in enumerate([(nlev, 3)] * 2 + [(1, 1)] * nsingle):
+        f = 250.0 + torch.cumsum(torch.randn((lev, sum(lens)), device="cuda", generator=g), 1) * 0.1
+        fields.append((f, torch.zeros_like(f), dims, (8, 16)[k % 2]))
+    ref = None
+    for settings in (None, (3, 16, 1), (2, 5, 64), (8, 1, 3)):
+        b = z.Batch(lens, fields)
+        if settings:
+            b.set_launch(settings[0])
+            b.set_unit_blocks(settings[1])
+            b.set_claim_units(settings[2])
+        s = torch.zeros(b.nbytes(), dtype=torch.uint8, device="cuda")
+        for f in fields:
+            f[1].zero_()
+        b.encode(s)
+        b.decode(s)
+        got = [s] + [f[1].clone() for f in fields]
+        ref = ref or got
+        assert all(torch.equal(a, c) for a, c in zip(got, ref))
+        b.close()
