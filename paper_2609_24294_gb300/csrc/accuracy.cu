@@ -44,6 +44,8 @@ __global__ void __launch_bounds__(kTile) acc_scan_tiles_kernel(const uint16_t *_
                                                                uint64_t *__restrict__ totals)
 {
     __shared__ uint32_t warp_sum[kTile / 32];
+    start_next();
+    wait_previous(lengths);
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const int64_t b = (int64_t)blockIdx.x * kTile + t;
     const uint32_t v = b < nblocks ? lengths[b] : 0u;
@@ -105,6 +107,8 @@ __global__ void __launch_bounds__(kTile) acc_scan_totals_kernel(const uint64_t *
                                                                 uint64_t *__restrict__ total_bits)
 {
     __shared__ uint64_t sums[kTile / 32];
+    start_next();
+    wait_previous(totals);
     uint64_t carry = 0, all;
     for (int64_t base = 0; base < ntiles; base += kTile) {
         const int64_t i = base + threadIdx.x;
@@ -166,9 +170,11 @@ __global__ void __launch_bounds__(32 * kPackWarps) acc_pack_kernel(AccList P, co
     __shared__ __align__(8) uint32_t buf[kPackWarps][kPackWords];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t g0 = ((int64_t)blockIdx.x * kPackWarps + wid) * 32;
-    if (g0 >= P.G) return;
+    start_next();
     uint32_t *w = buf[wid];
     for (int i = lane; i < kPackWords; i += 32) w[i] = 0u;
+    wait_previous(slots);
+    if (g0 >= P.G) return;
     const int n = (int)min((int64_t)32, P.G - g0);
     const int64_t g = g0 + min(lane, n - 1);
     uint64_t off;
@@ -230,6 +236,8 @@ __global__ void __launch_bounds__(32 * kPackWarps) acc_pack_kernel(AccList P, co
 __global__ void __launch_bounds__(256) acc_zero_tail_kernel(uint64_t *__restrict__ payload,
                                                             const uint64_t *__restrict__ count, int bits, int64_t words)
 {
+    start_next();
+    wait_previous(count);
     const int64_t used = (int64_t)(bits ? (*count + 63) / 64 : *count);
     for (int64_t i = used + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words;
          i += (int64_t)gridDim.x * blockDim.x)
@@ -279,9 +287,9 @@ int plan_geom(zfpx_plan p, LaunchGeom &g)
 
 int acc_scan(const AccWork &a, const uint16_t *lengths, uint64_t *total_bits, cudaStream_t st)
 {
-    acc_scan_tiles_kernel<<<(unsigned)a.ntiles, kTile, 0, st>>>(lengths, a.nblocks, a.local, a.totals);
+    launch_after(acc_scan_tiles_kernel, (unsigned)a.ntiles, kTile, 0, st, lengths, a.nblocks, a.local, a.totals);
     count_launch();
-    acc_scan_totals_kernel<<<1, kTile, 0, st>>>(a.totals, a.ntiles, a.tile_off, total_bits);
+    launch_after(acc_scan_totals_kernel, 1, kTile, 0, st, a.totals, a.ntiles, a.tile_off, total_bits);
     count_launch();
     return check_launch();
 }
@@ -290,12 +298,10 @@ int acc_scan(const AccWork &a, const uint16_t *lengths, uint64_t *total_bits, cu
 int acc_pack(const AccList &P, const uint8_t *slots, uint8_t *payload, const uint64_t *count, int bits, cudaStream_t st)
 {
     const int64_t per_cta = 32 * kPackWarps;
-    acc_pack_kernel<<<(unsigned)((P.G + per_cta - 1) / per_cta), 32 * kPackWarps, 0, st>>>(
-        P, slots, reinterpret_cast<uint64_t *>(payload));
+    launch_after(acc_pack_kernel, (unsigned)((P.G + per_cta - 1) / per_cta), 32 * kPackWarps, 0, st, P, slots, reinterpret_cast<uint64_t *>(payload));
     count_launch();
     const int64_t words = P.G * 16, want = (words + 255) / 256;
-    acc_zero_tail_kernel<<<(unsigned)std::min<int64_t>(want, (int64_t)num_sms() * 8), 256, 0, st>>>(
-        reinterpret_cast<uint64_t *>(payload), count, bits, words);
+    launch_after(acc_zero_tail_kernel, (unsigned)std::min<int64_t>(want, (int64_t)num_sms() * 8), 256, 0, st, reinterpret_cast<uint64_t *>(payload), count, bits, words);
     count_launch();
     return check_launch();
 }
@@ -424,6 +430,8 @@ __global__ void __launch_bounds__(kTile) pacc_messages_kernel(PlanAcc P, const u
                                                               uint64_t *words, int send, uint64_t *used)
 {
     __shared__ uint64_t sums[kTile / 32];
+    start_next();
+    wait_previous(local, tile_off, total);
     auto bit = [&](int64_t g) { return g < P.G ? tile_off[g / kTile] + local[g] : *total; };
     uint64_t carry = 0, all;
     for (int base = 0; base < P.M; base += kTile) {
@@ -463,6 +471,8 @@ __global__ void __launch_bounds__(256) pacc_exchange_kernel(PlanAcc P, const uin
                                                             const uint16_t *__restrict__ len_in,
                                                             uint16_t *__restrict__ len_out, int64_t cap_words)
 {
+    start_next();
+    wait_previous(words, pay_in, len_in);
     const int m = blockIdx.x;
     const AccMsg a = P.msgs[m];
     // counts that would run past either buffer are cut there
@@ -593,7 +603,7 @@ static int pack_compress_variable(zfpx_plan p, int minexp, int prec, const float
     if ((rc = acc_scan(w.scan, d_lengths, w.scan.total, st))) return rc;
     // the sum of the word counts, where the payload ends, in the scratch after the total
     uint64_t *used = w.scan.total + 1;
-    pacc_messages_kernel<<<1, kTile, 0, st>>>(w.P, w.scan.local, w.scan.tile_off, w.scan.total, d_msg_words, 1, used);
+    launch_after(pacc_messages_kernel, 1, kTile, 0, st, w.P, w.scan.local, w.scan.tile_off, w.scan.total, d_msg_words, 1, used);
     count_launch();
     if ((rc = check_launch())) return rc;
     return acc_pack(AccList{w.P.msgs, w.P.pay_send, d_lengths, w.scan.local, w.scan.tile_off, w.P.M, G}, w.slots,
@@ -633,12 +643,12 @@ int zfpx_exchange_accuracy(zfpx_plan p, const uint64_t *d_msg_words, const uint1
     PlanAccWork w;
     int rc = plan_acc_setup(p, d_work, work_bytes, st, &w);
     if (rc || w.P.M == 0) return rc;
-    pacc_messages_kernel<<<1, kTile, 0, st>>>(w.P, nullptr, nullptr, nullptr, const_cast<uint64_t *>(d_msg_words), 0,
+    launch_after(pacc_messages_kernel, 1, kTile, 0, st, w.P, nullptr, nullptr, nullptr, const_cast<uint64_t *>(d_msg_words), 0,
                                               nullptr);
     count_launch();
     // about eight CTAs per SM over all messages
     const unsigned parts = (unsigned)std::max<int64_t>(1, std::min<int64_t>(64, (int64_t)num_sms() * 8 / w.P.M));
-    pacc_exchange_kernel<<<dim3((unsigned)w.P.M, parts), 256, 0, st>>>(w.P, d_msg_words,
+    launch_after(pacc_exchange_kernel, dim3((unsigned)w.P.M, parts), 256, 0, st, w.P, d_msg_words,
                                                            reinterpret_cast<const uint64_t *>(d_pay_send),
                                                            reinterpret_cast<uint64_t *>(d_pay_recv), d_len_send,
                                                            d_len_recv, (int64_t)(cap / 8));
@@ -657,7 +667,7 @@ int zfpx_decompress_unpack_accuracy(zfpx_plan p, const uint64_t *d_msg_words, co
     PlanAccWork w;
     int rc = plan_acc_setup(p, d_work, work_bytes, st, &w);
     if (rc || G == 0) return rc;
-    pacc_messages_kernel<<<1, kTile, 0, st>>>(w.P, nullptr, nullptr, nullptr, const_cast<uint64_t *>(d_msg_words), 0,
+    launch_after(pacc_messages_kernel, 1, kTile, 0, st, w.P, nullptr, nullptr, nullptr, const_cast<uint64_t *>(d_msg_words), 0,
                                               nullptr);
     count_launch();
     if ((rc = acc_scan(w.scan, d_len_recv, w.scan.total, st))) return rc;

@@ -292,3 +292,41 @@ def test_batch_defaults(N, nlev, nsingle):
         ref = ref or got
         assert all(torch.equal(a, c) for a, c in zip(got, ref))
         b.close()
+
+
+# the variable-rate chain's launches overlap their predecessors; a replayed
+# capture of two encodes and a decode over one scratch gives the eager results
+@pytest.mark.parametrize("shape", [(3, 2, 5), (17, 75, 161)])
+def test_captured_accuracy_chain(shape):
+    n = tuple(reversed(shape))
+    r = np.random.default_rng(sum(shape))
+    xs = [torch.from_numpy(r.standard_normal(shape).astype(np.float32)).cuda() for _ in range(2)]
+    nb = int(np.prod([(k + 3) // 4 for k in n]))
+    work = torch.zeros(z.zfpx_accuracy_workspace_bytes(n), dtype=torch.uint8, device="cuda")
+
+    def outputs():
+        return [(torch.zeros(nb, dtype=torch.uint16, device="cuda"),
+                 torch.full((z.zfpx_accuracy_max_payload_bytes(n),), 255, dtype=torch.uint8, device="cuda"),
+                 torch.zeros(1, dtype=torch.int64, device="cuda")) for _ in xs], torch.zeros(shape, device="cuda")
+
+    def chain(outs, d):
+        for x, o in zip(xs, outs):
+            z.zfpx_encode_accuracy(x, 1e-3, *o, work)
+        z.zfpx_decode_accuracy(outs[1][0], outs[1][1], d, work)
+
+    want, dw = outputs()
+    got, dg = outputs()
+    chain(want, dw)
+    chain(got, dg)
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    graph = z.capture(lambda: chain(got, dg), st)
+    for o in got:
+        o[0].zero_(), o[1].fill_(255), o[2].zero_()
+    dg.zero_()
+    torch.cuda.synchronize()
+    graph.launch(st)
+    torch.cuda.synchronize()
+    for a, b in zip(want, got):
+        assert all(torch.equal(i.view(torch.uint8), j.view(torch.uint8)) for i, j in zip(a, b))
+    assert torch.equal(dw.view(torch.int32), dg.view(torch.int32))
