@@ -29,16 +29,10 @@
 // to TF32, and a b = a_hi b_hi + a_hi b_lo + a_lo b_hi, accumulated in float32
 // in tensor memory; the dropped a_lo b_lo and the TF32 rounding of the lo
 // parts leave about 2^-21 of sum |a b| per product, far below the float32
-// dot-product bound the transform is held to.  A CTA of four warps computes a
-// 128-row x Nt-column tile of one (m, p) block: one lane of warp 0 keeps TMA
-// loads of 32-deep K slices of both operands (128-byte swizzled) up to four
-// stages ahead, the other three warps derive the lo tiles in place, one of
-// their threads issues the MMAs (three per 8-deep K step) and commits them to
-// the stage's mbarrier, which frees the stage for the next load; after the
-// last slice each warp reads its 32 rows of the accumulator from tensor
-// memory and scatters them into the triangular output.  Every wait is
-// bounded; a wait that runs out sets the plan's status word and the CTA
-// stops.
+// dot-product bound the transform is held to.  One CTA per SM walks 128-row x
+// Nt-column tiles of the (m, p) blocks (legendre_mma_kernel below); each warp
+// role waits only on mbarriers, every wait is bounded, and a wait that runs
+// out sets the plan's status word and the CTA stops.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -60,12 +54,10 @@ struct zfpx_legendre_s {
     int nlat = 0, T = 0, nh = 0, nhs = 0, device = 0;
     int64_t table_rows = 0;
     float *d_table = nullptr;   // K-major: [table_rows][nhs] floats, columns >= nh zero
-    float *d_table_lo = nullptr;   // the table's TF32 low parts (tf32_lo), same layout
     LegItem *d_items = nullptr;
     int *d_status = nullptr;    // 0, or the code of a wait that ran out
     int nitems = 0;
     CUtensorMap tmap_table;     // TMA view of the table: {nh, table_rows}, boxes {32, 128}
-    CUtensorMap tmap_table_lo;  // the same view of its low parts
 };
 
 namespace zfpx {
@@ -219,62 +211,65 @@ __device__ __forceinline__ void mbar_expect(uint32_t mbar, uint32_t bytes)
 // TF32, to nearest with ties away from zero, by adding half of the last kept
 // bit to the magnitude bits and clearing the rest (the rounding of PTX's
 // cvt.rna.tf32.f32, as integer operations).
-__host__ __device__ inline float tf32_lo(float a)
+__device__ __forceinline__ float tf32_lo(float a)
 {
-#ifdef __CUDA_ARCH__
     const float l = a - __uint_as_float(__float_as_uint(a) & 0xffffe000u);
     return __uint_as_float((__float_as_uint(l) + 0x1000u) & 0xffffe000u);
-#else
-    uint32_t u;
-    std::memcpy(&u, &a, 4);
-    u &= 0xffffe000u;
-    float h;
-    std::memcpy(&h, &u, 4);
-    const float l = a - h;
-    std::memcpy(&u, &l, 4);
-    u = (u + 0x1000u) & 0xffffe000u;
-    float r;
-    std::memcpy(&r, &u, 4);
-    return r;
-#endif
 }
 
-// lo = tf32_lo(a) over n 16-byte chunks, by the `nthr` threads numbered t
-__device__ __forceinline__ void split_lo(const uint8_t *raw, uint8_t *lo, int nchunks, int t, int nthr)
+// lo = tf32_lo(a) over n <= 8 nthr 16-byte chunks, by the nthr threads numbered
+// t: every load ahead of the first store
+__device__ __forceinline__ void split_lo(const uint8_t *raw, uint8_t *lo, int n, int t, int nthr)
 {
-    for (int i = t; i < nchunks; i += nthr) {
-        const float4 a = reinterpret_cast<const float4 *>(raw)[i];
-        float v[4] = {a.x, a.y, a.z, a.w};
+    float4 a[8];
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            v[q] = tf32_lo(v[q]);
-        }
-        reinterpret_cast<float4 *>(lo)[i] = make_float4(v[0], v[1], v[2], v[3]);
-    }
+    for (int r = 0; r < 8; r++)
+        if (t + r * nthr < n) a[r] = reinterpret_cast<const float4 *>(raw)[t + r * nthr];
+#pragma unroll
+    for (int r = 0; r < 8; r++)
+        if (t + r * nthr < n)
+            reinterpret_cast<float4 *>(lo)[t + r * nthr] =
+                make_float4(tf32_lo(a[r].x), tf32_lo(a[r].y), tf32_lo(a[r].z), tf32_lo(a[r].w));
 }
 
 // Persistent and warp-specialised: one CTA per SM walks the tiles t =
 // blockIdx.x, blockIdx.x + gridDim.x, ... (a tile: 128 rows x nt columns of one
 // (m, p) block).  Roles:
-//   warp 0 (one lane)  TMA producer: the K slices of every tile in turn, up to
-//                      `stages` ahead, a stage refilled once the MMAs that read
-//                      it have completed (mma_bar);
-//   warps 1-11         wait for a slice (full_bar), derive the data tile's lo
-//                      part (the table's comes by TMA), meet at a named
-//                      barrier; one of their threads issues the slice's
-//                      MMAs into the tile's accumulator and commits them to the
-//                      stage, and after a tile's last slice to acc_full;
+//   warp 0 (one lane)  TMA producer: the K slices (32 deep) of every tile in
+//                      turn, up to `stages` ahead, a stage refilled once the
+//                      MMAs that read it have completed (mma_bar); of the table
+//                      only the 32-row boxes that hold rows of the tile;
+//   warp 1 (one lane)  waits for a slice's operands (lo_bar), issues its twelve
+//                      MMAs into the tile's accumulator and commits them to
+//                      the stage, and after a tile's last slice to acc_full;
+//   warps 4-7          bring the table slice from shared to tensor memory, a
+//                      thread per row: its 32 values and their low parts;
+//   warps 2, 3, 8-11   derive the data slice's low parts in shared memory;
 //   warps 12-15        epilogue: once a tile's accumulator is complete, each
 //                      reads the 32 rows of its TMEM lane quadrant, scatters
 //                      them into the triangular output and frees the
 //                      accumulator (acc_empty).
-// Two accumulators of 256 columns (all of the SM's tensor memory) alternate
-// between tiles, so a tile's epilogue overlaps the next tile's MMAs.
-// Dynamic shared memory: `stages` x {A raw, A lo, B raw, B lo}, 1024-aligned.
+// Tensor memory: two accumulators that alternate between tiles, so that a
+// tile's epilogue overlaps the next tile's MMAs, and two or three table slots.
+// Dynamic shared memory: `stages` x {table, data, data lo}, 1024-aligned.
+// What bounds it: reads from L2 (the loads alone take 173 us of the 273 at T639 on
+// 137 levels), then shared-memory traffic.  Measured there and at T319 on 91 levels,
+// us without the fold:
+//   low parts of both operands in shared memory, the table's read from a table
+//   of their own, one barrier over eleven warps per slice       350, 83
+//   a role per step, joined by mbarriers alone                  302, 84
+//   table through tensor memory, its low parts derived          328, 80
+//   the output's addresses kept instead of computed per store   280, 48
+//   only the table boxes with rows                              273, 48
+// Neither more split or epilogue warps (292) nor five stages with two low-part
+// buffers (283) is faster, nor tiles of both parities with 8-byte stores (96
+// columns so that four accumulators fit: 408).
 constexpr int kMaxStages = 4;
-constexpr int kConsumers = 352;                 // warps 1-11
+constexpr int kTableWarps = 4, kDataWarps = 6;  // warps 4-7; warps 2, 3, 8-11
 constexpr int kMmaThreads = 512;                // 16 warps
-constexpr int kAccCols = 256;
+constexpr int kBoxRows = 32;                    // rows per TMA copy of the table
+constexpr int kTmemCols = 512;                  // all of the SM's tensor memory
+constexpr int kMaxTile = 192;                   // columns per tile: two accumulators and two table slots fit
 
 // A bounded wait that also gives up once another role has failed.
 __device__ __forceinline__ bool role_wait(uint32_t mbar, uint32_t parity, volatile int *fail)
@@ -289,14 +284,29 @@ __device__ __forceinline__ bool role_wait(uint32_t mbar, uint32_t parity, volati
     return false;
 }
 
+// 32 columns of this warp's 32 tensor-memory lanes
+__device__ __forceinline__ void tmem_store32(uint32_t addr, const uint32_t (&v)[32])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+                 :: "r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
+                 : "memory");
+}
+
+__device__ __forceinline__ void tmem_load16(uint32_t addr, uint32_t (&v)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+                 : "r"(addr));
+}
+
 __global__ void __launch_bounds__(kMmaThreads, 1)
-legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_alo,
-                    const __grid_constant__ CUtensorMap tmap_b,
+legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                     const LegItem *__restrict__ items, LegGeom g, int stages, int ntiles_total,
                     float *__restrict__ are, float *__restrict__ aim, int *__restrict__ status)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[kMaxStages], mma_bar[kMaxStages], acc_full[2], acc_empty[2];
+    __shared__ __align__(8) uint64_t full_bar[kMaxStages], lo_bar[kMaxStages], mma_bar[kMaxStages], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_base;
     __shared__ int fail;
     volatile int *vfail = &fail;
@@ -304,15 +314,18 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
     const int tid = threadIdx.x, warp = tid >> 5;
     const int nt = g.nt;
     const uint32_t a_bytes = kBM * 128, b_bytes = (uint32_t)nt * 128;
-    const uint32_t stage_bytes = 2 * a_bytes + 2 * b_bytes;
+    const uint32_t stage_bytes = a_bytes + 2 * b_bytes;
     auto a_raw = [&](int s) { return smem + s * stage_bytes; };
-    auto a_lo = [&](int s) { return smem + s * stage_bytes + a_bytes; };
-    auto b_raw = [&](int s) { return smem + s * stage_bytes + 2 * a_bytes; };
-    auto b_lo = [&](int s) { return smem + s * stage_bytes + 2 * a_bytes + b_bytes; };
+    auto b_raw = [&](int s) { return smem + s * stage_bytes + a_bytes; };
+    auto b_lo = [&](int s) { return smem + s * stage_bytes + a_bytes + b_bytes; };
+    // tensor memory: two accumulators, then the table slots (32 columns of high,
+    // 32 of low parts: one slice each)
+    const int acc_cols = (nt + 31) / 32 * 32;
+    const int slots = min(stages, (kTmemCols - 2 * acc_cols) / (2 * kBK));
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(smem_u32(&tmem_base)), "n"(2 * kAccCols));
+                     :: "r"(smem_u32(&tmem_base)), "n"(kTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
@@ -320,6 +333,7 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
         for (int s = 0; s < stages; s++) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&full_bar[s])));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&mma_bar[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(&lo_bar[s])), "n"(kTableWarps + kDataWarps));
         }
         for (int a = 0; a < 2; a++) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&acc_full[a])));
@@ -327,7 +341,6 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" :: "l"(&tmap_a) : "memory");
-        asm volatile("prefetch.tensormap [%0];" :: "l"(&tmap_alo) : "memory");
         asm volatile("prefetch.tensormap [%0];" :: "l"(&tmap_b) : "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -343,7 +356,7 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
             for (int t = blockIdx.x; t < ntiles_total && !*vfail; t += gridDim.x) {
                 const LegItem it = items[t / g.ntiles];
                 const int ct = t % g.ntiles;
-                const int arow = (int)(it.arow + it.r0);
+                const int arow = (int)(it.arow + it.r0), abox = (it.nr + kBoxRows - 1) / kBoxRows;
                 const int brow = (int)(((int64_t)it.m * 2 + it.p) * g.ncp + (int64_t)ct * nt);
                 for (int k = 0; k < nk; k++, i++) {
                     const int s = i % stages;
@@ -352,53 +365,47 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                         break;
                     }
                     const uint32_t fb = smem_u32(&full_bar[s]);
-                    mbar_expect(fb, 2 * a_bytes + b_bytes);
-                    tma_load_2d(smem_u32(a_raw(s)), &tmap_a, k * kBK, arow, fb);
-                    tma_load_2d(smem_u32(a_lo(s)), &tmap_alo, k * kBK, arow, fb);
+                    mbar_expect(fb, abox * kBoxRows * 128 + b_bytes);
+                    for (int b = 0; b < abox; b++)
+                        tma_load_2d(smem_u32(a_raw(s) + b * kBoxRows * 128), &tmap_a, k * kBK, arow + b * kBoxRows, fb);
                     tma_load_2d(smem_u32(b_raw(s)), &tmap_b, k * kBK, brow, fb);
                 }
             }
         }
-    } else if (warp <= 11) {
-        // ---- lo tiles and MMAs
-        const int c = tid - 32;
-        const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(nt >> 3) << 17) |
-                               ((uint32_t)(kBM >> 4) << 24);
-        int i = 0, j = 0;                                // slices, tiles of this CTA
-        bool stop = false;
-        for (int t = blockIdx.x; t < ntiles_total && !stop; t += gridDim.x, j++) {
-            const int acc = j & 1;
-            const uint32_t d = tmem + (uint32_t)(acc * kAccCols);
-            // the accumulator's previous tile must have been read out
-            if (tid == 32 && j >= 2 && !role_wait(smem_u32(&acc_empty[acc]), (uint32_t)(j / 2 - 1) & 1u, vfail))
-                *vfail = 1;
-            for (int k = 0; k < nk; k++, i++) {
-                const int s = i % stages;
-                if (!role_wait(smem_u32(&full_bar[s]), (uint32_t)(i / stages) & 1u, vfail)) *vfail = 1;
-                split_lo(b_raw(s), b_lo(s), (int)(b_bytes / 16), c, kConsumers);   // the table's come with it
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                // the named barrier, reducing every consumer's view of the failure
-                // flag so that all of them take the same branch
-                uint32_t any_fail;
-                asm volatile("{\n\t.reg .pred q, r;\n\tsetp.ne.b32 q, %1, 0;\n\t"
-                             "bar.red.or.pred r, 1, %2, q;\n\tselp.u32 %0, 1, 0, r;\n\t}"
-                             : "=r"(any_fail) : "r"((uint32_t)*vfail), "n"(kConsumers) : "memory");
-                if (any_fail) { stop = true; break; }
-                if (tid == 32) {
+    } else if (warp == 1) {
+        // ---- MMAs
+        if (tid == 32) {
+            const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(nt >> 3) << 17) |
+                                   ((uint32_t)(kBM >> 4) << 24);
+            int i = 0, j = 0;                            // slices, tiles of this CTA
+            for (int t = blockIdx.x; t < ntiles_total && !*vfail; t += gridDim.x, j++) {
+                const int acc = j & 1;
+                const uint32_t d = tmem + (uint32_t)(acc * acc_cols);
+                // the accumulator's previous tile must have been read out
+                if (j >= 2 && !role_wait(smem_u32(&acc_empty[acc]), (uint32_t)(j / 2 - 1) & 1u, vfail)) {
+                    *vfail = 1;
+                    break;
+                }
+                for (int k = 0; k < nk; k++, i++) {
+                    const int s = i % stages;
+                    if (!role_wait(smem_u32(&lo_bar[s]), (uint32_t)(i / stages) & 1u, vfail)) {
+                        *vfail = 1;
+                        break;
+                    }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t ah = smem_u32(a_raw(s)), al = smem_u32(a_lo(s));
+                    const uint32_t ah = tmem + (uint32_t)(2 * acc_cols + i % slots * (2 * kBK)), al = ah + kBK;
                     const uint32_t bh = smem_u32(b_raw(s)), bl = smem_u32(b_lo(s));
 #pragma unroll
                     for (int q = 0; q < kBK / 8; q++) {     // 8-deep K steps, 32 bytes apart in the swizzle row
-                        const uint64_t dah = sw128_desc(ah + 32 * q), dal = sw128_desc(al + 32 * q);
                         const uint64_t dbh = sw128_desc(bh + 32 * q), dbl = sw128_desc(bl + 32 * q);
 #pragma unroll
                         for (int e = 0; e < 3; e++) {
-                            const uint64_t da = e == 2 ? dal : dah, db = e == 1 ? dbl : dbh;
+                            const uint32_t a = (e == 2 ? al : ah) + 8 * q;
+                            const uint64_t db = e == 1 ? dbl : dbh;
                             const uint32_t accum = (k > 0 || q > 0 || e > 0) ? 1u : 0u;
                             asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                                         "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-                                         :: "r"(d), "l"(da), "l"(db), "r"(idesc), "r"(accum));
+                                         "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}"
+                                         :: "r"(d), "r"(a), "l"(db), "r"(idesc), "r"(accum));
                         }
                     }
                     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
@@ -409,6 +416,57 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                 }
             }
         }
+    } else if (warp >= 4 && warp <= 7) {
+        // ---- table slices to tensor memory: a thread per row, its 32 values and
+        // their low parts; warp 4 + q reaches the lanes (rows) 32 q .. 32 q + 31
+        const int row = 32 * (warp - 4) + (tid & 31);
+        const uint32_t lanes = (uint32_t)(32 * (warp - 4)) << 16;
+        int i = 0;
+        bool stop = false;
+        for (int t = blockIdx.x; t < ntiles_total && !stop; t += gridDim.x)
+            for (int k = 0, live = 32 * (warp - 4) < items[t / g.ntiles].nr; k < nk; k++, i++) {
+                const int s = i % stages, f = i - slots;     // f: the slice whose slot this one takes
+                bool got = role_wait(smem_u32(&full_bar[s]), (uint32_t)(i / stages) & 1u, vfail);
+                if (got && f >= 0)
+                    got = role_wait(smem_u32(&mma_bar[f % stages]), (uint32_t)(f / stages) & 1u, vfail);
+                if (!__all_sync(0xffffffffu, got)) { *vfail = 1; stop = true; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (live) {
+                    const uint8_t *a = a_raw(s) + row * 128;
+                    uint32_t v[kBK];
+#pragma unroll
+                    for (int ch = 0; ch < 8; ch++) {             // 16-byte chunk ch of a swizzled row
+                        const uint4 x = *reinterpret_cast<const uint4 *>(a + 16 * (ch ^ (row & 7)));
+                        v[4 * ch] = x.x; v[4 * ch + 1] = x.y; v[4 * ch + 2] = x.z; v[4 * ch + 3] = x.w;
+                    }
+                    const uint32_t slot = tmem + lanes + (uint32_t)(2 * acc_cols + i % slots * (2 * kBK));
+                    tmem_store32(slot, v);
+#pragma unroll
+                    for (int e = 0; e < kBK; e++) v[e] = __float_as_uint(tf32_lo(__uint_as_float(v[e])));
+                    tmem_store32(slot + kBK, v);
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if ((tid & 31) == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&lo_bar[s])) : "memory");
+            }
+    } else if (warp <= 11) {
+        // ---- low parts of the data
+        const int c = tid - (warp < 4 ? 64 : 192);
+        int i = 0;
+        bool stop = false;
+        for (int t = blockIdx.x; t < ntiles_total && !stop; t += gridDim.x)
+            for (int k = 0; k < nk; k++, i++) {
+                const int s = i % stages;
+                const bool got = role_wait(smem_u32(&full_bar[s]), (uint32_t)(i / stages) & 1u, vfail);
+                if (!__all_sync(0xffffffffu, got)) { *vfail = 1; stop = true; break; }
+                split_lo(b_raw(s), b_lo(s), (int)(b_bytes / 16), c, 32 * kDataWarps);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if ((tid & 31) == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&lo_bar[s])) : "memory");
+            }
     } else {
         // ---- epilogue: warp 12 + q reads TMEM lanes 32 q .. 32 q + 31 (its warp
         // index mod 4 is q, the lane quadrant tcgen05.ld lets it reach)
@@ -423,24 +481,20 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
             const int ct = t % g.ntiles;
             const int row = 32 * q + lane;
             const bool live = row < it.nr;
+            // the row's output column c is at base[part] + c os, part 1 from column nlev on
             const int64_t o = tri_offset(it.m, g.T) + it.p + 2 * (int64_t)(it.r0 + row);
+            float *const base0 = are + o, *const base1 = aim + o - g.nlev * g.os;
+            const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * acc_cols);
             for (int c0 = 0; c0 < nt; c0 += 16) {
                 uint32_t v[16];
-                const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * kAccCols + c0);
-                asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                             : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                               "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                             : "r"(taddr));
+                tmem_load16(taddr + c0, v);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                const int c = ct * nt + c0;
+                int64_t off = (int64_t)c * g.os;
                 if (live) {
 #pragma unroll
-                    for (int e = 0; e < 16; e++) {
-                        const int col = ct * nt + c0 + e;
-                        if (col < g.N) {
-                            const int part = col >= g.nlev, lev = part ? col - g.nlev : col;
-                            (part ? aim : are)[(int64_t)lev * g.os + o] = __uint_as_float(v[e]);
-                        }
-                    }
+                    for (int e = 0; e < 16; e++, off += g.os)
+                        if (c + e < g.N) (c + e < g.nlev ? base0 : base1)[off] = __uint_as_float(v[e]);
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -460,7 +514,7 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(2 * kAccCols));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(kTmemCols));
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
@@ -494,15 +548,14 @@ int make_tmap(CUtensorMap *map, const float *base, int64_t k, int64_t rows, int6
     return r == CUDA_SUCCESS ? ZFPX_OK : ZFPX_ECUDA;
 }
 
-// columns per tile for N = 2 nlev columns: the fewest tiles of at most 256
-// columns, each a multiple of 16
+// the workspace's columns per (m, p) for N = 2 nlev columns, as nt * ntiles
 void column_tiles(int N, int &nt, int &ntiles)
 {
     ntiles = (N + 255) / 256;
     nt = ((N + ntiles - 1) / ntiles + 15) / 16 * 16;
 }
 
-size_t stage_bytes(int nt) { return 2 * kBM * 128 + 2 * (size_t)nt * 128; }
+size_t stage_bytes(int nt) { return kBM * 128 + 2 * (size_t)nt * 128; }
 
 // as many stages (2 .. 4) as fit beside one CTA's static shared memory
 int mma_stages(int nt)
@@ -571,7 +624,7 @@ int legendre_create(zfpx_legendre *out, int nlat, int T)
     for (int m = 0; m <= T; m++)
         for (int par = 0; par < 2; par++) rows += (T - m - par) >= 0 ? (T - m - par) / 2 + 1 : 0;
     p->table_rows = rows;
-    // the two tables (high and low TF32 parts) must fit on the device
+    // a table of more than half the device's memory is refused
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return ZFPX_ECUDA;
     if ((double)std::max<int64_t>(rows, 1) * nhs * 2 * sizeof(float) > (double)total_b) return ZFPX_ENOMEM;
@@ -610,20 +663,14 @@ int legendre_create(zfpx_legendre *out, int nlat, int T)
         }
     }
     p->nitems = (int)items.size();
-    std::vector<float> tab_lo(tab.size());
-    for (size_t i = 0; i < tab.size(); i++) tab_lo[i] = tf32_lo(tab[i]);
     if (cudaMalloc(&p->d_table, tab.size() * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&p->d_table_lo, tab.size() * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&p->d_items, std::max<size_t>(items.size(), 1) * sizeof(LegItem)) != cudaSuccess ||
         cudaMalloc(&p->d_status, sizeof(int)) != cudaSuccess ||
         cudaMemcpy(p->d_table, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(p->d_table_lo, tab_lo.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(p->d_items, items.data(), items.size() * sizeof(LegItem), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(p->d_status, 0, sizeof(int)) != cudaSuccess ||
-        make_tmap(&p->tmap_table, p->d_table, nh, std::max<int64_t>(rows, 1), nhs, kBM) != ZFPX_OK ||
-        make_tmap(&p->tmap_table_lo, p->d_table_lo, nh, std::max<int64_t>(rows, 1), nhs, kBM) != ZFPX_OK) {
+        make_tmap(&p->tmap_table, p->d_table, nh, std::max<int64_t>(rows, 1), nhs, kBoxRows) != ZFPX_OK) {
         cudaFree(p->d_table);
-        cudaFree(p->d_table_lo);
         cudaFree(p->d_items);
         cudaFree(p->d_status);
         return ZFPX_ECUDA;
@@ -663,7 +710,6 @@ void zfpx_legendre_destroy(zfpx_legendre p)
 {
     if (!p) return;
     cudaFree(p->d_table);
-    cudaFree(p->d_table_lo);
     cudaFree(p->d_items);
     cudaFree(p->d_status);
     delete p;
@@ -705,6 +751,8 @@ int zfpx_legendre_forward(zfpx_legendre p, const float *d_re, const float *d_im,
     g.N = 2 * g.nlev;
     column_tiles(g.N, g.nt, g.ntiles);
     g.ncp = g.nt * g.ntiles;
+    g.ntiles = (g.N + kMaxTile - 1) / kMaxTile;
+    g.nt = ((g.N + g.ntiles - 1) / g.ntiles + 15) / 16 * 16;
     g.is1 = stride[1]; g.is2 = stride[2]; g.os = out_stride;
     const int64_t grows = (int64_t)(p->T + 1) * 2 * g.ncp;
     if (grows > 0x7fffffff || p->table_rows > 0x7fffffff) return ZFPX_EINVAL;
@@ -732,7 +780,7 @@ int zfpx_legendre_forward(zfpx_legendre p, const float *d_re, const float *d_im,
     if (cudaFuncSetAttribute(legendre_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return ZFPX_ECUDA;
     const int grid = (int)std::min<int64_t>(nblk, num_sms());      // persistent: one CTA per SM
-    legendre_mma_kernel<<<grid, kMmaThreads, smem, st>>>(p->tmap_table, p->tmap_table_lo, tmap_g, p->d_items, g,
+    legendre_mma_kernel<<<grid, kMmaThreads, smem, st>>>(p->tmap_table, tmap_g, p->d_items, g,
                                                           mma_stages(g.nt), (int)nblk,
                                                           d_are, d_aim, p->d_status);
     count_launch();
