@@ -28,6 +28,7 @@
 #include "zfpx_smem.cuh"
 #include "zfpx_enc3.cuh"
 #include "zfpx_enc2.cuh"
+#include "zfpx_warp3.cuh"
 
 namespace zfpx {
 namespace {
@@ -411,6 +412,68 @@ decode3_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchG
     }
 }
 
+// A warp per block (zfpx_warp3.cuh): warp w of a unit's 32 codes its block w.
+// Values move one by one, two a lane, in the block's order.
+struct WarpBlock {
+    int64_t boff;             // the block's message in the stream buffer
+    int b, nx, ny, nz;        // block, and the values it holds along each axis
+    int64_t view;             // its first value in the view
+    __device__ __forceinline__ bool find(const LaunchGeom &g, const int64_t *s, int64_t view_off(const MsgDev &), int layout, int wid)
+    {
+        const int64_t c = blockIdx.x / (32 / kWarps);
+        MsgWalk walk;
+        walk.start(g.msgs, g.nmsg, c);
+        const MsgDev &m = g.msgs[walk.mi];
+        const int64_t q = (c - m.unit0) * 32 + blockIdx.x % (32 / kWarps) * kWarps + wid;
+        if (q >= m.nblocks) return false;
+        b = (int)q;
+        boff = layout ? m.off[1] : m.off[0];
+        const int t = (int)divu((uint32_t)b, m.bxm, m.bxl), z = (int)divu((uint32_t)t, m.bym, m.byl);
+        const int x0 = 4 * (b - t * m.bx), y0 = 4 * (t - z * m.by), z0 = 4 * z;
+        nx = m.nx - x0; ny = m.ny - y0; nz = m.nz - z0;
+        view = view_off(m) + (int64_t)z0 * s[2] + (int64_t)y0 * s[1] + (int64_t)x0 * s[0];
+        return true;
+    }
+};
+
+template <int RATE>
+__global__ void __launch_bounds__(kThreads)
+encode3_warp_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchGeom g, int layout)
+{
+    __shared__ warp3::Shared<RATE> sh[kWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    WarpBlock k;
+    if (!k.find(g, g.ss, [](const MsgDev &m) { return m.src_off; }, layout, wid)) return;
+    // rows past the end of the box repeat its last row, values its last value
+    const float *p = src + k.view + (int64_t)min(lane & 3, k.nx - 1) * g.ss[0] +
+                     (int64_t)min((lane >> 2) & 3, k.ny - 1) * g.ss[1];
+    const float x0 = __ldg(p + (int64_t)min(lane >> 4, k.nz - 1) * g.ss[2]);
+    const float x1 = __ldg(p + (int64_t)min((lane >> 4) + 2, k.nz - 1) * g.ss[2]);
+    warp3::encode<RATE>(x0, x1, sh[wid], lane);
+    if (lane < 2 * RATE)
+        reinterpret_cast<uint32_t *>(out + k.boff)[(int64_t)k.b * 2 * RATE + lane] = sh[wid].stream[lane];
+}
+
+template <int RATE>
+__global__ void __launch_bounds__(kThreads)
+decode3_warp_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchGeom g, int layout)
+{
+    __shared__ warp3::Shared<RATE> sh[kWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    WarpBlock k;
+    if (!k.find(g, g.ds, [](const MsgDev &m) { return m.dst_off; }, layout, wid)) return;
+    uint32_t *w = sh[wid].stream;
+    if (lane < 2 * RATE) w[lane] = __ldg(reinterpret_cast<const uint32_t *>(in + k.boff) + (int64_t)k.b * 2 * RATE + lane);
+    if (lane < 4) w[2 * RATE + lane] = 0u;
+    __syncwarp();
+    float x0, x1;
+    warp3::decode<RATE>(x0, x1, sh[wid], lane);
+    if ((lane & 3) >= k.nx || ((lane >> 2) & 3) >= k.ny) return;
+    float *p = dstf + k.view + (int64_t)(lane & 3) * g.ds[0] + (int64_t)((lane >> 2) & 3) * g.ds[1];
+    if ((lane >> 4) < k.nz) p[(int64_t)(lane >> 4) * g.ds[2]] = x0;
+    if ((lane >> 4) + 2 < k.nz) p[(int64_t)((lane >> 4) + 2) * g.ds[2]] = x1;
+}
+
 // ================================================================= 1-D kernels
 // Blocks of 4 values along x; a block is 4r bits (32 or 64), kept in one
 // register and moved with one coalesced 4- or 8-byte access per lane.  A lane
@@ -695,6 +758,20 @@ void launch3(void (*kernel)(In, Out, LaunchGeom, int, Acc), int warps, int encod
     kernel<<<(unsigned)grid, 32 * warps, 0, st>>>(in, out, g, layout, acc);
 }
 
+// A warp per block (zfpx_warp3.cuh) where that leaves an SM no more than 14 warps,
+// unless the units per warp were set.  Up to there a launch's time is one
+// warp's: 256 blocks at rate 8 / 16 compress in 6.2 / 6.2 us where a lane per block takes
+// 8.2 / 9.2, decompress in 8.2 / 8.2 against 10.3 / 12.3; 2048 blocks 6.2 / 6.2 against
+// 8.2 / 10.3 and 8.2 / 10.3 against 10.3 / 12.3.  Beyond, the eight times as many
+// instructions show: 4000 blocks 8.2 / 8.2 and 12.1 / 12.3 us (the same as a lane per
+// block, or more), 8192 blocks 11.1 / 11.3 and 16.4 / 18.5 against 8.2 / 10.3 and 10.3 / 12.3.
+constexpr int kWarpPerBlockPerSm = 14;
+bool warp_per_block(int encode, int rate, int64_t nunits)
+{
+    return g_upw[encode ? 1 : 0][rate == 16 ? 1 : 0].load(std::memory_order_relaxed) <= 0 &&
+           nunits * 32 <= (int64_t)kWarpPerBlockPerSm * num_sms();
+}
+
 // vec: rows start on 16 bytes wherever a block starts (x0 multiple of 4).
 bool vec_ok(const void *ptr, const int64_t s[3], const zfpx_plan_s *p, int which /*0 src,1 dst*/)
 {
@@ -713,7 +790,11 @@ int launch_encode(int dims, int rate, const float *src, uint8_t *out, const Laun
                   cudaStream_t st)
 {
     if (g.nunits == 0) return ZFPX_OK;
-    if (dims == 3) {
+    if (dims == 3 && warp_per_block(1, rate, g.nunits)) {
+        const unsigned grid = (unsigned)g.nunits * (32 / kWarps);
+        if (rate == 8) encode3_warp_kernel<8><<<grid, kThreads, 0, st>>>(src, out, g, layout);
+        else encode3_warp_kernel<16><<<grid, kThreads, 0, st>>>(src, out, g, layout);
+    } else if (dims == 3) {
         if (rate == 8)
             launch3(vec ? encode3_kernel<8, true, false> : encode3_kernel<8, false, false>, kEnc3Warps<8>, 1, 8, g, st, src, out,
                     layout);
@@ -735,7 +816,11 @@ int launch_decode(int dims, int rate, const uint8_t *in, float *dst, const Launc
                   cudaStream_t st)
 {
     if (g.nunits == 0) return ZFPX_OK;
-    if (dims == 3) {
+    if (dims == 3 && warp_per_block(0, rate, g.nunits)) {
+        const unsigned grid = (unsigned)g.nunits * (32 / kWarps);
+        if (rate == 8) decode3_warp_kernel<8><<<grid, kThreads, 0, st>>>(in, dst, g, layout);
+        else decode3_warp_kernel<16><<<grid, kThreads, 0, st>>>(in, dst, g, layout);
+    } else if (dims == 3) {
         if (rate == 8)
             launch3(vec ? decode3_kernel<8, true, false> : decode3_kernel<8, false, false>, kDec3Warps<8>, 0, 8, g, st, in, dst,
                     layout);

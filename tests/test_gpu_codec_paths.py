@@ -10,6 +10,19 @@ from paper_2609_24294_gb300 import zfpx as z
 pytestmark = pytest.mark.gpu
 
 
+# the 3-D codec by the library's choice (in small launches a warp per block) and
+# always with a lane per block
+@pytest.fixture(autouse=True, params=["chosen", "lane"])
+def path(request):
+    for encode in (0, 1):
+        for rate in (8, 16):
+            z.zfpx_set_units_per_warp(encode, rate, 1 if request.param == "lane" else 0)
+    yield request.param
+    for encode in (0, 1):
+        for rate in (8, 16):
+            z.zfpx_set_units_per_warp(encode, rate, 0)
+
+
 def round_trip(x, dims, rate):
     """Stream bytes and decoded values of x ([lev][lat][lon]) equal the oracle's."""
     n = tuple(reversed(x.shape))
@@ -330,3 +343,43 @@ def test_captured_accuracy_chain(shape):
     for a, b in zip(want, got):
         assert all(torch.equal(i.view(torch.uint8), j.view(torch.uint8)) for i, j in zip(a, b))
     assert torch.equal(dw.view(torch.int32), dg.view(torch.int32))
+
+
+# special blocks, partial along every axis, in views with any strides; one more
+# unit than a warp per block takes
+@pytest.mark.parametrize("shape", [(1, 1, 1), (3, 2, 5), (9, 7, 13), (5, 6, 66)])
+@pytest.mark.parametrize("rate", [8, 16])
+def test_small_arrays_of_any_layout(shape, rate):
+    r = np.random.default_rng(rate + sum(shape))
+    x = (r.standard_normal(shape) * 10.0 ** r.integers(-44, 38, shape)).astype(np.float32)
+    x[r.random(shape) < 0.1] = 0.0
+    x[r.random(shape) < 0.01] = np.inf
+    x[r.random(shape) < 0.01] = np.nan
+    x[r.random(shape) < 0.05] = np.float32(3.4e38)
+    n = tuple(reversed(shape))
+    ref = oc.encode_array(3, rate, x)
+    rd = np.empty_like(x)
+    oc.decode_array(3, rate, ref, rd)
+    for order, step in (((0, 1, 2), 1), ((2, 1, 0), 1), ((1, 2, 0), 1), ((0, 1, 2), 3)):
+        def view(a):                                   # the values in another memory order, `step` apart
+            big = torch.full([shape[i] * (step if k == 2 else 1) for k, i in enumerate(order)], 7.0, device="cuda")
+            v = big[..., ::step].permute(*[order.index(i) for i in range(3)])
+            v.copy_(torch.from_numpy(a))
+            return big, v
+        _, src = view(x)
+        big, dst = view(np.zeros_like(x))
+        s = torch.zeros(z.zfpx_stream_bytes(3, rate, n), dtype=torch.uint8, device="cuda")
+        z.zfpx_encode(3, rate, src, s)
+        z.zfpx_decode(3, rate, s, dst)
+        assert s.cpu().numpy().tobytes() == bytes(ref)
+        assert np.array_equal(dst.cpu().numpy().view(np.uint32), rd.view(np.uint32))
+        if step > 1:
+            assert bool((big.view(-1, step)[:, 1:] == 7.0).all())
+
+
+@pytest.mark.parametrize("rate", [8, 16])
+def test_either_side_of_a_warp_per_block(rate):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for units in (14 * sms // 32, 14 * sms // 32 + 1):
+        x = np.random.default_rng(units).standard_normal((4, 4 * units, 4 * 32)).astype(np.float32)
+        round_trip(x, 3, rate)
