@@ -174,8 +174,10 @@ def _check(rc, what):
 
 
 def _stream(stream):
+    # the current stream's handle without a Stream object around it: a call on a
+    # small field takes 5.4 us of the host, 9.4 with one
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return ctypes.c_void_p(stream.cuda_stream)
 
 
@@ -272,6 +274,8 @@ class Plan:
         return int(lib().zfpx_buffer_bytes(self.handle, rate))
 
     def _check_field(self, t, strides, what):
+        if t.dtype is torch.float32 and t.shape == self.n[::-1] and t.stride() == strides[::-1]:
+            return
         if t.dtype != torch.float32:
             raise ValueError("%s must be float32" % what)
         n, s = field_view(t)
