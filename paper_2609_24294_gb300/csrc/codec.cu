@@ -9,16 +9,18 @@
 //   x, y, z; coefficients in total-sequency order; negabinary; group-tested
 //   bit planes from 31 down, cut at exactly 4^d r bits.
 //
-// Mapping to the GPU: one lane owns one block.  A warp takes 32 consecutive
-// blocks of one message, so its compressed output (or input) is one
-// contiguous run of 32 * 8r bytes, staged through shared memory in a
-// [word][lane] layout (XOR-swizzled) and moved with coalesced 8-byte
-// accesses.  The 64 coefficients of a block live in registers; their 32 bit
-// planes are formed with two in-register 32x32 bit-matrix transposes
-// (byte permutes for the 16- and 8-bit stages, masked shifts below), after
-// which each plane is one 64-bit word and group testing is a find-first-set
-// per newly significant coefficient.  Each warp processes a contiguous range
-// of 32-block chunks, so the message lookup is a forward scan.
+// Mapping to the GPU: one lane owns one block (a warp owns one in the smallest
+// 3-D launches).  A warp takes 32 consecutive blocks of one message, so its
+// compressed output (or input) is one contiguous run of 32 * 8r bytes; each
+// lane moves its own stream with 16-byte accesses and keeps it in its own
+// column of a [word][lane] tile of shared memory.  The 64 coefficients of a
+// block live in registers; their 32 bit planes are formed with two in-register
+// 32x32 bit-matrix transposes (byte permutes for the 16- and 8-bit stages,
+// masked shifts below), after which each plane is one 64-bit word; the
+// encoder writes its group-tested part eight coefficients at a time through a
+// table (zfpx_enc3.cuh), the decoder reads it in 32-bit windows
+// (parse_planes64).  Each warp processes a contiguous range of 32-block
+// chunks, so the message lookup is a forward scan.
 #include <atomic>
 #include <climits>
 #include <cuda_runtime.h>

@@ -14,8 +14,9 @@
 // The functions are __host__ __device__ so the same block code serves the
 // kernels and can be compiled for a CPU.  On the GPU the 64 coefficients of a
 // 3-D block sit in registers, their 32 bit planes are built with two 32x32
-// bit-matrix transposes, and group testing is one find-first-set per newly
-// significant coefficient.
+// bit-matrix transposes.  The kernels decode with decode_block*_tile and the 1-D
+// functions of this file and encode 2-D and 3-D blocks with zfpx_enc2.cuh and
+// zfpx_enc3.cuh.
 #pragma once
 
 #include <cstdint>
@@ -447,7 +448,9 @@ ZFPX_HD uint64_t decode_plane(Reader &rd, int &n, int &R)
 }
 
 // ----------------------------------------------------------------- 3-D block
-// Encodes 64 values (x[i + 4j + 16k]) into exactly 64 RATE bits.
+// Encodes 64 values (x[i + 4j + 16k]) into exactly 64 RATE bits.  (The plain
+// statement of the stream, which the CPU tests compile; the kernels' encoder is
+// enc3::encode.)
 //
 // Two passes over the bit planes, so that lanes coding different blocks do
 // not diverge per plane.  Pass 1 walks the planes with closed forms: plane k

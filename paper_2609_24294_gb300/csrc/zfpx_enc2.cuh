@@ -15,7 +15,7 @@
 // every coefficient is significant the remaining planes go out verbatim, two
 // per word.
 //
-// What bounds it: instruction issue (issue slots 72 % busy, ALU pipe 70 %).  1940
+// What bounds it: instruction issue (issue slots 73 % busy, ALU pipe 72 %).  1800
 // warp instructions per 32 blocks at rate 16, where one step per newly
 // significant coefficient in a second pass, a 64-bit bit writer and a 32 x 32
 // transpose took 2875; compressing a 1280 x 640 x 37 field level by level over 4

@@ -38,14 +38,14 @@
 // most steps of any lane (about 22).
 //
 // What bounds it: instruction issue, half of it on the ALU pipe (ncu: issue
-// slots 58 % busy, ALU pipe 60 %, 16 to 18 warps per SM), and the latency of
+// slots 63-68 % busy, ALU pipe 67-73 %, 15 to 17 warps per SM), and the latency of
 // the gather.  Per 32 blocks at rate 8 about 3500 warp instructions: gather and
 // store 270, block maximum and quantisation 210, lifting 610, planes 440, the
 // coder the rest.  With one new coefficient per step instead of eight
 // through the table, each plane's part finished in a second pass, and the block
 // maximum by integer compares it was 4200; compressing a 1280 x 640 x 137
-// field over 8 x 8 ranks took 336 us at rate 8 and 420 us at rate 16 then, 286
-// and 357 us now.
+// field over 8 x 8 ranks took 336 us at rate 8 and 420 us at rate 16 then, 274
+// and 348 us now.
 //
 // How the lanes are kept together: phase A is one straight run of instructions
 // per plane (a lane without new ones codes zeros), each lane leaving it when
