@@ -531,9 +531,13 @@ int64_t plan_blocks(const zfpx_plan_s *p, std::vector<AccMsg> *msgs, std::vector
 size_t plan_acc_bytes(const zfpx_plan_s *p, int64_t G)
 {
     const size_t M = p->msgs.size();
+    // 40 bytes a message and three words where the tables below take 32 and two:
+    // the size stays what saved callers hold
     return align256((size_t)buffer_bytes(p, 16)) + acc_work_bytes(G) - align256((size_t)G * 128) +
-           align256(M * sizeof(AccMsg)) + align256(M * 4) + 2 * align256(M * 8);
+           align256(M * 40) + align256(M * 4) + 3 * align256(M * 8);
 }
+
+static_assert(sizeof(AccMsg) <= 40, "the scratch holds the message table");
 
 // Carves the scratch and uploads the message tables (pageable copies: the
 // host vectors have been read when the call returns).
