@@ -87,6 +87,23 @@ __device__ __forceinline__ uint32_t divu(uint32_t n, uint32_t m, int32_t l)
     const uint32_t t = __umulhi(n, m);
     return l ? (t + ((n - t) >> 1)) >> (l - 1) : n;
 }
+// The last message whose units start at or before u, by the whole warp: every
+// round the lanes look at 32 messages spread over the range that is left, so 512
+// messages take two rounds of loads where halving takes nine, each waiting for
+// the one before at the start of every warp.
+__device__ __forceinline__ int find_msg(const MsgDev *msgs, int nmsg, int64_t u)
+{
+    const int lane = threadIdx.x & 31;
+    int lo = 0, n = nmsg;
+    while (n > 1) {
+        const int step = (n + 31) >> 5;
+        const bool before = lane * step < n && msgs[lo + lane * step].unit0 <= u;
+        const int k = __popc(__ballot_sync(0xffffffffu, before)) - 1;    // msgs[lo] starts at or before u
+        lo += k * step;
+        n = min(step, n - k * step);
+    }
+    return lo;
+}
 #endif
 
 // Arguments common to every plan-driven launch.

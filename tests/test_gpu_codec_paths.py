@@ -5,6 +5,8 @@ import pytest
 import torch
 
 from oracle import codec as oc
+from oracle import packs as op
+from oracle import plan as opl
 from paper_2609_24294_gb300 import zfpx as z
 
 pytestmark = pytest.mark.gpu
@@ -383,3 +385,19 @@ def test_either_side_of_a_warp_per_block(rate):
     for units in (14 * sms // 32, 14 * sms // 32 + 1):
         x = np.random.default_rng(units).standard_normal((4, 4 * units, 4 * 32)).astype(np.float32)
         round_trip(x, 3, rate)
+
+
+# messages shorter than the 2 KB a warp moves at a time, longer, ending inside
+# it and inside 16 bytes, and empty ones (more ranks than values)
+@pytest.mark.parametrize("n,pr,pc", [((64, 32, 8), 2, 2), ((33, 17, 5), 3, 2), ((130, 67, 21), 2, 3), ((7, 3, 2), 4, 5)])
+@pytest.mark.parametrize("rate", [8, 16, z.RATE_F32, z.RATE_F16])
+def test_permute_of_any_message_size(n, pr, pc, rate):
+    for dims in (1, 3):
+        plan = z.Plan(n, pr, pc, 0, dims)
+        r = np.random.default_rng(sum(n))
+        s = r.integers(0, 256, plan.buffer_bytes(rate), dtype=np.uint8)
+        recv = torch.zeros(plan.buffer_bytes(rate), dtype=torch.uint8, device="cuda")
+        z.zfpx_permute(plan, rate, torch.from_numpy(s).cuda(), recv)
+        want = np.frombuffer(op.permute(opl.Plan(*n, pr, pc, 0, dims), rate, s), np.uint8)
+        assert np.array_equal(recv.cpu().numpy(), want)
+        plan.close()
