@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 3) rfft_lon_kernel(const float
         load_row_async(buf, src, H, lane);
         wait_rows();
         __syncwarp();
-        rfft_row(buf, buf + H, tw, g, lane, re + z * g.os2 + y * g.os1, im + z * g.os2 + y * g.os1);
+        rfft_row<true>(buf, buf + H, tw, g, lane, re + z * g.os2 + y * g.os1, im + z * g.os2 + y * g.os1);
     }
 }
 
@@ -68,7 +68,7 @@ rfft_lon64_kernel(const float *__restrict__ in, float *__restrict__ re, float *_
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int64_t gr = (int64_t)blockIdx.x * kRow64Warps + wid; gr < g.nrows; gr += (int64_t)gridDim.x * kRow64Warps) {
         const int64_t y = gr % g.ny, z = gr / g.ny;
-        rfft_row64<R1>(reinterpret_cast<const float2 *>(in + z * g.is2 + y * g.is1), buf[wid], tw, tw + g.N, g.K, lane,
+        rfft_row64<R1, true>(reinterpret_cast<const float2 *>(in + z * g.is2 + y * g.is1), buf[wid], tw, tw + g.N, g.K, lane,
                        re + z * g.os2 + y * g.os1, im + z * g.os2 + y * g.os1);
     }
 }

@@ -51,7 +51,7 @@ template <int R1>
 __device__ __noinline__ void row64_call(const float2 *src, float2 *buf, const float2 *__restrict__ tw,
                                         const float2 *__restrict__ tw2, int K, int lane, float *ore, float *oim)
 {
-    fft::rfft_row64<R1>(src, buf, tw, tw2, K, lane, ore, oim);
+    fft::rfft_row64<R1, false>(src, buf, tw, tw2, K, lane, ore, oim);
 }
 
 template <int RATE>
@@ -131,7 +131,7 @@ decode_rfft_kernel(const uint8_t *__restrict__ in, const FusedMsg *__restrict__ 
                 fft::load_row_async(X, src, fg.H, lane);
                 fft::wait_rows();
                 __syncwarp();
-                fft::rfft_row(X, Y, tw, fg, lane, re + o, im + o);
+                fft::rfft_row<false>(X, Y, tw, fg, lane, re + o, im + o);
             }
         }
         __syncthreads();
