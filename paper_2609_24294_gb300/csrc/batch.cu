@@ -353,7 +353,8 @@ batch_encode_kernel(BatchGeom bg, uint8_t *__restrict__ out)
 
 template <int RATE>
 __device__ __forceinline__ void dec3_lane(const FieldDevB &f, const GridDev &g, const ItemDevB &it, int64_t b,
-                                          int start, int lane, const uint8_t *in, uint32_t *t32, uint64_t *wpl)
+                                          int start, int lane, const uint8_t *in, uint32_t *t32, uint64_t *wpl,
+                                          const DropTable &drop)
 {
     const uint4 *src4 = reinterpret_cast<const uint4 *>(in + it.out_off) + b * (RATE / 2);
 #pragma unroll
@@ -370,7 +371,7 @@ __device__ __forceinline__ void dec3_lane(const FieldDevB &f, const GridDev &g, 
     const int q = upper_index_from(g.qpre, g.nq + 1, start, bg);
     const int bxi = (int)(bg - __ldg(g.qpre + q));
     float x[64];
-    const StreamTile tile{t32, lane};
+    const WithDrop<StreamTile> tile(StreamTile{t32, lane}, drop);
     SmemPlanes pl{wpl, lane};
     decode_block3_tile<RATE>(tile, x, pl);
     scatter_quad(f, g, q, bxi, it.z0, it.nz, x);
@@ -423,7 +424,10 @@ batch_decode_kernel(BatchGeom bg, const uint8_t *__restrict__ in)
     __shared__ uint32_t stile[WARPS][(2 * 16 + 2) * 32];
     __shared__ uint64_t splanes[WARPS][32 * 32];
     __shared__ Plane4Dec tab;
+    __shared__ DropTable drop;
     fill_plane4(bg, tab);
+    load_drop<32 * WARPS>(drop);
+    __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for_each_unit(bg, lane, [&](const GroupDev &G, int64_t c, int ii) {
         const ItemDevB it = bg.items[ii];
@@ -433,8 +437,8 @@ batch_decode_kernel(BatchGeom bg, const uint8_t *__restrict__ in)
             const int nact = (int)min((int64_t)32, it.nblocks - b0);
             if (lane < nact) {
                 const int start = upper_index(bg.grid.qpre, bg.grid.nq + 1, b0 + f.b0);
-                if (G.rate == 8) dec3_lane<8>(f, bg.grid, it, b0 + lane, start, lane, in, stile[wid], splanes[wid]);
-                else dec3_lane<16>(f, bg.grid, it, b0 + lane, start, lane, in, stile[wid], splanes[wid]);
+                if (G.rate == 8) dec3_lane<8>(f, bg.grid, it, b0 + lane, start, lane, in, stile[wid], splanes[wid], drop);
+                else dec3_lane<16>(f, bg.grid, it, b0 + lane, start, lane, in, stile[wid], splanes[wid], drop);
             }
         } else {
             const int64_t b0 = (c - it.unit0) * 32 * bg.lb1;

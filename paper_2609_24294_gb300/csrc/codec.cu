@@ -329,13 +329,16 @@ decode3_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchG
 {
     __shared__ uint32_t stile[kDec3Warps<RATE>][(2 * RATE + kTileZeroRows<RATE>) * 32];
     __shared__ uint64_t splanes[kDec3Warps<RATE>][32 * 32];
+    __shared__ DropTable drop;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t *t32 = stile[wid];
     SmemPlanes pl{splanes[wid], lane};
-    const StreamTile tile{t32, lane};
+    const WithDrop<StreamTile> tile(StreamTile{t32, lane}, drop);
+    load_drop<32 * kDec3Warps<RATE>>(drop);
 #pragma unroll
     for (int r = 0; r < kTileZeroRows<RATE>; r++) t32[(2 * RATE + r) * 32 + lane] = 0u;
     const UnitRange ur(g, kDec3Warps<RATE>, wid);
+    __syncthreads();
     if (ur.c >= ur.c1) return;
     MsgWalk walk;
     walk.start(g.msgs, g.nmsg, ur.c);
@@ -649,7 +652,10 @@ decode2_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchG
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t *t32 = stile[wid];
     SmemPlanes16 pl{splanes[wid], lane};
-    const StreamTile tile{t32, lane};
+    __shared__ DropTable drop;
+    const WithDrop<StreamTile> tile(StreamTile{t32, lane}, drop);
+    load_drop<kThreads>(drop);
+    __syncthreads();
     t32[NW * 32 + lane] = 0u;                 // a zero word after the stream
     const int64_t W = (int64_t)gridDim.x * kWarps;
     const int64_t gw = (int64_t)blockIdx.x * kWarps + wid;

@@ -21,7 +21,7 @@
 // memory), and the int64 arithmetic.  With all four transposes, a per-lane coder
 // that wrote bit by bit through 64-bit words and 64-bit index divisions, a 640 x
 // 320 x 91 field took 175 / 153 us to encode / decode at rate 8, 207 / 182 at 16
-// and 235 / 219 at 32, now 128 / 129, 139 / 161 and 164 / 217.
+// and 235 / 219 at 32, now 127 / 127, 139 / 156 and 164 / 211.
 #include <algorithm>
 #include <climits>
 #include <cuda_runtime.h>
@@ -362,6 +362,9 @@ __global__ void __launch_bounds__(32, kF64MinWarps) decode_f64_kernel(const uint
                                                                       double *__restrict__ dst, Geom64 g)
 {
     extern __shared__ uint64_t sm64[];
+    __shared__ DropTable drop;
+    load_drop<32>(drop);
+    __syncthreads();
     uint64_t *tile = sm64 + 64 * 32;
     const int lane = threadIdx.x;
     const Tile64 st{tile, lane};
@@ -388,7 +391,7 @@ __global__ void __launch_bounds__(32, kF64MinWarps) decode_f64_kernel(const uint
             const int e = (int)((head >> 1) & 0x7ffu);
             // the planes from bit 12 on; the tile's two zero 64-bit words let the
             // parser read past the budget without a test
-            const Tile64As32 t32{reinterpret_cast<const uint32_t *>(tile), lane};
+            const WithDrop<Tile64As32> t32(Tile64As32{reinterpret_cast<const uint32_t *>(tile), lane}, drop);
             const int kmin = parse_planes64<true>(t32, 12, 64 * g.rate, 63, pl);
             // planes below kmin are zero; the negabinary xor is the complement of
             // the odd planes

@@ -61,6 +61,9 @@ decode_rfft_kernel(const uint8_t *__restrict__ in, const FusedMsg *__restrict__ 
                    float *__restrict__ re, float *__restrict__ im, int64_t os1, int64_t os2, int warp_bytes)
 {
     extern __shared__ __align__(16) uint8_t fsmem[];
+    __shared__ DropTable drop;
+    load_drop<32 * kWarps>(drop);
+    __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, tid = threadIdx.x;
     uint8_t *wsm = fsmem + (size_t)wid * warp_bytes;
     uint32_t *t32 = reinterpret_cast<uint32_t *>(wsm);
@@ -90,7 +93,7 @@ decode_rfft_kernel(const uint8_t *__restrict__ in, const FusedMsg *__restrict__ 
                     t32[(4 * i + 3) * 32 + lane] = v.w;
                 }
                 float x[64];
-                const StreamTile tile{t32, lane};
+                const WithDrop<StreamTile> tile(StreamTile{t32, lane}, drop);
                 SmemPlanes pl{wpl, lane};
                 decode_block3_tile<RATE>(tile, x, pl);
                 const int xg = M.x0 + 4 * bx;

