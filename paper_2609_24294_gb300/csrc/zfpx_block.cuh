@@ -1160,6 +1160,10 @@ ZFPX_HD uint32_t gather4(uint32_t x)
     return (x | (x >> 12)) & 0xffu;
 }
 
+struct SpreadBits {                                                // spread4 by shifts
+    ZFPX_HD uint32_t operator()(uint32_t x) const { return spread4(x); }
+};
+
 // The word a 1-D block's 4 RATE bits fill, and the interleaves in it: as many
 // planes as can matter from bit 9 on.
 template <int RATE>
@@ -1170,13 +1174,14 @@ struct Word1 {
     {
         return ((T)(spread3(a >> 10) | (spread3(b >> 10) << 1)) << 30) | spread3(a) | (spread3(b) << 1);
     }
-    ZFPX_HD static T tail(const uint32_t (&v)[4], int p)
+    template <class Spread>
+    ZFPX_HD static T tail(const uint32_t (&v)[4], int p, const Spread &spread)
     {
         T r = 0;
 #pragma unroll
         for (int i = 0; i < 4; i++) {
             const uint32_t a = shr_any(v[i], p);
-            r |= (((T)spread4(a >> 8) << 32) | spread4(a)) << i;
+            r |= (((T)spread(a >> 8) << 32) | spread(a)) << i;
         }
         return r;
     }
@@ -1194,11 +1199,12 @@ struct Word1<8> {
     typedef uint32_t T;
     ZFPX_HD static T runs1(uint32_t a) { return spread2(a); }
     ZFPX_HD static T runs2(uint32_t a, uint32_t b) { return spread3(a) | (spread3(b) << 1); }
-    ZFPX_HD static T tail(const uint32_t (&v)[4], int p)
+    template <class Spread>
+    ZFPX_HD static T tail(const uint32_t (&v)[4], int p, const Spread &spread)
     {
         T r = 0;
 #pragma unroll
-        for (int i = 0; i < 4; i++) r |= spread4(shr_any(v[i], p)) << i;
+        for (int i = 0; i < 4; i++) r |= spread(shr_any(v[i], p)) << i;
         return r;
     }
     ZFPX_HD static uint32_t of_runs1(T w) { return gather2(w); }
@@ -1209,8 +1215,8 @@ struct Word1<8> {
 };
 
 // Encodes K blocks x[b][0..3]; w[b] = the block's 4 RATE bits.
-template <int RATE, int K>
-ZFPX_HD void encode_blocks1(const float (&x)[K][4], const Plane4Enc &tab, uint64_t (&w)[K])
+template <int RATE, int K, class Spread = SpreadBits>
+ZFPX_HD void encode_blocks1(const float (&x)[K][4], const Plane4Enc &tab, uint64_t (&w)[K], const Spread &spread = Spread())
 {
     typedef typename Word1<RATE>::T T;
 #pragma unroll
@@ -1257,14 +1263,24 @@ ZFPX_HD void encode_blocks1(const float (&x)[K][4], const Plane4Enc &tab, uint64
             pos += 3 * run;
             if (e2 < 32) event(e2);
         }
-        if (n >= 3) r |= shl_any(Word1<RATE>::tail(v, p), pos);
+        if (n >= 3) r |= shl_any(Word1<RATE>::tail(v, p, spread), pos);
         w[b] = zero ? 0ull : (uint64_t)r;
     }
 }
 
+// The planes from p on of w, every coefficient significant, into v by shifts.
+struct TailBits {
+    template <class Word>
+    ZFPX_HD void add(typename Word::T w, int p, uint32_t (&v)[4]) const
+    {
+#pragma unroll
+        for (int i = 0; i < 4; i++) v[i] |= shl_any(Word::of_tail(w, i), p);
+    }
+};
+
 // Decodes K blocks from their 4 RATE-bit words.
-template <int RATE, int K>
-ZFPX_HD void decode_blocks1(const uint64_t (&win)[K], const Plane4Dec &tab, float (&x)[K][4])
+template <int RATE, int K, class Tail = TailBits>
+ZFPX_HD void decode_blocks1(const uint64_t (&win)[K], const Plane4Dec &tab, float (&x)[K][4], const Tail &tail = Tail())
 {
     typedef typename Word1<RATE>::T T;
     constexpr int END = 4 * RATE;
@@ -1313,10 +1329,7 @@ ZFPX_HD void decode_blocks1(const uint64_t (&win)[K], const Plane4Dec &tab, floa
             if (p + run < 32 && t) event(p + run);
             else n = -1;
         }
-        if (n >= 3) {
-#pragma unroll
-            for (int i = 0; i < 4; i++) v[i] |= shl_any(Word1<RATE>::of_tail(w, i), p);
-        }
+        if (n >= 3) tail.template add<Word1<RATE>>(w, p, v);
         if (!(win[b] & 1ull)) {
             x[b][0] = x[b][1] = x[b][2] = x[b][3] = 0.0f;
             continue;
