@@ -130,19 +130,29 @@ __device__ __forceinline__ void load_rows(const float *p, const int64_t *s, int 
 }
 
 // The same with partial rows (nx < 4 values, the last one repeated): four
-// values at a time through the lane's column of `stage` (64 rows of 32 floats),
-// kept rolled so that the complete blocks' code stays compact.
-__device__ __forceinline__ void load_edge(const float *p, const int64_t *s, int nx, int ny, int nz, float *stage,
+// values at a time through `own`, the lane's own words of the plane tile ([32][32]
+// 64-bit, this lane's column, two values a word), kept rolled so that the
+// complete blocks' code stays compact.  No other lane's words are touched, so
+// the other lanes may be storing planes, or still reading them, meanwhile.
+__device__ __forceinline__ void load_edge(const float *p, const int64_t *s, int nx, int ny, int nz, uint64_t *own,
                                           float (&x)[64])
 {
 #pragma unroll 1
     for (int r = 0; r < 16; r++) {
         const float *row = p + (int64_t)min(r >> 2, nz - 1) * s[2] + (int64_t)min(r & 3, ny - 1) * s[1];
 #pragma unroll
-        for (int i = 0; i < 4; i++) stage[32 * (4 * r + i)] = __ldg(row + (int64_t)min(i, nx - 1) * s[0]);
+        for (int h = 0; h < 2; h++) {
+            const float a = __ldg(row + (int64_t)min(2 * h, nx - 1) * s[0]);
+            const float b = __ldg(row + (int64_t)min(2 * h + 1, nx - 1) * s[0]);
+            own[32 * (2 * r + h)] = (uint64_t)f2u(b) << 32 | f2u(a);
+        }
     }
 #pragma unroll
-    for (int r = 0; r < 64; r++) x[r] = stage[32 * r];
+    for (int r = 0; r < 32; r++) {
+        const uint64_t v = own[32 * r];
+        x[2 * r] = u2f((uint32_t)v);
+        x[2 * r + 1] = u2f((uint32_t)(v >> 32));
+    }
 }
 
 // The inverses: only rows inside the box are written.
@@ -171,18 +181,21 @@ __device__ __forceinline__ void store_rows(float *p, const int64_t *s, int ny, i
         }
     }
 }
-__device__ __forceinline__ void store_edge(float *p, const int64_t *s, int nx, int ny, int nz, float *stage,
+__device__ __forceinline__ void store_edge(float *p, const int64_t *s, int nx, int ny, int nz, uint64_t *own,
                                            const float (&x)[64])
 {
 #pragma unroll
-    for (int r = 0; r < 64; r++) stage[32 * r] = x[r];
+    for (int r = 0; r < 32; r++) own[32 * r] = (uint64_t)f2u(x[2 * r + 1]) << 32 | f2u(x[2 * r]);
 #pragma unroll 1
     for (int r = 0; r < 16; r++) {
         if ((r >> 2) >= nz || (r & 3) >= ny) continue;
         float *row = p + (int64_t)(r >> 2) * s[2] + (int64_t)(r & 3) * s[1];
 #pragma unroll
-        for (int i = 0; i < 4; i++)
-            if (i < nx) row[(int64_t)i * s[0]] = stage[32 * (4 * r + i)];
+        for (int h = 0; h < 2; h++) {
+            const uint64_t v = own[32 * (2 * r + h)];
+            if (2 * h < nx) row[(int64_t)(2 * h) * s[0]] = u2f((uint32_t)v);
+            if (2 * h + 1 < nx) row[(int64_t)(2 * h + 1) * s[0]] = u2f((uint32_t)(v >> 32));
+        }
     }
 }
 
@@ -250,7 +263,7 @@ encode3_kernel(const float *__restrict__ src, uint8_t *__restrict__ out, LaunchG
                 const float *p = base + (int64_t)z0 * g.ss[2] + (int64_t)y0 * g.ss[1] + (int64_t)x0 * g.ss[0];
                 const int kind = VEC ? ROWS_ANY : row_kind(base, g.ss);
                 if (x0 + 4 > nx)
-                    load_edge(p, g.ss, nx - x0, ny - y0, nz - z0, reinterpret_cast<float *>(v.planes) + lane, x);
+                    load_edge(p, g.ss, nx - x0, ny - y0, nz - z0, v.planes + lane, x);
                 else if (!VEC && kind == ROWS_8)
                     load_rows<ROWS_8>(p, g.ss, ny - y0, nz - z0, x);
                 else if (!VEC && kind == ROWS_4_8_4)
@@ -386,7 +399,7 @@ decode3_kernel(const uint8_t *__restrict__ in, float *__restrict__ dstf, LaunchG
                 float *p = base + (int64_t)z0 * g.ds[2] + (int64_t)y0 * g.ds[1] + (int64_t)x0 * g.ds[0];
                 const int kind = VEC ? ROWS_ANY : row_kind(base, g.ds);
                 if (x0 + 4 > nx)
-                    store_edge(p, g.ds, nx - x0, ny - y0, nz - z0, reinterpret_cast<float *>(splanes[wid]) + lane, v);
+                    store_edge(p, g.ds, nx - x0, ny - y0, nz - z0, splanes[wid] + lane, v);
                 else if (!VEC && kind == ROWS_8)
                     store_rows<ROWS_8>(p, g.ds, ny - y0, nz - z0, v);
                 else if (!VEC && kind == ROWS_4_8_4)
