@@ -746,6 +746,9 @@ int zfpx_legendre_forward(zfpx_legendre p, const float *d_re, const float *d_im,
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return ZFPX_ECUDA;
     if (dev != p->device) return ZFPX_EINVAL;
+    // the tensor map is encoded through the driver, which wants a current context:
+    // a host thread that has made no runtime call yet has none
+    if (cudaSetDevice(dev) != cudaSuccess) return ZFPX_ECUDA;
     LegGeom g{};
     g.nlat = p->nlat; g.nh = p->nh; g.nhs = p->nhs; g.T = p->T; g.nlev = (int)n[2];
     g.N = 2 * g.nlev;
