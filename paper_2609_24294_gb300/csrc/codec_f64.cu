@@ -493,14 +493,6 @@ unsigned grid_f64(const void *fn, int warps, int64_t nunits, size_t smem)
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>((nunits + warps - 1) / warps, cap));
 }
 
-// Dynamic shared memory above 48 KB is opted into per kernel.
-int f64_prepare(const void *fn, size_t smem)
-{
-    if (smem <= 48 * 1024) return ZFPX_OK;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess
-               ? ZFPX_OK : ZFPX_ECUDA;
-}
-
 bool valid_f64_args(int rate, const int64_t n[3], const int64_t stride[3])
 {
     if (rate < 1 || rate > kMaxRate || !n || !stride) return false;
@@ -530,7 +522,7 @@ int zfpx_encode_f64(int rate, const double *d_in, const int64_t n[3], const int6
     if (cap < zfpx_stream_bytes_f64(rate, n)) return ZFPX_ESIZE;
     const Geom64 g = make_geom(n, stride, rate, d_in);
     const size_t smem = f64_enc_smem_bytes(rate);
-    const int rc = f64_prepare((const void *)encode_f64_kernel, smem);
+    const int rc = allow_smem((const void *)encode_f64_kernel, smem);
     if (rc) return rc;
     encode_f64_kernel<<<grid_f64((const void *)encode_f64_kernel, kEncWarps, g.nunits, smem), 32 * kEncWarps, smem,
                         (cudaStream_t)stream>>>(d_in, d_out, g);
@@ -546,7 +538,7 @@ int zfpx_decode_f64(int rate, const uint8_t *d_in, size_t len, const int64_t n[3
     if (len < zfpx_stream_bytes_f64(rate, n)) return ZFPX_ESIZE;
     const Geom64 g = make_geom(n, stride, rate, d_out);
     const size_t smem = f64_dec_smem_bytes(rate);
-    const int rc = f64_prepare((const void *)decode_f64_kernel, smem);
+    const int rc = allow_smem((const void *)decode_f64_kernel, smem);
     if (rc) return rc;
     decode_f64_kernel<<<grid_f64((const void *)decode_f64_kernel, 1, g.nunits, smem), 32, smem, (cudaStream_t)stream>>>(
         d_in, d_out, g);

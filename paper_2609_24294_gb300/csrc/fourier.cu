@@ -174,8 +174,7 @@ int zfpx_rfft_lon(const float *d_in, const int64_t n[3], const int64_t stride[3]
         return check_launch();
     }
     const size_t smem = 2 * sizeof(float2) * (size_t)warps * g.H;
-    if (cudaFuncSetAttribute(rfft_lon_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return ZFPX_ECUDA;
+    if ((rc = allow_smem((const void *)rfft_lon_kernel, smem))) return rc;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rfft_lon_kernel, 32 * warps, smem) != cudaSuccess)
         return ZFPX_ECUDA;

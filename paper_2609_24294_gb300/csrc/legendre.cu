@@ -780,8 +780,7 @@ int zfpx_legendre_forward(zfpx_legendre p, const float *d_re, const float *d_im,
     if (nblk > 0x7fffffff) return ZFPX_EINVAL;
     if (nblk == 0) return ZFPX_OK;
     const size_t smem = mma_smem_bytes(g.nt);
-    if (cudaFuncSetAttribute(legendre_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return ZFPX_ECUDA;
+    if ((rc = allow_smem((const void *)legendre_mma_kernel, smem))) return rc;
     const int grid = (int)std::min<int64_t>(nblk, num_sms());      // persistent: one CTA per SM
     legendre_mma_kernel<<<grid, kMmaThreads, smem, st>>>(p->tmap_table, tmap_g, p->d_items, g,
                                                           mma_stages(g.nt), (int)nblk,

@@ -40,6 +40,28 @@ int occupancy(const void *fn, int threads)
     return n;
 }
 
+int allow_smem(const void *fn, size_t smem)
+{
+    static std::mutex mu;
+    static std::map<std::pair<const void *, int>, size_t> limits;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return ZFPX_ECUDA;
+    std::lock_guard<std::mutex> g(mu);
+    auto key = std::make_pair(fn, dev);
+    auto it = limits.find(key);
+    if (it == limits.end()) {
+        int most = 0;
+        cudaFuncAttributes a{};
+        if (cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+            cudaFuncGetAttributes(&a, fn) != cudaSuccess)
+            return ZFPX_ECUDA;
+        most -= (int)a.sharedSizeBytes;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess) return ZFPX_ECUDA;
+        it = limits.emplace(key, (size_t)most).first;
+    }
+    return smem <= it->second ? ZFPX_OK : ZFPX_ECUDA;
+}
+
 int check_launch()
 {
     cudaError_t e = cudaGetLastError();

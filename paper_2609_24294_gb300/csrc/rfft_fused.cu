@@ -260,7 +260,7 @@ int zfpx_decompress_rfft(zfpx_plan p, int rate, const uint8_t *d_recv, size_t le
     const int wb = warp_bytes(rate, fg.H);
     const size_t smem = (size_t)kWarps * wb;
     const void *fn = rate == 8 ? (const void *)decode_rfft_kernel<8> : (const void *)decode_rfft_kernel<16>;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return ZFPX_ECUDA;
+    if ((rc = allow_smem(fn, smem))) return rc;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * kWarps, smem) != cudaSuccess) return ZFPX_ECUDA;
     per_sm = std::max(1, std::min(per_sm, kMaxCtasPerSm));

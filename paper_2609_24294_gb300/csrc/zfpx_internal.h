@@ -204,6 +204,12 @@ bool codec_vec_ok(const void *ptr, const int64_t s[3], const zfpx_plan_s *p);
 int num_sms();
 // Resident CTAs per SM of `fn` at `threads` threads (cached per kernel).
 int occupancy(const void *fn, int threads);
+// For a launch of `fn` with `smem` bytes of dynamic shared memory: lifts the
+// kernel's limit on them to what the device offers beside its static ones, once per
+// device.  The limit is the kernel's, not the call's, so one set to each call's own
+// size could be lowered by another thread between a call's set and its launch.
+// ZFPX_ECUDA if smem is more than the device offers.
+int allow_smem(const void *fn, size_t smem);
 void count_launch();
 void uncount_launches(uint64_t n);   // launches recorded into a graph, not run
 bool valid_codec_rate(int rate);

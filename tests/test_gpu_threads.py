@@ -72,3 +72,26 @@ def test_first_call_of_a_thread(make, size):
     torch.cuda.synchronize()
     assert not failed
     assert all(torch.equal(o, w) for o, w in zip(outs, want))
+
+
+# The limit on dynamic shared memory belongs to the kernel: no call may lower what
+# another has asked for.  float64 rates of 49664 and 51712 bytes; the others'
+# smallest and a large launch.
+@pytest.mark.parametrize("make,sizes", [(f64, (28, 32)), (rfft, (20, 8100)), (fused, (20, 3750)), (legendre, (8, 96))])
+def test_calls_of_two_sizes_from_four_threads(make, sizes):
+    calls = []
+    for size in sizes:
+        fn, outs = make(size)
+        fn(torch.cuda.current_stream())
+        calls.append((fn, outs, [o.clone() for o in outs], torch.cuda.Stream()))
+    for _, outs, _, _ in calls:
+        for o in outs:
+            o.zero_()
+    torch.cuda.synchronize()
+    threads = [new_thread_runs(lambda fn=fn, st=st: fn(st), 6000) for fn, _, _, st in calls for _ in range(2)]
+    for t, _ in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not any(failed for _, failed in threads)
+    for _, outs, want, _ in calls:
+        assert all(torch.equal(o, w) for o, w in zip(outs, want))
