@@ -263,6 +263,16 @@ encode_f64_kernel(const double *__restrict__ src, uint8_t *__restrict__ out, Geo
         for (int r = 0; r < 64; r++) amax = max(amax, (uint32_t)((uint64_t)v[r] >> 32) & 0x7fffffffu);
         const int e = block_exponent(amax);
         const bool act = valid && e;
+        // nothing to code in the whole warp: the streams are zero (640 x 320 x 91 zeros:
+        // 98 -> 50 us at rate 8, 110 -> 66 at 32; nothing more for other fields)
+        if (!__any_sync(0xffffffffu, act)) {
+            uint8_t *dst = out + (b0 + lane) * (int64_t)g.rate * 8;
+            if (valid && out16)
+                for (int i = 0; i < g.rate; i += 2) *reinterpret_cast<uint4 *>(dst + 8 * i) = make_uint4(0u, 0u, 0u, 0u);
+            else if (valid)
+                for (int i = 0; i < g.rate; i++) *reinterpret_cast<uint2 *>(dst + 8 * i) = make_uint2(0u, 0u);
+            continue;
+        }
 #pragma unroll
         for (int r = 0; r < 64; r++) v[r] = quantize64((uint64_t)v[r], e);
         xform3_fwd64(v);

@@ -59,6 +59,9 @@ __device__ __forceinline__ void encode(const float (&x)[16], bool valid, const V
     const uint32_t amax = f2u(am) & 0x7fffffffu;
     const int E = (int)(amax >> 23);
     const bool act = valid && amax >= 0x00400000u && E != 255;   // else a single 0 bit
+    // nothing to code in the whole warp (dry or masked areas): the streams are zero,
+    // as the tile is (120 zero levels of 1280 x 640 at rate 8: 119 -> 82 us)
+    if (!__any_sync(0xffffffffu, act)) return;
     const QuantScale qs(act ? E : 127);
     int32_t q[16];
 #pragma unroll
