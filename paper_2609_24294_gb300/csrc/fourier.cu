@@ -56,6 +56,24 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 3) rfft_lon_kernel(const float
     }
 }
 
+// Rows of a length whose stages are fixed (rfft_row_fixed), one warp per row.
+template <int N, int... P>
+__global__ void __launch_bounds__(32 * kMaxWarps, 3)
+rfft_lon_fixed_kernel(const float *__restrict__ in, float *__restrict__ re, float *__restrict__ im,
+                      const float2 *__restrict__ tw, FftGeom g)
+{
+    __shared__ __align__(16) float2 buf[kMaxWarps][N];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int64_t gr = (int64_t)blockIdx.x * kMaxWarps + wid; gr < g.nrows; gr += (int64_t)gridDim.x * kMaxWarps) {
+        const int64_t y = gr % g.ny, z = gr / g.ny;
+        load_row_async(buf[wid], reinterpret_cast<const float2 *>(in + z * g.is2 + y * g.is1), N / 2, lane);
+        wait_rows();
+        __syncwarp();
+        rfft_row_fixed<true, N, P...>(buf[wid], buf[wid] + N / 2, tw, g.K, lane, re + z * g.os2 + y * g.os1,
+                                      im + z * g.os2 + y * g.os1);
+    }
+}
+
 // Rows of N = 64 R1 (rfft_row64), one warp per row.  The bound leaves 102
 // registers, which both passes fit, and 20 warps per SM.
 constexpr int kRow64Warps = 4;
@@ -160,16 +178,22 @@ int zfpx_rfft_lon(const float *d_in, const int64_t n[3], const int64_t stride[3]
     const float2 *tw = nullptr;
     int rc = fft_twiddles(g.N, &tw);
     if (rc) return rc;
-    if (g.r1) {
-        void (*k64)(const float *, float *, float *, const float2 *, FftGeom) = nullptr;
-        switch (g.r1) {
-#define ZFPX_FFT_CASE(R) case R: k64 = rfft_lon64_kernel<R>; break;
-            ZFPX_FFT_ROW64_RADICES(ZFPX_FFT_CASE)
+    void (*special)(const float *, float *, float *, const float2 *, FftGeom) = nullptr;
+    switch (g.r1) {
+#define ZFPX_FFT_CASE(R) case R: special = rfft_lon64_kernel<R>; break;
+        ZFPX_FFT_ROW64_RADICES(ZFPX_FFT_CASE)
 #undef ZFPX_FFT_CASE
-        }
-        const int64_t groups = (g.nrows + kRow64Warps - 1) / kRow64Warps;
-        const int64_t cap = (int64_t)num_sms() * occupancy((const void *)k64, 32 * kRow64Warps);
-        k64<<<(unsigned)std::min<int64_t>(groups, cap), 32 * kRow64Warps, 0, (cudaStream_t)stream>>>(d_in, d_re, d_im, tw, g);
+    }
+    switch (g.N) {
+#define ZFPX_FFT_CASE(N_, ...) case N_: special = rfft_lon_fixed_kernel<N_, __VA_ARGS__>; break;
+        ZFPX_FFT_FIXED_LENGTHS(ZFPX_FFT_CASE)
+#undef ZFPX_FFT_CASE
+    }
+    if (special) {
+        const int w = g.r1 ? kRow64Warps : kMaxWarps;
+        const int64_t groups = (g.nrows + w - 1) / w;
+        const int64_t cap = (int64_t)num_sms() * occupancy((const void *)special, 32 * w);
+        special<<<(unsigned)std::min<int64_t>(groups, cap), 32 * w, 0, (cudaStream_t)stream>>>(d_in, d_re, d_im, tw, g);
         count_launch();
         return check_launch();
     }

@@ -54,6 +54,16 @@ __device__ __noinline__ void row64_call(const float2 *src, float2 *buf, const fl
     fft::rfft_row64<R1, false>(src, buf, tw, tw2, K, lane, ore, oim);
 }
 
+template <int N, int... P>
+__device__ __noinline__ void fixed_call(float2 *X, float2 *Y, const float2 *src, const float2 *__restrict__ tw, int K,
+                                        int lane, float *ore, float *oim)
+{
+    fft::load_row_async(X, src, N / 2, lane);
+    fft::wait_rows();
+    __syncwarp();
+    fft::rfft_row_fixed<false, N, P...>(X, Y, tw, K, lane, ore, oim);
+}
+
 template <int RATE>
 __global__ void __launch_bounds__(32 * kWarps)
 decode_rfft_kernel(const uint8_t *__restrict__ in, const FusedMsg *__restrict__ msgs, const FusedUnit *__restrict__ units,
@@ -131,10 +141,16 @@ decode_rfft_kernel(const uint8_t *__restrict__ in, const FusedMsg *__restrict__ 
                 ZFPX_FFT_ROW64_RADICES(ZFPX_FFT_CASE)
 #undef ZFPX_FFT_CASE
             default:
-                fft::load_row_async(X, src, fg.H, lane);
-                fft::wait_rows();
-                __syncwarp();
-                fft::rfft_row<false>(X, Y, tw, fg, lane, re + o, im + o);
+                switch (fg.N) {
+#define ZFPX_FFT_CASE(N_, ...) case N_: fixed_call<N_, __VA_ARGS__>(X, Y, src, tw, fg.K, lane, re + o, im + o); break;
+                    ZFPX_FFT_FIXED_LENGTHS(ZFPX_FFT_CASE)
+#undef ZFPX_FFT_CASE
+                default:
+                    fft::load_row_async(X, src, fg.H, lane);
+                    fft::wait_rows();
+                    __syncwarp();
+                    fft::rfft_row<false>(X, Y, tw, fg, lane, re + o, im + o);
+                }
             }
         }
         __syncthreads();

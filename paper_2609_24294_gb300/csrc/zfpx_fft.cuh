@@ -18,7 +18,7 @@ struct FastDiv {
     uint32_t d, m;
     __device__ __forceinline__ uint32_t div(uint32_t n) const { return m ? __umulhi(n, m) : n; }
 };
-__host__ inline FastDiv make_fastdiv(uint32_t d)
+__host__ __device__ constexpr FastDiv make_fastdiv(uint32_t d)
 {
     return FastDiv{d, d == 1 ? 0u : (uint32_t)((((uint64_t)1 << 32) + d - 1) / d)};
 }
@@ -225,6 +225,32 @@ __device__ __forceinline__ void rfft_row(float2 *X, float2 *Y, const float2 *__r
     }
     split_real<STREAM>(X, tw, H, g.K, scale, lane, ore, oim);
 }
+
+// rfft_row for a length whose stages P ... are fixed when it is compiled: the same
+// values in half the instructions (no dispatch over the radices, and every index
+// and twiddle distance a constant).
+template <int N, int L, int P, int... REST>
+__device__ __forceinline__ float2 *fixed_stages(float2 *X, float2 *Y, const float2 *__restrict__ tw, int lane)
+{
+    fft_stage<P, L == 1>(X, Y, tw, N, N / 2, L, lane, make_fastdiv(N / 2 / L / P));
+    __syncwarp();
+    if constexpr (sizeof...(REST) > 0) return fixed_stages<N, L * P, REST...>(Y, X, tw, lane);
+    return Y;
+}
+template <bool STREAM, int N, int... P>
+__device__ __forceinline__ void rfft_row_fixed(float2 *X, float2 *Y, const float2 *__restrict__ tw, int K, int lane,
+                                               float *ore, float *oim)
+{
+    split_real<STREAM>(fixed_stages<N, 1, P...>(X, Y, tw, lane), tw, N / 2, K, 1.0f / (float)N, lane, ore, oim);
+}
+// Built for the multiples of 32 below the two register passes, in
+// factor_half_impl's order: their stages leave lanes idle, so the dispatch weighs
+// most there, and pairs of outputs (split_real) take longer than an output a lane.
+// us for 262144 rows, K = N / 2, general stages with an output a lane, with pairs,
+// and these: N = 32: 164, 178, 94; 64: 216, 229, 105; 96: 244, 232, 121; 128: 228,
+// 244, 134; 160: 277, 263, 161; 192: 305, 308, 164.
+// Fn: a macro taking N and the radices.
+#define ZFPX_FFT_FIXED_LENGTHS(F) F(32, 16) F(64, 16, 2) F(96, 16, 3) F(128, 16, 4) F(160, 16, 5) F(192, 16, 2, 3)
 
 // ------------------------------------------------------------------ N = 64 r1
 // The H = 32 r1 points in two passes of registers.  Pass 1: lane k takes the r1
