@@ -106,7 +106,6 @@ __device__ __forceinline__ void fill_plane4(const BatchGeom &bg, Tab &tab)
     for (int i = 0; i < bg.ngroups; i++) any1 |= bg.groups[i].dims == 1;
     if (!any1) return;
     plane4_fill(tab, threadIdx.x, blockDim.x);
-    __syncthreads();
 }
 
 // Work distribution of the batch kernels.  A batch with no more units than
@@ -121,8 +120,12 @@ __device__ __forceinline__ void fill_plane4(const BatchGeom &bg, Tab &tab)
 // cache -- and then helps the other groups until every queue is empty.
 // fn has one call site for both cases: the kernels inline the codec of every
 // kind into it, and a second copy of that code costs instruction-cache misses.
-template <class Fn>
-__device__ __forceinline__ void for_each_unit(const BatchGeom &bg, int lane, Fn &&fn)
+// ready() is called once by every warp of the CTA, its first unit found, before fn:
+// the wait for the CTA's tables, which the search hides (8 levels at rate 8 and a 1-D
+// field on a grid of 640 rows: 32 -> 26 us encode, 33 -> 27 decode with the wait
+// first and then; 20 levels on 1280 rows 148 -> 137 and 125 -> 114).
+template <class Ready, class Fn>
+__device__ __forceinline__ void for_each_unit(const BatchGeom &bg, int lane, Ready &&ready, Fn &&fn)
 {
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const bool single = bg.nunits <= nwarps;                     // a small batch: one unit per warp, no claims
@@ -140,7 +143,10 @@ __device__ __forceinline__ void for_each_unit(const BatchGeom &bg, int lane, Fn 
     };
     if (single) {
         const int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-        if (c >= bg.nunits) return;
+        if (c >= bg.nunits) {
+            ready();
+            return;
+        }
         while (gi + 1 < bg.ngroups && c >= bg.groups[gi + 1].u0) gi++;
         u = (uint32_t)(c - bg.groups[gi].u0);
     } else {
@@ -152,7 +158,10 @@ __device__ __forceinline__ void for_each_unit(const BatchGeom &bg, int lane, Fn 
         C = size(0);
         u = __shfl_sync(0xffffffffu, claim(C), 0);
     }
-    for (;;) {
+    // the first unit's item ahead of the barrier, whose wait its search hides
+    int ii = (int64_t)u < bg.groups[gi].n ? item_of_unit(bg.items, bg.nitems, bg.groups[gi].u0 + u) : -1;
+    ready();
+    for (;; ii = -1) {
         while (!single && (int64_t)u >= bg.groups[gi].n) {       // this queue is empty: the next group's
             if (tried++ == bg.ngroups) return;
             gi = gi + 1 == bg.ngroups ? 0 : gi + 1;
@@ -164,7 +173,7 @@ __device__ __forceinline__ void for_each_unit(const BatchGeom &bg, int lane, Fn 
         const uint32_t next = single ? 0u : claim(nextC);        // claimed ahead: its latency hides behind fn
         // the claim's units in order; a unit's item is the last one starting at or before it
         const uint32_t ue = single ? u + 1 : (uint32_t)min((int64_t)u + C, G.n);
-        int ii = item_of_unit(bg.items, bg.nitems, G.u0 + u);
+        if (ii < 0) ii = item_of_unit(bg.items, bg.nitems, G.u0 + u);
         for (; u < ue; u++) {
             const int64_t c = G.u0 + u;
             while (ii + 1 < bg.nitems && __ldg(&bg.items[ii + 1].unit0) <= c) ii++;
@@ -333,9 +342,7 @@ batch_encode_kernel(BatchGeom bg, uint8_t *__restrict__ out)
     const enc3::View v = sh[wid].view(expand);
     enc3::clear(v, lane, enc3::kWords<16>);
     fill_plane4(bg, tab);
-    enc3::wait_expand();
-    __syncthreads();
-    for_each_unit(bg, lane, [&](const GroupDev &G, int64_t c, int ii) {
+    for_each_unit(bg, lane, []() { enc3::wait_expand(); __syncthreads(); }, [&](const GroupDev &G, int64_t c, int ii) {
         const ItemDevB it = bg.items[ii];
         const FieldDevB f = bg.fields[it.field];
         if (G.dims == 3) {
@@ -425,11 +432,10 @@ batch_decode_kernel(BatchGeom bg, const uint8_t *__restrict__ in)
     __shared__ uint64_t splanes[WARPS][32 * 32];
     __shared__ Plane4Dec tab;
     __shared__ DropTable drop;
+    load_drop_async(drop);
     fill_plane4(bg, tab);
-    load_drop<32 * WARPS>(drop);
-    __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for_each_unit(bg, lane, [&](const GroupDev &G, int64_t c, int ii) {
+    for_each_unit(bg, lane, []() { enc3::wait_expand(); __syncthreads(); }, [&](const GroupDev &G, int64_t c, int ii) {
         const ItemDevB it = bg.items[ii];
         const FieldDevB f = bg.fields[it.field];
         if (G.dims == 3) {
@@ -680,8 +686,13 @@ int launch_batch(const BatchGeom &g, int warps, int ctas_per_sm, bool encode, co
 {
     if (g.nunits == 0) return ZFPX_OK;
     // where the caller has set none: CTAs of two warps, sixteen warps to an SM, for
-    // batches that fill the device (885 / 867 us against 911 / 879 with three), else
-    // three, which spread a small batch's units better over the schedulers
+    // batches that fill the device (encode / decode of three 3-D and two 1-D fields on
+    // 1280 rows 332 / 300 us, 344 / 312 with three warps; 60 levels on 896 rows 197 /
+    // 164 against 202 / 172), else three, better by up to a tenth where a small batch
+    // holds 1-D fields (8 levels and one 1-D field on 64 rows 14.9 / 16.4 against
+    // 16.0 / 18.4) and mostly the same without (8 levels at rate 16 on 64 to 384 rows;
+    // 60 levels on 192 rows 20.5 / 18.5 against 18.4 / 16.9).  The line is where
+    // every resident warp of the three has a unit.
     if (!warps) warps = g.nunits > (int64_t)num_sms() * 15 ? 2 : 3;
     if (!batch_warps_ok(warps)) return ZFPX_EINVAL;
     const void *fn = warps == 2 ? batch_kernel<2>(encode) : warps == 3 ? batch_kernel<3>(encode)

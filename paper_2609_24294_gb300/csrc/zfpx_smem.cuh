@@ -53,7 +53,7 @@ struct StreamTile {
 // the most of them needs.  Decompressing a 1280 x 640 x 137 field over 8 x 8 ranks:
 // 289 -> 278 us at rate 8, 361 -> 350 at rate 16; 37 levels of 2-D blocks over 4
 // x 4 ranks 129 -> 122 and 139 -> 133 (with all four lookups at once 126 and 139).
-struct DropTable {
+struct __align__(16) DropTable {
     uint32_t w[64];
 };
 constexpr DropTable make_drop_table()
@@ -79,6 +79,15 @@ __device__ __forceinline__ void load_drop(DropTable &tab)
 #pragma unroll
         for (int i = 0; i < 64; i += THREADS) tab.w[i + threadIdx.x] = __ldg(g_drop.w + i + threadIdx.x);
     }
+}
+
+// The same copied asynchronously by the first warp; ready after cp.async.wait_all
+// by its threads and a __syncthreads().
+__device__ __forceinline__ void load_drop_async(DropTable &tab)
+{
+    if (threadIdx.x < 16)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(tab.w + 4 * threadIdx.x)),
+                     "l"(g_drop.w + 4 * threadIdx.x) : "memory");
 }
 
 // A stream tile with the table.
