@@ -165,10 +165,11 @@ ZFPX_API int zfpx_decompress_unpack(zfpx_plan plan, int rate, const uint8_t *d_i
 
 /* Launch shape of the 3-D codec kernels: every warp codes `upw` consecutive
  * units of 32 blocks (encode != 0: compression, else decompression; rate 8
- * or 16); 0 restores the library's default (2, 1 in launches of few units, and
- * a warp per block in the smallest).
+ * or 16); 0, the state at the start, leaves it to the library, launch by launch
+ * (2, 1 in launches of few units, and a warp per block in the smallest).
  * Process-wide; results never depend on it (the autotuner sets it).  Errors:
- * ZFPX_EINVAL.  zfpx_get_units_per_warp returns the value in use. */
+ * ZFPX_EINVAL.  zfpx_get_units_per_warp returns the value set, 0 if that is the
+ * library's choice. */
 ZFPX_API int zfpx_set_units_per_warp(int encode, int rate, int upw);
 ZFPX_API int zfpx_get_units_per_warp(int encode, int rate);
 

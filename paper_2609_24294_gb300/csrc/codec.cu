@@ -790,7 +790,7 @@ template <class In, class Out, class Acc>
 void launch3(void (*kernel)(In, Out, LaunchGeom, int, Acc), int warps, int encode, int rate, LaunchGeom g,
              cudaStream_t st, In in, Out out, int layout, const Acc &acc = Acc{})
 {
-    g.upw = g_upw[encode ? 1 : 0][rate == 16 ? 1 : 0].load(std::memory_order_relaxed);
+    g.upw = units_per_warp(encode, rate);
     if (g.upw <= 0) {
         const int64_t resident = (int64_t)num_sms() * occupancy((const void *)kernel, 32 * warps) * warps;
         g.upw = g.nunits <= kFewUnits * resident ? 1 : kDefaultUpw;
@@ -810,8 +810,7 @@ void launch3(void (*kernel)(In, Out, LaunchGeom, int, Acc), int warps, int encod
 constexpr int kWarpPerBlockPerSm = 14;
 bool warp_per_block(int encode, int rate, int64_t nunits)
 {
-    return g_upw[encode ? 1 : 0][rate == 16 ? 1 : 0].load(std::memory_order_relaxed) <= 0 &&
-           nunits * 32 <= (int64_t)kWarpPerBlockPerSm * num_sms();
+    return units_per_warp(encode, rate) <= 0 && nunits * 32 <= (int64_t)kWarpPerBlockPerSm * num_sms();
 }
 
 // vec: rows start on 16 bytes wherever a block starts (x0 multiple of 4).
@@ -901,8 +900,7 @@ int launch_decode_payload(float *dst, const LaunchGeom &g, int vec, const AccDec
 
 int units_per_warp(int encode, int rate)
 {
-    const int v = g_upw[encode ? 1 : 0][rate == 16 ? 1 : 0].load(std::memory_order_relaxed);
-    return v > 0 ? v : kDefaultUpw;
+    return g_upw[encode ? 1 : 0][rate == 16 ? 1 : 0].load(std::memory_order_relaxed);
 }
 }  // namespace zfpx
 

@@ -214,8 +214,8 @@ void count_launch();
 void uncount_launches(uint64_t n);   // launches recorded into a graph, not run
 bool valid_codec_rate(int rate);
 int check_launch();   // cudaGetLastError -> ZFPX_OK / ZFPX_ECUDA
-// Work units per warp of the 3-D codec kernels for (direction, rate); 0 = the
-// library's default.  Set through zfpx_set_units_per_warp (the autotuner).
+// Work units per warp of the 3-D codec kernels set for (direction, rate); 0 = the
+// library's choice by the launch's size.  Set through zfpx_set_units_per_warp.
 int units_per_warp(int encode, int rate);
 
 }  // namespace zfpx

@@ -752,11 +752,13 @@ def zfpx_decompress_rfft(plan, rate, recv, re, im, work=None, stream=None):
 
 
 def zfpx_set_units_per_warp(encode, rate, upw):
-    """Launch shape of the 3-D codec kernels: 32-block units per warp (0 = default)."""
+    """Launch shape of the 3-D codec kernels: 32-block units per warp (0 = the
+    library's choice, launch by launch)."""
     _check(lib().zfpx_set_units_per_warp(int(bool(encode)), rate, upw), "zfpx_set_units_per_warp")
 
 
 def zfpx_get_units_per_warp(encode, rate):
+    """What zfpx_set_units_per_warp has set; 0 if that is the library's choice."""
     return int(lib().zfpx_get_units_per_warp(int(bool(encode)), rate))
 
 
