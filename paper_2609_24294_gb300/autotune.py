@@ -4,8 +4,8 @@ The kernels' results never depend on the launch shape; only their speed
 does.  The tuner times a small set of candidate shapes on the real workload
 (CUDA events on the launching stream, after a warm-up, median of a few
 repetitions) and keeps the fastest.  Choices are cached in a JSON file keyed
-by the workload's signature, the GPU name and its SM count, so a workload is
-tuned once per machine type.
+by the workload's signature, the GPU name, its SM count and the sources the
+library was built from, so a workload is tuned once per machine type and kernels.
 
 Candidates:
 * batched ragged kernels: warps per CTA (2, 3, 4 or 8: the per-warp
@@ -16,7 +16,10 @@ Candidates:
   units a warp claims at a time (fewer atomics against a shorter tail);
 * plan codec kernels (3-D blocks): consecutive 32-block units per warp (the
   blocks-per-warp knob; each CTA of the grid codes units-per-warp x warps
-  units, so it also sets the grid size), per direction and rate.
+  units, so it also sets the grid size), per direction and rate; 0 is the
+  library's own choice, launch by launch.  That setting is the process's, so
+  a number takes the place of 0 only where it is faster by more than UPW_MARGIN on
+  the plan at hand: a launch of another size would lose the choice made for it.
 """
 import hashlib
 import json
@@ -25,6 +28,8 @@ import statistics
 
 import torch
 
+from . import build as _build
+
 CACHE = os.environ.get("ZFPX_TUNE_CACHE", os.path.join(os.path.expanduser("~"), ".cache", "zfpx", "tune.json"))
 
 BATCH_CANDIDATES = [(3, 0), (2, 0), (4, 0), (3, 3), (8, 0)]
@@ -32,12 +37,22 @@ LB1_DEFAULT = 16
 LB1_CANDIDATES = (2, 4, 8, 16, 32)
 UPC_DEFAULT = 4
 UPC_CANDIDATES = (1, 2, 4, 8)
-UPW_CANDIDATES = (1, 2, 3, 4, 8)
+UPW_CANDIDATES = (0, 1, 2, 3, 4, 8)
+UPW_MARGIN = 0.02
 
 
 def _device_key():
     p = torch.cuda.get_device_properties(torch.cuda.current_device())
-    return "%s/%d" % (p.name, p.multi_processor_count)
+    return "%s/%d/%s" % (p.name, p.multi_processor_count, _library_key())
+
+
+def _library_key():
+    """The sources the library was built from (their hash, beside the library)."""
+    try:
+        with open(_build.STAMP) as f:
+            return f.read().strip()[:16]
+    except OSError:
+        return "unknown"
 
 
 def _load():
@@ -157,6 +172,8 @@ def tune_codec(plan, rate, src, buf, dst, candidates=None, reps=3, use_cache=Tru
             z.zfpx_set_units_per_warp(d == "encode", rate, u)
             timings[d][str(u)] = time_call(fn, reps=reps)
         best = min(timings[d], key=timings[d].get)
+        if timings[d].get("0", float("inf")) <= (1.0 + UPW_MARGIN) * timings[d][best]:
+            best = "0"
         choice[d] = int(best)
         z.zfpx_set_units_per_warp(d == "encode", rate, choice[d])
     if use_cache:
