@@ -115,7 +115,8 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-CODEC_SOURCES = ("codec.cu", "zfpx_block.cuh", "zfpx_enc3.cuh", "zfpx_internal.h", "zfpx_smem.cuh")
+CODEC_SOURCES = ("codec.cu", "zfpx_block.cuh", "zfpx_enc2.cuh", "zfpx_enc3.cuh", "zfpx_internal.h", "zfpx_smem.cuh",
+                 "zfpx_warp3.cuh")
 
 
 def kernel_source_sha():
