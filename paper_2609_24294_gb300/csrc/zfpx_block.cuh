@@ -830,7 +830,9 @@ ZFPX_HD void xform2_inv(int32_t (&q)[16])
     for (int j = 0; j < 4; j++) lift_inv(q[4 * j], q[4 * j + 1], q[4 * j + 2], q[4 * j + 3]);
 }
 
-// Encodes x[i + 4j] into 16 RATE bits.  The 16 coefficients' bit planes come
+// Encodes x[i + 4j] into 16 RATE bits.  (The plain statement of the stream, as
+// encode_block3, which the CPU tests compile; the kernels' encoder is enc2::encode,
+// which the GPU tests compare with the oracle.)  The 16 coefficients' bit planes come
 // from one 32x32 transpose whose lower 16 rows are zero (the coefficients sit
 // in rows 16..31, so plane k is the high 16 bits of word k and the stages
 // below 16 only touch the upper rows), parked in the lane's plane slots;
@@ -1347,23 +1349,6 @@ ZFPX_HD void decode_blocks1(const uint64_t (&win)[K], const Plane4Dec &tab, floa
             x[b][2] = dequantize_small(q2, e); x[b][3] = dequantize_small(q3, e);
         }
     }
-}
-
-template <int RATE>
-ZFPX_HD uint64_t encode_block1(const float (&x)[4], const Plane4Enc &tab)
-{
-    const float (&xx)[1][4] = reinterpret_cast<const float (&)[1][4]>(x);
-    uint64_t w[1];
-    encode_blocks1<RATE, 1>(xx, tab, w);
-    return w[0];
-}
-
-template <int RATE>
-ZFPX_HD void decode_block1(uint64_t w, float (&x)[4], const Plane4Dec &tab)
-{
-    const uint64_t win[1] = {w};
-    float (&xx)[1][4] = reinterpret_cast<float (&)[1][4]>(x);
-    decode_blocks1<RATE, 1>(win, tab, xx);
 }
 
 }  // namespace blk

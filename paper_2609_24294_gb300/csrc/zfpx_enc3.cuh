@@ -117,8 +117,8 @@ struct PlaneCut {
     }
 };
 
-// One warp's shared memory: tile (kWords<RATE> * 32 words, or more), planes
-// (32 * 32), spos (32 * 32).
+// One warp's shared memory: tile (kWords<RATE> * 32 words, or more) and planes
+// (32 * 32); the CTA's table.
 struct View {
     uint32_t *tile;
     uint64_t *planes;
@@ -133,12 +133,6 @@ struct Shared {
     __device__ __forceinline__ View view(const Expand &tab) { return View{tile, planes, tab.e}; }
 };
 
-__device__ __forceinline__ uint32_t shl(uint32_t a, uint32_t s)
-{
-    uint32_t r;
-    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(s));   // s >= 32 gives 0
-    return r;
-}
 __device__ __forceinline__ uint32_t shr(uint32_t a, uint32_t s)
 {
     uint32_t r;

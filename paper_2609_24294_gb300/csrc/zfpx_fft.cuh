@@ -394,9 +394,12 @@ __device__ __forceinline__ void rfft_row64(const float2 *src, float2 *buf, const
     split_real<STREAM>(buf, tw, H, K, 1.0f / (float)(2 * H), lane, ore, oim);
 }
 
-// rfft_row64 for the first radices it is built for: the 2-3-5 numbers from 4
-// to 20 (lengths 256 to 1280), whose pass 1 fits the registers of pass 2.
-// Fn: a generic call taking an integral constant.
+// The first radices rfft_row64 is built for: the 2-3-5 numbers from 4 to 20.  us
+// for 65536 rows, K = N / 2, the stages above against the two passes: N = 256: 76,
+// 58; 320: 88, 62; 384: 93, 68; 512: 124, 70; 576: 126, 75; 640: 115, 82; 768: 133,
+// 86; 960: 179, 101; 1024: 187, 99; 1152: 214, 119; 1280: 201, 122.  Longer rows take
+// the stages: the passes are neither built nor measured for them.
+// Fn: a macro taking the radix.
 #define ZFPX_FFT_ROW64_RADICES(F) F(4) F(5) F(6) F(8) F(9) F(10) F(12) F(15) F(16) F(18) F(20)
 inline bool row64_radix(int r1)
 {

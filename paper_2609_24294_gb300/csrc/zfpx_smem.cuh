@@ -13,12 +13,7 @@ struct SmemPlanes {
     uint64_t *sm;
     int lane;
     __device__ __forceinline__ void store(int k, uint64_t X) { sm[k * 32 + lane] = X; }
-    __device__ __forceinline__ uint64_t load(int k) const { return sm[k * 32 + lane]; }
     // the low (half 0) or high (half 1) 32 bits of plane k
-    __device__ __forceinline__ void store_half(int k, int half, uint32_t v)
-    {
-        reinterpret_cast<uint32_t *>(sm)[2 * (k * 32 + lane) + half] = v;
-    }
     __device__ __forceinline__ uint32_t load_half(int k, int half) const
     {
         return reinterpret_cast<const uint32_t *>(sm)[2 * (k * 32 + lane) + half];
