@@ -173,11 +173,17 @@ def _check(rc, what):
         raise ZfpxError(rc, what)
 
 
+# not part of PyTorch's documented interface: a build without it gets the Stream object
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
     # the current stream's handle without a Stream object around it: a call on a
     # small field takes 5.4 us of the host, 9.4 with one
     if stream is None:
-        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        if _raw_stream is not None:
+            return ctypes.c_void_p(_raw_stream(torch.cuda.current_device()))
+        stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream)
 
 
