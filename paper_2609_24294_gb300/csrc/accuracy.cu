@@ -23,8 +23,8 @@
 // What bounds it: the codec; the rest moves a slot once out and once in.  With a
 // parse of every slot for L, a zeroed payload filled by atomics, and slots
 // copied out for the decoder, compress, exchange and decompress of a 640 x 320 x
-// 137 field over 4 x 4 ranks at tolerance 1e-3 took 359, 97 and 215 us; now 155,
-// 27 and 146.
+// 137 field over 4 x 4 ranks at tolerance 1e-3 took 351, 93 and 212 us; now 138,
+// 23 and 126.
 #include <algorithm>
 #include <cmath>
 #include <vector>

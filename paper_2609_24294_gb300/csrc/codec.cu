@@ -208,8 +208,8 @@ __device__ __forceinline__ void store_edge(float *p, const int64_t *s, int nx, i
 // Four scalar accesses per row and partial blocks value by value through a local
 // array took 5760 (compress) and 5130 (decompress) warp instructions per 32
 // blocks of a 1000 x 501 x 91 field on 3 x 3 ranks, against 3540 and 4040 for
-// aligned rows: 192 / 174 us at rate 8, now 172 / 131; a 233 x 117 x 137 array of
-// aligned rows, one partial block in 59, went from 26.6 / 26.6 to 22.5 / 20.5 us.
+// aligned rows: 192 / 174 us at rate 8, now 168 / 125; a 233 x 117 x 137 array of
+// aligned rows, one partial block in 59, went from 26.6 / 26.6 to 20.5 / 18.5 us.
 // LEN: the variable-rate modes, which also want every block's bit count (acc).
 template <int RATE, bool VEC, bool LEN>
 __global__ void __launch_bounds__(32 * kEnc3Warps<RATE>, kEnc3MinBlocks)

@@ -958,8 +958,8 @@ ZFPX_HD void transpose16_pairs(uint32_t (&w)[32])
 // 31 bits (n verbatim bits, the group bit, and a value and a group bit for
 // each of the rest but the implied last one), so one 32-bit window holds it.
 // Issue-bound; with 64-bit windows and 32-word transposes decompressing a 1280
-// x 640 x 37 field level by level over 4 x 4 ranks took 182 us at rate 8 and 201
-// at rate 16, now 121 and 133.
+// x 640 x 37 field level by level over 4 x 4 ranks took 172 us at rate 8 and 201
+// at rate 16, now 117 and 132.
 template <int RATE, class Tile, class Planes>
 ZFPX_HD void decode_block2_tile(const Tile &tile, float (&x)[16], Planes &pl)
 {

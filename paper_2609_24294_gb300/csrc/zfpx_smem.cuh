@@ -46,8 +46,8 @@ struct StreamTile {
 // lookups give 16 bits, two more 32 (rarely needed), each byte's ones moved down
 // by the ones before it; the loop over the ones runs as often as the lane with
 // the most of them needs.  Decompressing a 1280 x 640 x 137 field over 8 x 8 ranks:
-// 289 -> 278 us at rate 8, 361 -> 350 at rate 16; 37 levels of 2-D blocks over 4
-// x 4 ranks 129 -> 122 and 139 -> 133 (with all four lookups at once 126 and 139).
+// 289 -> 278 us at rate 8, 361 -> 350 at rate 16; 2-D blocks (decode_block2_tile)
+// 5 % (with all four lookups at once 2 % and none).
 struct __align__(16) DropTable {
     uint32_t w[64];
 };
