@@ -284,6 +284,13 @@ __device__ __forceinline__ bool role_wait(uint32_t mbar, uint32_t parity, volati
     return false;
 }
 
+// How often stage s of `stages` has been used once `n` slices have gone through
+// them in turn: its barrier's last phase is the one before that.
+__host__ __device__ constexpr int stage_uses(int n, int s, int stages) { return (n - s + stages - 1) / stages; }
+static_assert(stage_uses(0, 0, 4) == 0 && stage_uses(0, 3, 4) == 0 && stage_uses(1, 0, 4) == 1 && stage_uses(1, 1, 4) == 0 &&
+              stage_uses(4, 3, 4) == 1 && stage_uses(5, 0, 4) == 2 && stage_uses(5, 1, 4) == 1 && stage_uses(7, 2, 2 + 1) == 2,
+              "uses of a stage");
+
 // 32 columns of this warp's 32 tensor-memory lanes
 __device__ __forceinline__ void tmem_store32(uint32_t addr, const uint32_t (&v)[32])
 {
@@ -309,6 +316,7 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
     __shared__ __align__(8) uint64_t full_bar[kMaxStages], lo_bar[kMaxStages], mma_bar[kMaxStages], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_base;
     __shared__ int fail;
+    __shared__ int issued[2];                            // slices loaded, slices whose MMAs were committed
     volatile int *vfail = &fail;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -371,6 +379,7 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                     tma_load_2d(smem_u32(b_raw(s)), &tmap_b, k * kBK, brow, fb);
                 }
             }
+            issued[0] = i;
         }
     } else if (warp == 1) {
         // ---- MMAs
@@ -415,6 +424,7 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                                      :: "r"(smem_u32(&acc_full[acc])) : "memory");
                 }
             }
+            issued[1] = i;
         }
     } else if (warp >= 4 && warp <= 7) {
         // ---- table slices to tensor memory: a thread per row, its 32 values and
@@ -505,10 +515,12 @@ legendre_mma_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
     __syncthreads();
     if (*vfail && tid == 0) {
         atomicExch(status, 1);
-        // let copies and MMAs still in flight land before the CTA leaves
+        // let copies and MMAs still in flight land before the CTA leaves: the last
+        // phase that each stage's barriers have been given
         for (int s = 0; s < stages; s++) {
-            mbar_wait(smem_u32(&full_bar[s]), 0u);
-            mbar_wait(smem_u32(&mma_bar[s]), 0u);
+            const int loads = stage_uses(issued[0], s, stages), mmas = stage_uses(issued[1], s, stages);
+            if (loads) mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(loads - 1) & 1u);
+            if (mmas) mbar_wait(smem_u32(&mma_bar[s]), (uint32_t)(mmas - 1) & 1u);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
