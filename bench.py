@@ -137,7 +137,7 @@ def recorded_pipes(kernel_key, sha):
             if m and m.group(1) == kernel_key and m.group(5) == sha:
                 return {"unit": "alu pipe (integer)", "alu_pct_of_peak": float(m.group(2)),
                         "issue_slots_pct": float(m.group(3)), "dram_pct_of_peak": float(m.group(4)),
-                        "source": "ncu --set full, profiles/" + os.path.basename(f)}
+                        "source": "ncu, profiles/" + os.path.basename(f)}
     return None
 
 
